@@ -309,95 +309,109 @@ __global__ void k_coarsen_faces(const double *__restrict__ fx, const double *__r
 
 // ---------------------------------------------- A9: coarsest direct solve
 // Dense M = -At + 11^T/n (symmetric positive definite; the 11^T/n term only
-// for a singular operator) as the left half of [M | I] (row-major, n x 2n);
-// one thread per row, each row written once.
+// for a singular operator), row-major n x n, one thread per entry.  Neighbours
+// that coincide (an axis of two cells) add up in a fixed order.
 __global__ void k_dense_build(const double *__restrict__ bx, const double *__restrict__ by,
                               const double *__restrict__ bz, const double *__restrict__ diag,
                               double *__restrict__ M, Dims d, int singular) {
-  int n = d.nx * d.ny * d.nz;
-  int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= n) return;
-  int i = r % d.nx, j = (r / d.nx) % d.ny, k = r / (d.nx * d.ny);
-  double *row = M + (size_t)r * 2 * n;
-  double inv_n = singular ? 1.0 / n : 0.0;
-  for (int c = 0; c < n; ++c) row[c] = inv_n;
-  for (int c = 0; c < n; ++c) row[n + c] = (c == r) ? 1.0 : 0.0;
-  row[r] += diag[r];
-  row[at(d, wlo(i, d.nx), j, k)] -= bx[r];
-  row[at(d, whi(i, d.nx), j, k)] -= bx[at(d, whi(i, d.nx), j, k)];
-  row[at(d, i, wlo(j, d.ny), k)] -= by[r];
-  row[at(d, i, whi(j, d.ny), k)] -= by[at(d, i, whi(j, d.ny), k)];
-  row[at(d, i, j, wlo(k, d.nz))] -= bz[r];
-  row[at(d, i, j, whi(k, d.nz))] -= bz[at(d, i, j, whi(k, d.nz))];
+  const int n = d.nx * d.ny * d.nz;
+  const int c = blockIdx.x * blockDim.x + threadIdx.x, r = blockIdx.y;
+  if (c >= n) return;
+  const int i = r % d.nx, j = (r / d.nx) % d.ny, k = r / (d.nx * d.ny);
+  double v = singular ? 1.0 / n : 0.0;
+  if (c == r) v += diag[r];
+  const int xl = (int)at(d, wlo(i, d.nx), j, k), xh = (int)at(d, whi(i, d.nx), j, k);
+  const int yl = (int)at(d, i, wlo(j, d.ny), k), yh = (int)at(d, i, whi(j, d.ny), k);
+  const int zl = (int)at(d, i, j, wlo(k, d.nz)), zh = (int)at(d, i, j, whi(k, d.nz));
+  if (c == xl) v -= bx[r];
+  if (c == xh) v -= bx[xh];
+  if (c == yl) v -= by[r];
+  if (c == yh) v -= by[yh];
+  if (c == zl) v -= bz[r];
+  if (c == zh) v -= bz[zh];
+  M[(size_t)r * n + c] = v;
 }
 
-// Gauss-Jordan elimination of [M | I] -> [I | M^-1] by one block (M is SPD,
-// so no pivoting).  n <= 512.  The inverse (symmetric) is copied to Minv.
-__global__ void k_gauss_jordan(double *__restrict__ M, double *__restrict__ Minv, int n) {
-  __shared__ double col[512];
-  const int w = 2 * n;
-  for (int p = 0; p < n; ++p) {
-    for (int r = threadIdx.x; r < n; r += blockDim.x) col[r] = M[(size_t)r * w + p];
-    __syncthreads();
-    double inv = 1.0 / col[p];
-    for (int c = threadIdx.x; c < w; c += blockDim.x) M[(size_t)p * w + c] *= inv;
-    __syncthreads();
-    for (int e = threadIdx.x; e < n * w; e += blockDim.x) {
-      int r = e / w, c = e - r * w;
-      if (r != p) M[(size_t)r * w + c] -= col[r] * M[(size_t)p * w + c];
-    }
-    __syncthreads();
+// One step of the blocked in-place Gauss-Jordan inversion of the SPD coarsest
+// matrix (no pivoting): with the pivot block A_pp of GJ_B rows and columns and
+// P = A_pp^-1,
+//   A_pp <- P,  A_pj <- P A_pj,  A_ip <- -A_ip P,  A_ij <- A_ij - A_ip P A_pj,
+// from src into dst; after ceil(n / GJ_B) steps dst is the inverse.  A block owns
+// one T x T tile and forms P (in one warp's registers) and its part of P A_pj
+// itself, so a step needs nothing but the previous step's matrix.
+// What bounds it: the chain of a step (load, 16 dependent pivots, two products:
+// ~14 us) up to ~200 unknowns, this part's FP64 rate (2 multiply-adds per cycle
+// and SM) above.  Measured, whole inversion, against one Cholesky per column
+// (n <= 112) and one block eliminating column by column (above), which held
+// the n^3 on one SM: 64 unknowns 60 us (133), 105: 102 us (309), 300: 350 us
+// (16.2 ms).  T = 16 puts more SMs on a small matrix, T = 32 repeats the pivot
+// inverse less: 16 / 32 take 60 / 81 us at 64 unknowns, 350 / 377 at 300,
+// 590 / 622 at 392, 1226 / 816 at 512 (GJ_SMALL).
+constexpr int GJ_B = 16, GJ_THREADS = 256;
+constexpr int GJ_SMALL = 400;  // unknowns up to which the inversion takes 16 x 16 tiles
+template <int T>
+__global__ void __launch_bounds__(GJ_THREADS)
+k_gj_step(const double *__restrict__ src, double *__restrict__ dst, int n, int q0) {
+  griddep_wait();
+  __shared__ double P[GJ_B][GJ_B + 1], B[GJ_B][T + 1], A[T][GJ_B + 1], W[GJ_B][T + 1];
+  const int tid = threadIdx.x, i0 = blockIdx.y * T, j0 = blockIdx.x * T;
+  const int bs = min(GJ_B, n - q0);
+  {
+    const int r = tid / GJ_B, c = tid % GJ_B;  // GJ_THREADS = GJ_B^2: one entry each
+    P[r][c] = r < bs && c < bs ? src[(size_t)(q0 + r) * n + q0 + c] : (r == c ? 1.0 : 0.0);
   }
-  for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
-    int r = e / n, c = e - r * n;
-    Minv[e] = M[(size_t)r * w + n + c];
+  for (int e = tid; e < GJ_B * T; e += GJ_THREADS) {
+    const int r = e / T, c = e % T;
+    B[r][c] = r < bs && j0 + c < n ? src[(size_t)(q0 + r) * n + j0 + c] : 0.0;
   }
-}
-
-// Inverse of the SPD coarsest matrix M (left half of [M | I]) by columns, for
-// n <= GJ_SMEM_MAX: block j factors M = L L^T in shared memory (every block the
-// same factor) and solves L L^T x = e_j into column j.  The n blocks run on n
-// SMs at once; one block's Gauss-Jordan elimination is bound by a single SM's
-// FP64 rate, which is low on this part.
-constexpr int GJ_SMEM_MAX = 112;
-__global__ void k_inverse_cols(const double *__restrict__ Maug, double *__restrict__ Minv, int n) {
-  extern __shared__ double L[];  // n x n, then the right-hand side / solution (n)
-  __shared__ double inv_d[GJ_SMEM_MAX];
-  double *y = L + n * n;
-  const int w = 2 * n, j = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
-  for (int e = tid; e < n * n; e += nt) L[e] = Maug[(size_t)(e / n) * w + (e % n)];
-  for (int e = tid; e < n; e += nt) y[e] = e == j ? 1.0 : 0.0;
+  for (int e = tid; e < GJ_B * T; e += GJ_THREADS) {
+    const int r = e / GJ_B, c = e % GJ_B;
+    A[r][c] = i0 + r < n && c < bs ? src[(size_t)(i0 + r) * n + q0 + c] : 0.0;
+  }
   __syncthreads();
-  for (int k = 0; k < n; ++k) {  // right-looking Cholesky, lower triangle
-    if (tid == 0) {
-      const double dkk = sqrt(L[k * n + k]);
-      L[k * n + k] = dkk;
-      inv_d[k] = 1.0 / dkk;
+  if (tid < 32) {  // lane: row r, columns 8h .. 8h + 7; a row is scaled by its pivot at the end
+    const int r = tid & 15, h = tid >> 4;
+    double a[8], own = 1.0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) a[q] = P[r][8 * h + q];
+#pragma unroll
+    for (int k = 0; k < GJ_B; ++k) {
+      const int hk = k >> 3, kk = k & 7;
+      const double inv = __drcp_rn(__shfl_sync(0xffffffffu, a[kk], k + 16 * hk));
+      const double f = __shfl_sync(0xffffffffu, a[kk], r + 16 * hk) * inv;
+      const double s = r == k ? 0.0 : f;
+#pragma unroll
+      for (int q = 0; q < 8; ++q)
+        a[q] = fma(-s, __shfl_sync(0xffffffffu, a[q], k + 16 * h), a[q]);
+      if (h == hk) a[kk] = r == k ? 1.0 : -s;
+      if (r == k) own = inv;
     }
-    __syncthreads();
-    const double id = inv_d[k];
-    for (int r = k + 1 + tid; r < n; r += nt) L[r * n + k] *= id;
-    __syncthreads();
-    const int m = n - k - 1;
-    for (int e = tid; e < m * m; e += nt) {
-      const int r = k + 1 + e / m, c = k + 1 + e % m;
-      if (c <= r) L[r * n + c] -= L[r * n + k] * L[c * n + k];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) P[r][8 * h + q] = a[q] * own;
+  }
+  __syncthreads();
+  for (int e = tid; e < GJ_B * T; e += GJ_THREADS) {
+    const int r = e / T, c = e % T;
+    double s = 0.0;
+#pragma unroll
+    for (int k = 0; k < GJ_B; ++k) s = fma(P[r][k], B[k][c], s);
+    W[r][c] = s;
+  }
+  __syncthreads();
+  for (int e = tid; e < T * T; e += GJ_THREADS) {
+    const int r = e / T, c = e % T, gi = i0 + r, gj = j0 + c;
+    if (gi >= n || gj >= n) continue;
+    const bool pr = gi >= q0 && gi < q0 + bs, pc = gj >= q0 && gj < q0 + bs;
+    double v;
+    if (pr) {
+      v = pc ? P[gi - q0][gj - q0] : W[gi - q0][c];
+    } else {
+      v = pc ? 0.0 : src[(size_t)gi * n + gj];
+#pragma unroll
+      for (int k = 0; k < GJ_B; ++k) v = fma(-A[r][k], pc ? P[k][gj - q0] : W[k][c], v);
     }
-    __syncthreads();
+    dst[(size_t)gi * n + gj] = v;
   }
-  for (int c = 0; c < n; ++c) {  // L y = e_j (column-oriented)
-    if (tid == 0) y[c] *= inv_d[c];
-    __syncthreads();
-    for (int r = c + 1 + tid; r < n; r += nt) y[r] -= L[r * n + c] * y[c];
-    __syncthreads();
-  }
-  for (int c = n - 1; c >= 0; --c) {  // L^T x = y
-    if (tid == 0) y[c] *= inv_d[c];
-    __syncthreads();
-    for (int r = tid; r < c; r += nt) y[r] -= L[c * n + r] * y[c];
-    __syncthreads();
-  }
-  for (int r = tid; r < n; r += nt) Minv[(size_t)r * n + j] = y[r];
 }
 
 // e = M^-1 (-(b - mean b)), FP64 internally for any storage type T (the

@@ -1302,14 +1302,20 @@ mp_status geometry(mp_poisson *hd, const double *phi, double rho_l, double rho_g
   Level &lc = hd->L.back();
   const int lcl = (int)hd->L.size() - 1;
   const double nc = (double)hd->nc;
-  LAUNCH(hd, K_DENSE, lcl, nc * 2.0 * nc * 8.0, k_dense_build, (hd->nc + 127) / 128, 128, lc.bx,
-         lc.by, lc.bz, lc.diag, hd->Maug, lc.d, hd->outflow == 0 ? 1 : 0);
-  if (hd->nc <= GJ_SMEM_MAX)
-    LAUNCH_SMEM(hd, K_GJ, lcl, nc * 3.0 * nc * 8.0, k_inverse_cols, hd->nc, 256,
-                (size_t)(hd->nc + 1) * hd->nc * sizeof(double), hd->Maug, hd->Minv, hd->nc);
-  else
-    LAUNCH(hd, K_GJ, lcl, nc * 3.0 * nc * 8.0, k_gauss_jordan, 1, 1024, hd->Maug, hd->Minv,
-           hd->nc);
+  LAUNCH(hd, K_DENSE, lcl, nc * nc * 8.0, k_dense_build, dim3((hd->nc + 127) / 128, hd->nc), 128,
+         lc.bx, lc.by, lc.bz, lc.diag, hd->Maug, lc.d, hd->outflow == 0 ? 1 : 0);
+  // the inverse, GJ_B columns per launch, between the two halves of Maug and
+  // into Minv at the last step
+  const int tile = hd->nc <= GJ_SMALL ? 16 : 32;
+  const dim3 gt((hd->nc + tile - 1) / tile, (hd->nc + tile - 1) / tile);
+  auto kgj = tile == 16 ? k_gj_step<16> : k_gj_step<32>;
+  const double *src = hd->Maug;
+  for (int q0 = 0, s = 0; q0 < hd->nc; q0 += GJ_B, ++s) {
+    double *dst = q0 + GJ_B >= hd->nc ? hd->Minv
+                                      : hd->Maug + (s % 2 == 0 ? (size_t)hd->nc * hd->nc : 0);
+    LAUNCH_PDL(hd, K_GJ, lcl, nc * 2.0 * nc * 8.0, kgj, gt, GJ_THREADS, 0, src, dst, hd->nc, q0);
+    src = dst;
+  }
   CKS(launch_ok());
   CKS(deflation_setup(hd));
   CK(cudaStreamSynchronize(hd->st));
@@ -1544,8 +1550,6 @@ mp_status create(mp_poisson *hd, mp_grid g, double h, const mp_bc bc[3]) {
   // fused FP32 sweep: levels above the one-CTA tail with nx a multiple of 8
   CKS(fused_setup(hd));
   CKS(ctail_setup(hd));
-  CK(cudaFuncSetAttribute(k_inverse_cols, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                          (int)((GJ_SMEM_MAX + 1) * GJ_SMEM_MAX * sizeof(double))));
   CK(cudaFuncSetAttribute(k_tail<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                           (int)std::max<size_t>(hd->tail64_bytes, 1)));
   CK(cudaFuncSetAttribute(k_tail<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,

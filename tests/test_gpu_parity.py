@@ -843,3 +843,26 @@ def test_cluster_tail_on_anisotropic_grids(shape):
     assert rel_l2(host(p), ref["p"]) < PARITY
     print(shape, [(e["name"], e["level"]) for e in s.profile() if e["name"] == "coarse_cluster_f32"])
     s.close()
+
+
+@pytest.mark.parametrize("shape", [(2, 3, 2), (3, 5, 3), (3, 3, 5), (7, 4, 4), (9, 5, 7), (7, 7, 8),
+                                   (9, 7, 7), (9, 7, 8)])
+@pytest.mark.parametrize("outflow", [False, True])
+def test_coarsest_inverse_solves_a_single_level_directly(shape, outflow):
+    """A grid that does not coarsen is one dense level: a stationary step is a
+    multiplication by its inverse, so two steps (the second a refinement) reach
+    the target whatever the size (12 to 504 unknowns: below one pivot block,
+    ragged last blocks, both tile sizes), singular or not."""
+    nz, ny, nx = shape
+    bc = (N, N, oracle.NEUMANN_DIRICHLET if outflow else N)
+    g = np.random.Generator(np.random.PCG64(nx * ny * nz))
+    phi = g.random(shape) - 0.5
+    rhs = g.standard_normal(shape)
+    ref = oracle.solve(phi, rhs, 1.0, 1.0, 1e-3, 0.05, bc, tol=REF_TOL)
+    for precision in (0, 1):
+        s = make(phi, dict(h=1.0, bc=bc, rho_l=1.0, rho_g=1e-3, sigma=0.05), method=1,
+                 max_iters=2 if precision == 0 else 4, precision=precision)
+        p, it, _ = s.solve(dev(rhs), tol=TOL)
+        assert s.stats()["relres"] <= TOL and s.stats()["levels"] == 1
+        assert rel_l2(host(p), ref["p"]) < PARITY
+        s.close()
