@@ -47,6 +47,9 @@ typedef struct mp_net *mp_net_handle;
  * w: [cout][27][ca+cb] BF16; bias: cout FP32 or NULL.  Output y (BF16)
  * or, when y32 is not NULL, FP32 into y32 instead.  All device pointers,
  * 16-byte aligned.  Grid dims multiples of 8 (x) and 4 (y, z).
+ * Scratch (here and in mp_conv3d_wgrad) comes from a stream-ordered pool per
+ * device that keeps up to 64 MB between calls, returned when a network is
+ * destroyed.
  */
 mp_status mp_conv3d_fwd(int nx, int ny, int nz, const void *xa, int ca, int up_a, const void *xb,
                         int cb, const void *w, const float *bias, int cout, int relu, void *y,

@@ -1062,6 +1062,7 @@ __global__ void k_to_pressure(const float *__restrict__ q, size_t n, const doubl
 #include <atomic>
 #include <cmath>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <vector>
 
@@ -1135,6 +1136,49 @@ mp_status nalloc(mp_net *net, T **p, size_t count) {
   net->allocs.push_back(v);
   *p = (T *)v;
   return MP_OK;
+}
+
+// Workspace of the single-layer calls (weight image, split-K partials, status
+// word): a private stream-ordered pool per device, so calls on any thread and
+// stream draw from it safely.  The default pool returns its memory to the
+// driver at every synchronisation, and these calls end in one; mapping it again
+// took most of a call (a 16-16 layer at 128^3, whose kernel takes 65 us: 287 us
+// a call, 102 with this pool).  It keeps up to WS_KEEP bytes (more is returned
+// at the next synchronisation) until a network is destroyed.
+constexpr uint64_t WS_KEEP = 64ull << 20;
+constexpr int WS_DEVICES = 64;
+std::mutex ws_mutex;
+cudaMemPool_t ws_pools[WS_DEVICES] = {};
+
+mp_status ws_pool(cudaMemPool_t *out) {
+  int dev = 0;
+  NCK(cudaGetDevice(&dev));
+  if (dev < 0 || dev >= WS_DEVICES) return MP_ERR_CUDA;
+  std::lock_guard<std::mutex> lock(ws_mutex);
+  if (!ws_pools[dev]) {
+    cudaMemPoolProps p = {};
+    p.allocType = cudaMemAllocationTypePinned;
+    p.location.type = cudaMemLocationTypeDevice;
+    p.location.id = dev;
+    cudaMemPool_t pool = nullptr;
+    NCK(cudaMemPoolCreate(&pool, &p));
+    uint64_t keep = WS_KEEP;
+    if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+      cudaGetLastError();
+      cudaMemPoolDestroy(pool);
+      return MP_ERR_CUDA;
+    }
+    ws_pools[dev] = pool;
+  }
+  *out = ws_pools[dev];
+  return MP_OK;
+}
+// return what the current device's pool keeps and no call uses
+void ws_trim() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= WS_DEVICES) return;
+  std::lock_guard<std::mutex> lock(ws_mutex);
+  if (ws_pools[dev]) cudaMemPoolTrimTo(ws_pools[dev], 0);
 }
 
 bool cout_ok(int c) { return c == 16 || c == 32 || c == 48 || c == 64 || c == 96 || c == 128; }
@@ -1486,10 +1530,12 @@ mp_status mp_conv3d_fwd(int nx, int ny, int nz, const void *xa, int ca, int up_a
   CUtensorMap ma, mb;
   NCKS(make_maps(g, (const bf16 *)xa, (const bf16 *)xb, &ma, &mb));
   const size_t nw = (size_t)cout * 27 * g.cin;
-  int *err = nullptr;
+  // one block: the packed weights (a multiple of 16 bytes), then the status word
+  cudaMemPool_t pool;
+  NCKS(ws_pool(&pool));
   bf16 *img = nullptr;
-  NCK(cudaMallocAsync((void **)&err, sizeof(int), st));
-  NCK(cudaMallocAsync((void **)&img, nw * sizeof(bf16), st));
+  NCK(cudaMallocFromPoolAsync((void **)&img, nw * sizeof(bf16) + sizeof(int), pool, st));
+  int *err = reinterpret_cast<int *>(img + nw);
   NCK(cudaMemsetAsync(err, 0, sizeof(int), st));
   k_pack_img<bf16><<<grid_for(nw), 256, 0, st>>>((const bf16 *)w, cout, g.cin, 0, nc_of(cout), img);
   mp_status s = conv_fwd(g, ma, mb, (const bf16 *)xa, img, bias, cout, (bf16 *)y, y32, relu, err,
@@ -1497,7 +1543,6 @@ mp_status mp_conv3d_fwd(int nx, int ny, int nz, const void *xa, int ca, int up_a
   int h = 0;
   if (s == MP_OK) NCK(cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, st));
   NCK(cudaFreeAsync(img, st));
-  NCK(cudaFreeAsync(err, st));
   NCK(cudaStreamSynchronize(st));
   if (s != MP_OK) return s;
   return h ? MP_ERR_TIMEOUT : MP_OK;
@@ -1512,17 +1557,18 @@ mp_status mp_conv3d_wgrad(int nx, int ny, int nz, const void *xa, int ca, int up
     return MP_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)stream;
   ConvGeom geo{nx, ny, nz, ca, cb, up_a ? 1 : 0, ca + cb};
-  int *err = nullptr;
+  cudaMemPool_t pool;
+  NCKS(ws_pool(&pool));
+  const size_t np = wgrad_partial_floats(geo, cout);
   float *part = nullptr;
-  NCK(cudaMallocAsync((void **)&err, sizeof(int), st));
-  NCK(cudaMallocAsync((void **)&part, wgrad_partial_floats(geo, cout) * sizeof(float), st));
+  NCK(cudaMallocFromPoolAsync((void **)&part, np * sizeof(float) + sizeof(int), pool, st));
+  int *err = reinterpret_cast<int *>(part + np);
   NCK(cudaMemsetAsync(err, 0, sizeof(int), st));
   mp_status s = conv_wgrad(geo, (const bf16 *)xa, (const bf16 *)xb, (const bf16 *)g, cout, part,
                            dw, err, st);
   int h = 0;
   if (s == MP_OK) NCK(cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, st));
   NCK(cudaFreeAsync(part, st));
-  NCK(cudaFreeAsync(err, st));
   NCK(cudaStreamSynchronize(st));
   if (s != MP_OK) return s;
   return h ? MP_ERR_TIMEOUT : MP_OK;
@@ -1885,6 +1931,7 @@ void mp_net_destroy(mp_net_handle net) {
   cudaStreamSynchronize(net->st);
   for (void *p : net->allocs) cudaFree(p);
   if (net->hscal) cudaFreeHost(net->hscal);
+  ws_trim();
   delete net;
 }
 

@@ -702,3 +702,35 @@ def test_train_step_from_an_external_gradient_equals_the_fused_step():
         assert torch.equal(a.get_params(), b.get_params()), step
     a.close()
     b.close()
+
+
+def test_layer_calls_from_several_threads_share_the_workspace_pool():
+    """Single-layer calls take their workspace from one pool per device: calls
+    of different sizes running at once on several host threads give the bits of
+    the same calls run one after the other."""
+    import threading
+    g = torch.Generator(device="cuda").manual_seed(3)
+    jobs = []
+    for n, ca, cout in ((16, 16, 16), (24, 32, 32), (32, 16, 64), (32, 64, 32)):
+        x = torch.randn(n, n, n, ca, generator=g, device="cuda").bfloat16()
+        w = (0.05 * torch.randn(cout, 27, ca, generator=g, device="cuda")).bfloat16()
+        gy = torch.randn(n, n, n, cout, generator=g, device="cuda").bfloat16()
+        jobs.append((x, w, gy, cout))
+    run = lambda j: (mp_conv3d_fwd(j[0], j[1], j[3]), mp_conv3d_wgrad(j[0], j[2]))  # noqa: E731
+    ref = [run(j) for j in jobs]
+    torch.cuda.synchronize()
+    out = [[] for _ in jobs]
+
+    def work(k):
+        for _ in range(5):
+            out[k].append(run(jobs[k]))
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(len(jobs))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    for k, runs in enumerate(out):
+        assert len(runs) == 5
+        for y, dw in runs:
+            assert torch.equal(y, ref[k][0]) and torch.equal(dw, ref[k][1])
