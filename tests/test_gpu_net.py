@@ -722,6 +722,7 @@ def test_layer_calls_from_several_threads_share_the_workspace_pool():
     out = [[] for _ in jobs]
 
     def work(k):
+        torch.cuda.set_device(0)  # the thread's current context
         for _ in range(5):
             out[k].append(run(jobs[k]))
     threads = [threading.Thread(target=work, args=(k,)) for k in range(len(jobs))]
