@@ -47,7 +47,7 @@ typedef enum {
   MP_ERR_DIVERGED = 3,      /* NaN/Inf residual; p is unspecified */
   MP_ERR_CUDA = 4,          /* a CUDA runtime call failed */
   MP_ERR_OOM = 5,           /* device or pinned allocation failed */
-  MP_ERR_TIMEOUT = 6,       /* reserved: a bounded device wait gave up */
+  MP_ERR_TIMEOUT = 6,       /* a bounded device wait gave up */
   MP_ERR_NO_NET = 7         /* learned initial guess requested without weights */
 } mp_status;
 
@@ -104,20 +104,20 @@ typedef struct {
                         levels, which the V-cycle resolves poorly at density ratio 1000;
                         0 = plain MG-preconditioned CG.  Same converged answer.  Applies to
                         periodic and wall boundaries (off with an outflow side). */
-  int smoother;      /* FP32 V-cycle levels (mixed precision) with nx a multiple of 8 and
-                        no outflow side:
-                        1 (default) = one fused pass per red-black sweep (both colours,
-                        shared-memory halo staging, second iterate buffer); 0 = one
+  int smoother;      /* 1 (default): FP32 V-cycle levels (mixed precision) of at least 4e6 cells
+                        with nx a multiple of 8 and no outflow side run one fused pass per
+                        red-black sweep (both colours, shared-memory halo staging, second
+                        iterate buffer), and FP32 levels of at most 6e5 cells and FP64 levels
+                        that fit the chip's shared memory one launch per visit; 0 = one
                         in-place launch per colour.  Bitwise the same result. */
   int label_limit;   /* bound on every find walk and union retry of the gas-component
                         labelling (default 8192; walks are a few steps long in practice).
                         A geometry whose labelling reaches it is solved without deflation
                         (mp_stats.components = 0). */
-  int coarse_cluster; /* FP32 V-cycle: 1 (default) runs the level above the one-CTA tail and
-                        every coarser level as one launch of an 8-CTA thread-block cluster
-                        (distributed shared memory, cluster barriers between steps) where
-                        the levels' z-planes split evenly; 0 = per-level launches down to
-                        the one-CTA tail.  Same method, slightly different rounding. */
+  int coarse_cluster; /* 1 (default): the V-cycle's levels of at most 65536 (FP32) or 16384
+                        (FP64) cells run as one launch of a thread-block cluster (distributed
+                        shared memory); 0 = per-level launches down to the one-CTA tail.  Same
+                        method, slightly different rounding. */
   void *stream;      /* cudaStream_t; NULL = legacy default stream. */
 } mp_opts;
 

@@ -985,7 +985,9 @@ __global__ void k_prolong_vec(T *__restrict__ x, const T *__restrict__ ec, Dims 
 
 // --------------------------------------------------------- Krylov kernels
 // Scalars kept on the device between kernels (no host round trip).
-enum { S_RZ = 0, S_RZOLD, S_DQ, S_ALPHA, S_BETA, S_RR, S_BB, S_MEAN, S_TMP, S_COUNT };
+enum { S_RZ = 0, S_RZOLD, S_DQ, S_ALPHA, S_BETA, S_RR, S_BB, S_MEAN, S_TMP,
+       S_ERR,  // set by a kernel whose bounded wait gave up
+       S_COUNT };
 enum { OP_STORE = 0, OP_ALPHA, OP_BETA, OP_MEAN };
 
 // Stencil kernels with a reduction walk a column of `zper` planes per

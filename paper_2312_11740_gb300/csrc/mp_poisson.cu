@@ -20,6 +20,7 @@
 #include "../../include/mp_poisson.h"
 #include "mp_kernels.cuh"
 #include "mp_sweep.cuh"
+#include "mp_visit.cuh"
 #include "mp_ctail.cuh"
 #include "mp_deflate.cuh"
 
@@ -29,6 +30,20 @@ namespace {
 
 constexpr int MAX_COARSE = 512;
 constexpr int VEC_BLOCKS = 152 * 4;  // fixed grid for vector kernels: 4 resident per SM (152 SMs)
+
+// blocks of a level visit (mp_visit.cuh); py = 0: the level is not visited in one launch
+struct VisitPlan {
+  int py = 0, pz = 0, bym = 0, bzm = 0;
+  size_t smem = 0;
+};
+
+// cluster tail (mp_ctail.cuh): its top level (-1: not used), CTAs, shared memory
+// per CTA, the exchange slots in it and every level's blocks
+struct CtPlan {
+  int top = -1, ctas = 0, mail = 0, mail_words = 0;
+  size_t bytes = 0;
+  struct Cut { int py, pz, bym, bzm, off; } cut[CT_MAX_LEVELS] = {};
+};
 
 struct Level {
   Dims d;
@@ -41,6 +56,7 @@ struct Level {
   float *b32 = nullptr, *e32 = nullptr;
   float *t32 = nullptr;  // second FP32 iterate of the fused sweep (levels it runs on)
   int ftx = 0, fty = 0, fchunk = 0;  // fused sweep grid: tiles in x, y; z-chunks
+  VisitPlan vis64, vis32;
   // outflow sides: the boundary-face coefficients per side (planes, null for
   // other sides) and the per-cell outflow diagonal (null without outflow)
   double *bnd[6] = {};
@@ -51,15 +67,15 @@ struct Level {
 
 enum KernelId {
   K_CURV, K_FACES, K_JUMP, K_DIAG, K_COARSEN, K_DENSE, K_GJ,
-  K_RBGS64, K_RBGS32, K_RBGS32F, K_TAIL64, K_TAIL32, K_CTAIL32, K_RESTR64, K_RESTR32, K_PROL64, K_PROL32, K_COARSE64, K_COARSE32,
+  K_RBGS64, K_RBGS32, K_RBGS32F, K_VISIT64, K_TAIL64, K_TAIL32, K_CTAIL64, K_CTAIL32, K_RESTR64, K_RESTR32, K_PROL64, K_PROL32, K_COARSE64, K_COARSE32,
   K_APPLY64, K_APPLY32, K_RESID64, K_RESID32, K_RESIDMIX, K_DOT64, K_DOT32, K_AXPY64, K_AXPY32,
   K_XPBY64, K_XPBY32, K_ADD64, K_ADD32, K_ADDF32, K_SUM, K_SUBMEAN, K_REDUCE, K_ASSEMBLE,
   K_ASSEMBLE_U, K_PROJECT, K_DIV, K_SCALE, K_DEFL, K_DEFL_LABEL, K_DEFL_DOT, K_COUNT
 };
 const char *const kKernelNames[K_COUNT] = {
   "curvature", "gfm_faces", "jump", "diag", "coarsen_faces", "dense_build", "gauss_jordan",
-  "rbgs_f64", "rbgs_f32", "rbgs_f32_fused", "coarse_tail_f64", "coarse_tail_f32",
-  "coarse_cluster_f32",
+  "rbgs_f64", "rbgs_f32", "rbgs_f32_fused", "level_visit_f64", "coarse_tail_f64", "coarse_tail_f32",
+  "coarse_cluster_f64", "coarse_cluster_f32",
   "resid_restrict_f64", "resid_restrict_f32", "prolong_f64",
   "prolong_f32", "coarse_solve_f64", "coarse_solve_f32io", "apply_dot_f64", "apply_dot_f32",
   "residual_f64", "residual_f32", "residual_mixed", "dot_f64", "dot_f32", "axpy2_f64",
@@ -68,7 +84,18 @@ const char *const kKernelNames[K_COUNT] = {
   "deflation_band", "deflation_label", "deflation_dot"};
 constexpr int MAX_LEVELS = 16;
 constexpr int TAIL32_NU_MAX = 4;  // sweeps per level in the one-CTA FP32 tail
-constexpr size_t CT_SMEM_MAX = 200 * 1024;  // shared memory per CTA of the cluster tail
+// largest level of the cluster tail: above it a half-sweep takes longer on the
+// cluster's SMs than a launch or a level visit spread over all of them (FP64: the
+// pipe's rate)
+constexpr size_t CT_TOP32 = 65536, CT_TOP64 = 16384;
+// Smallest level of the fused sweep and largest of an FP32 visit.  A level that
+// stays in L2 streams its faces for every colour from there: measured per CG
+// iteration, fused sweep / one launch per colour on the finest level: 128^3
+// 248 / 236 us, 128 x 128 x 160 282 / 263, 160^3 406 / 406, 192 x 192 x 160
+// 437 / 448, 256^3 904 / 956.  Visit / launches: 64 x 64 x 80 second level 263 /
+// 273, 96^3 finest 185 / 181; FP64 96 x 64 x 48 249 / 258, 112 x 80 x 96 350 / 356
+// (every level that fits).
+constexpr size_t FUSED_MIN = 4000000, VISIT_TOP32 = 600000;
 constexpr int EVENT_POOL = 4096;
 constexpr int MAX_SLABS = 8;  // z-slabs of the host-buffer step's copy pipeline
 
@@ -149,11 +176,14 @@ struct mp_poisson {
   cudaEvent_t xev[2 * MAX_SLABS + 2] = {};
   // first level of the one-CTA coarse tail per precision, and its smem bytes
   int tail64 = 0, tail32 = 0;
-  // FP32 cluster tail (mp_ctail.cuh): its top level (-1: not used), shared memory per
-  // CTA and the offset of its coarsest-rhs scratch
-  int ctail32 = -1, ctail_scratch = 0;
-  size_t ctail_bytes = 0;
+  CtPlan ct32, ct64;  // cluster tails
   size_t tail64_bytes = 0, tail32_bytes = 0;
+  // level visits: exchange slots, {epoch base, CTAs done}, epochs used since the
+  // slots were last cleared (an upper bound) and per V-cycle
+  unsigned long long *mail = nullptr;
+  unsigned *epoch = nullptr;
+  size_t mail_words = 0;
+  unsigned long long epochs_used = 0, epochs_cycle = 0;
   bool capturing = false;
   std::vector<int> cap_ids, cap_levels;
 };
@@ -330,11 +360,26 @@ mp_status reduce_after(mp_poisson *hd, int np, int op, int slot) {
   return launch_ok();
 }
 
+// empty the exchange slots of the level visits and restart their epochs
+mp_status clear_visits(mp_poisson *hd) {
+  if (hd->mail) {
+    CK(cudaMemsetAsync(hd->mail, 0, hd->mail_words * sizeof(unsigned long long), hd->st));
+    CK(cudaMemsetAsync(hd->epoch, 0, 2 * sizeof(unsigned), hd->st));
+  }
+  hd->epochs_used = 0;
+  return MP_OK;
+}
+
 mp_status read_scalars(mp_poisson *hd) {
   CK(cudaMemcpyAsync(hd->scal_h, hd->scal, S_COUNT * sizeof(double), cudaMemcpyDeviceToHost,
                      hd->st));
   CK(cudaStreamSynchronize(hd->st));
   prof_resolve(hd);
+  if (hd->scal_h[S_ERR] != 0.0) {  // a bounded device wait gave up: start over clean
+    CKS(clear_visits(hd));
+    CK(cudaMemsetAsync(hd->scal + S_ERR, 0, sizeof(double), hd->st));
+    return MP_ERR_TIMEOUT;
+  }
   return MP_OK;
 }
 
@@ -361,48 +406,103 @@ template <> struct LV<float> {
   static float *dd(Level &l) { return l.dd32; }
 };
 
-// The FP32 cluster tail from level l down (one launch of a CT_CTAS cluster).
-mp_status ctail_launch(mp_poisson *hd, int l, const float *rhs, float *x) {
-  CtArgs a{};
-  a.nlev = (int)hd->L.size() - l;
+template <typename T>
+const CtPlan &ct_plan(const mp_poisson *hd) {
+  if constexpr (sizeof(T) == 8)
+    return hd->ct64;
+  else
+    return hd->ct32;
+}
+
+// The cluster tail from its top level down: one launch of one cluster.
+template <typename T>
+mp_status ctail_launch(mp_poisson *hd, const T *rhs, T *x) {
+  const CtPlan &pl = ct_plan<T>(hd);
+  CtArgs<T> a{};
+  a.nlev = (int)hd->L.size() - pl.top;
   a.Minv = hd->Minv;
   a.singular = hd->outflow == 0;
-  int off = 0;
+  a.mail = pl.mail;
+  a.mail_words = pl.mail_words;
+  a.err = hd->scal + S_ERR;
   double bytes = 0.0;
   for (int q = 0; q < a.nlev; ++q) {
-    Level &t = hd->L[l + q];
-    // the levels the one-CTA tail would take keep its sweep cap
-    const int cap = l + q >= hd->tail32 ? TAIL32_NU_MAX : 1 << 20;
-    const int ppc = std::max(1, t.d.nz / CT_CTAS);
-    a.lv[q] = CtLevel{t.d, (int)t.n, std::min(t.nu1, cap), std::min(t.nu2, cap), ppc, off,
-                      t.bx32, t.by32, t.bz32, t.idiag32, hd->outflow ? t.dd32 : nullptr};
-    off += ct_slab_floats(t.d, ppc, hd->outflow != 0);
-    bytes += 16.0 * t.n;
+    Level &t = hd->L[pl.top + q];
+    // the levels the FP32 one-CTA tail would take keep its sweep cap
+    const int cap = sizeof(T) == 4 && pl.top + q >= hd->tail32 ? TAIL32_NU_MAX : 1 << 20;
+    const CtPlan::Cut &c = pl.cut[q];
+    a.lv[q] = CtLevel<T>{t.d, (int)t.n, std::min(t.nu1, cap), std::min(t.nu2, cap), c.py, c.pz,
+                         c.bym, c.bzm, c.off, LV<T>::bx(t), LV<T>::by(t), LV<T>::bz(t),
+                         LV<T>::idiag(t), hd->outflow ? LV<T>::dd(t) : nullptr};
+    bytes += 4.0 * sizeof(T) * t.n;
   }
-  prof_begin(hd, K_CTAIL32, l);
+  const int id = kid<T>(K_CTAIL64, K_CTAIL32);
+  prof_begin(hd, id, pl.top);
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(CT_CTAS);
+  cfg.gridDim = dim3(pl.ctas);
   cfg.blockDim = dim3(CTL_THREADS);
-  cfg.dynamicSmemBytes = hd->ctail_bytes;
+  cfg.dynamicSmemBytes = pl.bytes;
   cfg.stream = hd->st;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = CT_CTAS;
+  attr[0].val.clusterDim.x = pl.ctas;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = hd->prof_on ? 1 : 2;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, k_ctail, a, hd->ctail_scratch, rhs, x);
+  cudaError_t e = cudaLaunchKernelEx(&cfg, k_ctail<T>, a, rhs, x);
   if (e != cudaSuccess && cfg.numAttrs == 2) {  // without the programmatic launch
     cudaGetLastError();
     cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, k_ctail, a, hd->ctail_scratch, rhs, x);
+    e = cudaLaunchKernelEx(&cfg, k_ctail<T>, a, rhs, x);
   }
-  prof_end(hd, K_CTAIL32, l, bytes);
+  prof_end(hd, id, pl.top, bytes);
   if (e != cudaSuccess) return MP_ERR_CUDA;
   return launch_ok();
+}
+
+// One visit of level l in one cooperative launch (mp_visit.cuh): down from a zero
+// iterate to the coarser right-hand side, or up from the coarser iterate.
+template <typename T, bool UP>
+mp_status visit_launch(mp_poisson *hd, int l, const T *rhs, T *x) {
+  Level &lv = hd->L[l], &lc = hd->L[l + 1];
+  const VisitPlan &pl = sizeof(T) == 8 ? lv.vis64 : lv.vis32;
+  VisitArgs<T> a{};
+  a.x = x;
+  a.rhs = rhs;
+  if constexpr (sizeof(T) == 8) {
+    a.hx = lv.bx, a.hy = lv.by, a.hz = lv.bz;
+    a.idiag = lv.idiag, a.diag = lv.diag;
+  } else {
+    a.hx = lv.bx16, a.hy = lv.by16, a.hz = lv.bz16;
+    a.dd = hd->outflow ? lv.dd16 : nullptr;
+  }
+  a.ec = LV<T>::e(lc);
+  a.bc = LV<T>::b(lc);
+  a.d = lv.d, a.dc = lc.d;
+  a.nu = UP ? lv.nu2 : lv.nu1;
+  a.py = pl.py, a.pz = pl.pz, a.bym = pl.bym, a.bzm = pl.bzm;
+  a.fs = hd->fs16, a.inv_fs = 1.f / hd->fs16;
+  a.mail = hd->mail, a.epoch = hd->epoch, a.err = hd->scal + S_ERR;
+  const int id = kid<T>(K_VISIT64, K_RBGS32F);
+  // b and the faces once; x written (up: also read), the coarser level's vector
+  const double face = sizeof(T) == 8 ? 4.0 * 8.0 : 3.0 * 2.0;
+  prof_begin(hd, id, l);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(pl.py * pl.pz);
+  cfg.blockDim = dim3(VS_THREADS);
+  cfg.dynamicSmemBytes = pl.smem;
+  cfg.stream = hd->st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = pl.py * pl.pz > 1 ? 1 : 0;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, k_visit<T, UP>, a);
+  prof_end(hd, id, l, lv.n * ((UP ? 3.125 : 2.125) * sizeof(T) + face));
+  return e == cudaSuccess ? MP_OK : MP_ERR_CUDA;
 }
 
 // One symmetric V-cycle with zero initial guess: x ~= At^-1 rhs on level l.
@@ -413,9 +513,7 @@ mp_status ctail_launch(mp_poisson *hd, int l, const float *rhs, float *x) {
 template <typename T>
 mp_status vcycle(mp_poisson *hd, int l, const T *rhs, T *x) {
   Level &lv = hd->L[l];
-  if constexpr (sizeof(T) == 4) {
-    if (l == hd->ctail32 && hd->opts.coarse_cluster) return ctail_launch(hd, l, rhs, x);
-  }
+  if (l == ct_plan<T>(hd).top && hd->opts.coarse_cluster) return ctail_launch<T>(hd, rhs, x);
   const int tail = sizeof(T) == 8 ? hd->tail64 : hd->tail32;
   if (l == tail && l < (int)hd->L.size() - 1) {
     TailArgs a{};
@@ -448,6 +546,11 @@ mp_status vcycle(mp_poisson *hd, int l, const T *rhs, T *x) {
     return launch_ok();
   }
   Level &lc = hd->L[l + 1];
+  if ((sizeof(T) == 8 ? lv.vis64 : lv.vis32).py > 0 && hd->opts.smoother == 1) {
+    CKS((visit_launch<T, false>(hd, l, rhs, x)));
+    CKS(vcycle<T>(hd, l + 1, LV<T>::b(lc), LV<T>::e(lc)));
+    return visit_launch<T, true>(hd, l, rhs, x);
+  }
   T *bx = LV<T>::bx(lv), *by = LV<T>::by(lv), *bz = LV<T>::bz(lv);
   T *diag = LV<T>::diag(lv), *idiag = LV<T>::idiag(lv);
   const double sz = sizeof(T), nl = (double)lv.n;
@@ -545,6 +648,7 @@ void destroy_graphs(mp_poisson *hd) {
 // small coarse levels where launch latency, not bandwidth, sets the time.
 template <typename T>
 mp_status run_vcycle(mp_poisson *hd, const T *rhs, T *x) {
+  hd->epochs_used += hd->epochs_cycle;
   if (hd->prof_on) return vcycle<T>(hd, 0, rhs, x);
   mp_poisson::Graph *g = nullptr;
   for (auto &e : hd->graphs)
@@ -1043,6 +1147,8 @@ mp_status diag_fields(mp_poisson *hd, int mode);
 mp_status solve_assembled(mp_poisson *hd, double *p, double tol, std::vector<double> *hist) {
   Level &l0 = hd->L[0];
   const mp_opts &o = hd->opts;
+  // epochs are 32-bit: clear the exchange slots long before they come round
+  if (hd->epochs_used > (1ull << 30)) CKS(clear_visits(hd));
   CKS(read_scalars(hd));
   hd->bnorm = std::sqrt(hd->scal_h[S_BB]);
   hd->stats = mp_stats{};
@@ -1228,6 +1334,8 @@ void apply_nu(mp_poisson *hd) {
     hd->L[l].nu2 = (int)std::min<long>(hd->opts.nu_max, (long)hd->opts.nu2 * f);
     f = std::min<long>(f * hd->opts.nu_growth, 1L << 20);
   }
+  hd->epochs_cycle = 0;
+  for (const Level &lv : hd->L) hd->epochs_cycle += 2ull * lv.nu1 + 2ull * lv.nu2;
 }
 
 // Per-level diagonal and face copies for the precisions in mode (bits: 1 = the
@@ -1323,8 +1431,75 @@ mp_status geometry(mp_poisson *hd, const double *phi, double rho_l, double rho_g
   return MP_OK;
 }
 
-// Grid of the fused sweep for every FP32 level it runs on (levels above the
-// one-CTA tail, nx a multiple of 8), and the second iterate buffer.  The
+// Blocks of a level visit: whole x rows, cuts at even y and z, at most one CTA
+// per SM.  Of the cuts that fit shared memory the one of least estimated
+// half-sweep time: the largest block's cells (FP32: ~16 ns per 32 updates; FP64:
+// the pipe's rate, 7 operations an update), its halo words, and the L2 round
+// trip of an exchange (~1.3 us) unless one block holds the level.
+template <typename T>
+mp_status visit_plan(VisitPlan *out, const Dims &d, bool dd, int sms, size_t limit) {
+  *out = VisitPlan{};
+  if (d.nx % 2 || d.ny % 2 || d.nz % 2) return MP_OK;
+  const int uy = d.ny / 2, uz = d.nz / 2;
+  double best = 0.0;
+  for (int py = 1; py <= std::min(uy, sms); ++py)
+    for (int pz = 1; pz <= std::min(uz, sms / py); ++pz) {
+      VisitPlan p;
+      p.py = py, p.pz = pz;
+      p.bym = 2 * ((uy + py - 1) / py), p.bzm = 2 * ((uz + pz - 1) / pz);
+      p.smem = vs_smem<T>(d.nx, p.bym, p.bzm, dd);
+      if (p.smem > limit) continue;
+      const double cells = (double)d.nx * p.bym * p.bzm;
+      double ns = sizeof(T) == 8 ? 100.0 + 0.89 * cells : 60.0 + 0.25 * cells;
+      if (py * pz > 1) ns += 1300.0 + 0.06 * (double)vs_slots(d.nx, p.bym, p.bzm);
+      if (out->py == 0 || ns < best) {
+        best = ns;
+        *out = p;
+      }
+    }
+  if (out->py == 0) return MP_OK;
+  auto down = k_visit<T, false>;
+  auto up = k_visit<T, true>;
+  CK(cudaFuncSetAttribute(down, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit));
+  CK(cudaFuncSetAttribute(up, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit));
+  int occ_d = 0, occ_u = 0;
+  CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_d, down, VS_THREADS, out->smem));
+  CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_u, up, VS_THREADS, out->smem));
+  if (occ_d < 1 || occ_u < 1) *out = VisitPlan{};
+  return MP_OK;
+}
+
+// Plans of every level above the one-CTA tails, and the exchange slots they need
+mp_status visit_setup(mp_poisson *hd) {
+  int dev = 0, sms = 0, coop = 0, optin = 0;
+  CK(cudaGetDevice(&dev));
+  CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  CK(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
+  CK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+  if (!coop) return MP_OK;
+  size_t words = 0;
+  for (int l = 0; l + 1 < (int)hd->L.size(); ++l) {
+    Level &lv = hd->L[l];
+    if (l < hd->tail64) {
+      CKS((visit_plan<double>(&lv.vis64, lv.d, false, sms, (size_t)optin)));
+      const VisitPlan &p = lv.vis64;
+      words = std::max(words, 2 * vs_slots(lv.d.nx, p.bym, p.bzm) * p.py * p.pz * 2);
+    }
+    if (l < hd->tail32 && lv.n <= VISIT_TOP32) {
+      CKS((visit_plan<float>(&lv.vis32, lv.d, hd->outflow != 0, sms, (size_t)optin)));
+      const VisitPlan &p = lv.vis32;
+      words = std::max(words, 2 * vs_slots(lv.d.nx, p.bym, p.bzm) * p.py * p.pz);
+    }
+  }
+  if (words == 0) return MP_OK;
+  hd->mail_words = words;
+  CKS(dalloc(hd, &hd->mail, words));
+  CKS(dalloc(hd, &hd->epoch, (size_t)2));
+  return MP_OK;
+}
+
+// Grid of the fused sweep for every FP32 level it runs on (at least FUSED_MIN
+// cells, nx a multiple of 8), and the second iterate buffer.  The
 // z-chunk count minimises (waves of resident CTAs) x (planes per chunk +
 // the ~3.5 planes a chunk stages beyond its own).
 mp_status fused_setup(mp_poisson *hd) {
@@ -1340,7 +1515,7 @@ mp_status fused_setup(mp_poisson *hd) {
   const long slots = (long)std::max(1, sms) * std::max(1, per_sm);
   for (int l = 0; l < hd->tail32 && l < (int)hd->L.size() - 1; ++l) {
     Level &lv = hd->L[l];
-    if (lv.d.nx % 8 != 0) continue;
+    if (lv.d.nx % 8 != 0 || lv.n < FUSED_MIN) continue;
     lv.ftx = (lv.d.nx + FS_TX - 1) / FS_TX;
     lv.fty = (lv.d.ny + FS_TY - 1) / FS_TY;
     const long tiles = (long)lv.ftx * lv.fty;
@@ -1359,46 +1534,86 @@ mp_status fused_setup(mp_poisson *hd) {
   return MP_OK;
 }
 
-// FP32 cluster tail (mp_ctail.cuh): the level above the one-CTA tail and every
-// level below it in the shared memory of a CT_CTAS-CTA cluster, when every
-// level's z-planes split evenly, the slabs fit and the device runs the cluster
-mp_status ctail_setup(mp_poisson *hd) {
-  hd->ctail32 = -1;
-  const int nl = (int)hd->L.size(), top = hd->tail32 - 1;
-  if (top < 0 || hd->tail32 >= nl - 1 || nl - top > CT_MAX_LEVELS) return MP_OK;
-  if (hd->L.back().n > (size_t)CT_MAX_COARSE) return MP_OK;
-  size_t floats = 0;
-  for (int l = top; l < nl; ++l) {
-    const Dims &d = hd->L[l].d;
-    if (d.nz > CT_CTAS && d.nz % CT_CTAS != 0) return MP_OK;
-    floats += ct_slab_floats(d, std::max(1, d.nz / CT_CTAS), hd->outflow != 0);
-  }
-  const size_t bytes = (floats + CT_MAX_COARSE) * sizeof(float);
-  if (bytes > CT_SMEM_MAX) return MP_OK;
-  if (cudaFuncSetAttribute(k_ctail, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) !=
-      cudaSuccess) {
+// Cluster tail (mp_ctail.cuh): from the largest level of at most CT_TOP cells
+// whose blocks, and those of every coarser level, fit the shared memory of a
+// cluster this device can run.  A level is cut into the blocks of least
+// estimated half-sweep time: the largest block's cells and, with more than one
+// block, an exchange (~0.35 us).
+template <typename T>
+mp_status ctail_setup(mp_poisson *hd, CtPlan *out) {
+  *out = CtPlan{};
+  int dev = 0, optin = 0;
+  CK(cudaGetDevice(&dev));
+  CK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+  const int nl = (int)hd->L.size();
+  const bool dd = hd->outflow != 0;
+  const double per_cell = sizeof(T) == 8 ? 1.1 : 0.19;  // ns a half-sweep
+  if (cudaFuncSetAttribute(k_ctail<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
+      cudaSuccess)
     cudaGetLastError();
-    return MP_OK;
-  }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(CT_CTAS);
-  cfg.blockDim = dim3(CTL_THREADS);
-  cfg.dynamicSmemBytes = bytes;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = CT_CTAS;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  int clusters = 0;
-  if (cudaOccupancyMaxActiveClusters(&clusters, k_ctail, &cfg) != cudaSuccess || clusters < 1) {
-    cudaGetLastError();
-    return MP_OK;
-  }
-  hd->ctail32 = top;
-  hd->ctail_bytes = bytes;
-  hd->ctail_scratch = (int)floats;
+  for (int ctas = CT_MAX_CTAS; ctas >= 8; ctas /= 2)
+    for (int top = 0; top < nl - 1; ++top) {
+      const Dims &dt = hd->L[top].d;
+      if (hd->L[top].n > (sizeof(T) == 8 ? CT_TOP64 : CT_TOP32) || dt.nx > 2 * CTL_THREADS ||
+          nl - top > CT_MAX_LEVELS)
+        continue;
+      CtPlan p;
+      p.top = top;
+      p.ctas = ctas;
+      size_t elems = 0;
+      int slots = 0;
+      for (int l = top; l < nl; ++l) {
+        const Dims &d = hd->L[l].d;
+        CtPlan::Cut &c = p.cut[l - top];
+        const bool coarsest = l == nl - 1;
+        c = CtPlan::Cut{1, 1, d.ny, d.nz, (int)elems};
+        if (!coarsest) {
+          const int uy = d.ny / 2, uz = d.nz / 2;
+          double best = -1.0;
+          for (int py = 1; py <= std::min(uy, ctas); ++py)
+            for (int pz = 1; pz <= std::min(uz, ctas / py); ++pz) {
+              const int bym = 2 * ((uy + py - 1) / py), bzm = 2 * ((uz + pz - 1) / pz);
+              const double words = 0.5 * d.nx * ((py > 1 ? 2 * bzm : 0) + (pz > 1 ? 2 * bym : 0));
+              const double ns =
+                  per_cell * d.nx * bym * bzm + (py * pz > 1 ? 350.0 + 0.2 * words : 0.0);
+              if (best < 0.0 || ns < best) {
+                best = ns;
+                c = CtPlan::Cut{py, pz, bym, bzm, (int)elems};
+              }
+            }
+          if (c.py * c.pz > 1) slots = std::max(slots, ct_slots(d, c.bym, c.bzm));
+        }
+        elems += ((size_t)ct_elems(d, c.bym, c.bzm, dd, coarsest) + 3) / 4 * 4;
+      }
+      p.mail = (int)(elems * sizeof(T));
+      p.mail_words = 2 * slots * (sizeof(T) == 8 ? 2 : 1);
+      p.bytes = (size_t)p.mail + (size_t)p.mail_words * 8;
+      if (p.bytes + 1024 > (size_t)optin) continue;  // (a little is static)
+      if (cudaFuncSetAttribute(k_ctail<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               optin - 1024) != cudaSuccess) {
+        cudaGetLastError();
+        return MP_OK;
+      }
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(ctas);
+      cfg.blockDim = dim3(CTL_THREADS);
+      cfg.dynamicSmemBytes = p.bytes;
+      cudaLaunchAttribute attr[1];
+      attr[0].id = cudaLaunchAttributeClusterDimension;
+      attr[0].val.clusterDim.x = ctas;
+      attr[0].val.clusterDim.y = 1;
+      attr[0].val.clusterDim.z = 1;
+      cfg.attrs = attr;
+      cfg.numAttrs = 1;
+      int clusters = 0;
+      if (cudaOccupancyMaxActiveClusters(&clusters, k_ctail<T>, &cfg) != cudaSuccess ||
+          clusters < 1) {
+        cudaGetLastError();
+        continue;
+      }
+      *out = p;
+      return MP_OK;
+    }
   return MP_OK;
 }
 
@@ -1548,8 +1763,10 @@ mp_status create(mp_poisson *hd, mp_grid g, double h, const mp_bc bc[3]) {
     }
   }
   // fused FP32 sweep: levels above the one-CTA tail with nx a multiple of 8
+  CKS(visit_setup(hd));
   CKS(fused_setup(hd));
-  CKS(ctail_setup(hd));
+  CKS(ctail_setup<float>(hd, &hd->ct32));
+  CKS(ctail_setup<double>(hd, &hd->ct64));
   CK(cudaFuncSetAttribute(k_tail<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                           (int)std::max<size_t>(hd->tail64_bytes, 1)));
   CK(cudaFuncSetAttribute(k_tail<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -866,3 +866,83 @@ def test_coarsest_inverse_solves_a_single_level_directly(shape, outflow):
         assert s.stats()["relres"] <= TOL and s.stats()["levels"] == 1
         assert rel_l2(host(p), ref["p"]) < PARITY
         s.close()
+
+
+def _smoother_case(shape, bc, seed=3):
+    """Two bubbles (and a pool where z allows) in a box of `shape` (nz, ny, nx) cells, and
+    a random right-hand side."""
+    nz, ny, nx = shape
+    h = 1.0 / max(shape)
+    lo = min(ny, nz, nx) * h
+    bub = [((0.3 * nx * h, 0.4 * ny * h, 0.3 * nz * h), 0.2 * lo),
+           ((0.7 * nx * h, 0.6 * ny * h, 0.75 * nz * h), 0.15 * lo)]
+    phi = synth.level_set(shape, h, bub, bc=[P if b == P else N for b in bc])
+    rhs = rng_np(seed).standard_normal(shape)
+    return dev(phi), dev(rhs), h
+
+
+@pytest.mark.parametrize("shape,bc,precision,opts", [
+    ((56, 24, 40), (P, P, N), 0, {}), ((56, 24, 40), (P, P, N), 1, {}),
+    ((24, 20, 16), (N, N, N), 0, {"nu1": 3, "nu2": 3}), ((24, 20, 16), (N, N, N), 1, {}),
+    ((48, 64, 96), (D, N, P), 0, {}), ((48, 64, 96), (D, N, P), 1, {}),
+    ((40, 12, 28), (P, P, P), 1, {}), ((40, 12, 28), (P, P, P), 0, {"nu1": 1, "nu2": 1}),
+    ((64, 64, 64), (P, N, ND), 1, {"method": 1, "max_iters": 5}), ((64, 64, 64), (P, P, N), 0, {}),
+    ((96, 64, 80), (P, P, N), 1, {})])
+def test_level_visits_bitwise_equal_per_colour_launches(shape, bc, precision, opts):
+    """A level visited in one launch (all its sweeps in shared memory, boundary rows exchanged
+    between the blocks, restriction or prolongation included) gives the bits of the launches it
+    replaces: one block and many, blocks of unequal size, axes that one block spans, walls,
+    periodic and outflow sides, FP32 on FP16 faces and FP64."""
+    phi, rhs, h = _smoother_case(shape, bc)
+    out = []
+    for smoother in (1, 0):
+        s = Poisson(phi, h, bc, 1.0, 1e-3, 0.05, precision=precision, smoother=smoother,
+                    coarse_cluster=0, **opts)
+        p, it, hist = s.solve(rhs, tol=TOL, allow_not_converged="max_iters" in opts)
+        out.append((p, it, list(hist)))
+        names = {e["name"] for e in s.profile()}
+        visited = "rbgs_f32_fused" if precision else "level_visit_f64"
+        assert (visited in names) == (smoother == 1), names
+        s.close()
+    assert out[0][1] == out[1][1] and out[0][2] == out[1][2]
+    assert torch.equal(out[0][0], out[1][0])
+
+
+@pytest.mark.parametrize("shape,bc", [((160, 192, 160), (P, N, N)), ((192, 160, 160), (N, P, P))])
+def test_fused_sweep_bitwise_on_ragged_large_levels(shape, bc):
+    """The fused sweep's smallest levels (just above 4e6 cells): x tiles that overhang the grid,
+    walls and wrapping in x and y."""
+    phi, rhs, h = _smoother_case(shape, bc)
+    out = []
+    for smoother in (1, 0):
+        s = Poisson(phi, h, bc, 1.0, 1e-3, 0.05, precision=1, smoother=smoother, max_iters=6)
+        p, it, hist = s.solve(rhs, tol=TOL, allow_not_converged=True)
+        out.append((p, list(hist)))
+        fused = [e for e in s.profile() if e["name"] == "rbgs_f32_fused" and e["level"] == 0]
+        assert bool(fused) == (smoother == 1)
+        s.close()
+    assert out[0][1] == out[1][1] and torch.equal(out[0][0], out[1][0])
+
+
+@pytest.mark.parametrize("shape,bc", [((56, 24, 40), (P, P, N)), ((24, 20, 40), (N, D, P)),
+                                      ((28, 12, 20), (P, P, P)), ((16, 48, 12), (N, N, ND)),
+                                      ((8, 8, 8), (P, P, N)), ((64, 16, 32), (P, P, N))])
+@pytest.mark.parametrize("precision", [0, 1])
+def test_cluster_tail_on_ragged_and_outflow_grids(shape, bc, precision):
+    """The cluster tail on grids whose planes do not split evenly, with outflow sides, one block
+    or many, a coarsest level of odd size, FP32 and FP64: the oracle's pressure, and the
+    iterations of the per-level launches to within two."""
+    phi, rhs, h = _smoother_case(shape, bc)
+    ref = oracle.solve(host(phi), host(rhs), h, 1.0, 1e-3, 0.05, bc, tol=REF_TOL)
+    its = []
+    for cl in (1, 0):
+        s = Poisson(phi, h, bc, 1.0, 1e-3, 0.05, precision=precision, coarse_cluster=cl)
+        p, it, _ = s.solve(rhs, tol=TOL)
+        assert s.stats()["relres"] <= TOL
+        assert rel_l2(host(p), ref["p"]) < PARITY
+        ran = any(e["name"] == ("coarse_cluster_f32" if precision else "coarse_cluster_f64")
+                  for e in s.profile())
+        assert ran == (cl == 1)
+        its.append(it)
+        s.close()
+    assert abs(its[0] - its[1]) <= 2
