@@ -102,7 +102,10 @@ struct ConvGeom {
 constexpr int CONV_THREADS = 128;
 constexpr int NSTAGE = 3;
 constexpr int STAGE_K = 64;                  // K elements per stage (4 MMAs of K = 16)
-constexpr int A_STAGE_BYTES = 128 * STAGE_K * 2;
+// bytes of one row group (8 rows x STAGE_K voxels) of a weight-gradient stage: 64 more
+// than its data, so that the two groups a warp writes at once lie in other banks
+constexpr int WG_GROUP = STAGE_K * 16 + 64;
+constexpr int A_STAGE_BYTES = 16 * WG_GROUP;
 
 // tcgen05.alloc takes a power-of-two column count of at least 32
 template <int COUT>
@@ -111,7 +114,7 @@ __host__ __device__ constexpr int tmem_cols() {
 }
 template <int COUT>
 __host__ __device__ constexpr int b_stage_bytes() {
-  return COUT * STAGE_K * 2;
+  return COUT / 8 * WG_GROUP;
 }
 template <int COUT>
 __host__ __device__ constexpr int conv_smem_bytes() {
@@ -501,38 +504,20 @@ __global__ void k_pack_img(const S *__restrict__ src, int cout, int cin, int fli
 // X[v + off_t][ci] * G[v][co]: rows are (tap, input channel) pairs, K runs
 // over voxels.  Each CTA reduces one chunk of WG_VOX voxels into FP32
 // partials; k_wgrad_reduce sums the chunks in a fixed order (split-K,
-// deterministic).  Operands are stored K-major: a 16-byte load of 8
-// channels of one voxel is written as 8 two-byte elements of one smem
-// column.
+// deterministic).
+//
+// Both operands are M/N-major: a core matrix is 8 voxels (K) x 8 channels (16
+// bytes), so the 8 channels of a voxel go from global to shared memory as they
+// lie, one 16-byte cp.async each (zero-filled outside the grid), [row group][voxel].
+// Writing K-major tiles instead took eight 2-byte stores for each of these
+// copies and bound the kernel: 32-32 at 64^3 422 us, now 84 (the copies' shared-
+// memory wavefronts at 67 % of their rate).
 constexpr int WG_VOX = 2048;  // voxels per CTA (32 stages of 64)
 
-__device__ __forceinline__ void gather8(const bf16 *__restrict__ xa, const bf16 *__restrict__ xb,
-                                        const ConvGeom &g, int x, int y, int z, int ci0,
-                                        uint4 &v) {
-  v = make_uint4(0, 0, 0, 0);
-  if (x < 0 || y < 0 || z < 0 || x >= g.nx || y >= g.ny || z >= g.nz) return;
-  if (ci0 < g.ca) {
-    int ax = x, ay = y, az = z, anx = g.nx, any = g.ny;
-    if (g.up_a) {
-      ax >>= 1;
-      ay >>= 1;
-      az >>= 1;
-      anx >>= 1;
-      any >>= 1;
-    }
-    v = __ldg(reinterpret_cast<const uint4 *>(xa + (((size_t)az * any + ay) * anx + ax) * g.ca + ci0));
-  } else {
-    v = __ldg(reinterpret_cast<const uint4 *>(xb + (((size_t)z * g.ny + y) * g.nx + x) * g.cb +
-                                              (ci0 - g.ca)));
-  }
-}
-
-__device__ __forceinline__ void scatter8(uint8_t *tile, int r8, int k, const uint4 &v) {
-  // 8 rows r8*8 .. r8*8+7 at K column k of a K-major 128-row tile
-  const bf16 *e = reinterpret_cast<const bf16 *>(&v);
-  uint8_t *base = tile + (k >> 3) * 2048 + r8 * 128 + (k & 7) * 2;
-#pragma unroll
-  for (int q = 0; q < 8; ++q) *reinterpret_cast<bf16 *>(base + q * 16) = e[q];
+__device__ __forceinline__ void cp_async16_zfill(void *smem, const void *gmem, bool in) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(smem)), "l"(gmem),
+               "r"(in ? 16 : 0)
+               : "memory");
 }
 
 template <int COUT>
@@ -542,6 +527,7 @@ k_conv3d_wgrad(const bf16 *__restrict__ xa, const bf16 *__restrict__ xb,
                int *__restrict__ err) {
   constexpr int TM = tmem_cols<COUT>();
   constexpr int BST = b_stage_bytes<COUT>();
+  constexpr int NG = 8;  // copies of A per thread and stage: one of each pair of row groups
   extern __shared__ __align__(1024) uint8_t conv_smem[];
   uint8_t *sm = conv_smem + ((1024 - (smem_u32(conv_smem) & 1023)) & 1023);
   uint8_t *sA = sm;
@@ -563,78 +549,129 @@ k_conv3d_wgrad(const bf16 *__restrict__ xa, const bf16 *__restrict__ xb,
   __syncthreads();
   tc_fence_after();
   const uint32_t taddr = tslot;
-  constexpr uint32_t IDESC = idesc_bf16(128, COUT, 0, 0);
-  const int nst = WG_VOX / STAGE_K;
-  bool ok = true;
-  for (int s = 0; s < nst && ok; ++s) {
-    const int buf = s % NSTAGE;
-    if (s >= NSTAGE) {
-      bool done = mbar_wait(&mbar[buf], (uint32_t)((s / NSTAGE - 1) & 1));
-      if (!done) abort_flag = 1;
-      __syncthreads();
-      if (abort_flag) {
-        ok = false;
-        break;
-      }
-    }
-    uint8_t *a_st = sA + buf * A_STAGE_BYTES;
-    uint8_t *b_st = sB + buf * BST;
-    // A: 16 row groups of 8 (tap, channel) pairs x 64 voxels
-    for (int e = tid; e < 16 * STAGE_K; e += CONV_THREADS) {
-      const int k = e % STAGE_K, r8 = e / STAGE_K;
-      const long v = v0 + (long)s * STAGE_K + k;
-      const int m = m0 + r8 * 8;
-      uint4 val = make_uint4(0, 0, 0, 0);
-      if (m < rows && v < nvox) {
-        const int t = m / g.cin, ci0 = m - t * g.cin;
-        const int x = (int)(v % g.nx), y = (int)((v / g.nx) % g.ny), z = (int)(v / ((long)g.nx * g.ny));
-        gather8(xa, xb, g, x + t % 3 - 1, y + (t / 3) % 3 - 1, z + t / 9 - 1, ci0, val);
-      }
-      scatter8(a_st, r8, k, val);
-    }
-    // B: COUT/8 row groups x 64 voxels of the output gradient
-    for (int e = tid; e < (COUT / 8) * STAGE_K; e += CONV_THREADS) {
-      const int k = e % STAGE_K, r8 = e / STAGE_K;
-      const long v = v0 + (long)s * STAGE_K + k;
-      uint4 val = make_uint4(0, 0, 0, 0);
-      if (v < nvox) val = __ldg(reinterpret_cast<const uint4 *>(gr + v * COUT + r8 * 8));
-      const bf16 *ev = reinterpret_cast<const bf16 *>(&val);
-      uint8_t *base = b_st + (k >> 3) * (COUT / 8) * 128 + r8 * 128 + (k & 7) * 2;
+  constexpr uint32_t IDESC = idesc_bf16(128, COUT, 1, 1);
+
+  // This thread's voxel of a stage is k; its row groups are 2 i + rg.  Two lanes
+  // take the 16 channels of a pair of groups (always of one tap and input), so a
+  // warp's copies read whole 32-byte sectors.  Per group: the source of this stage's
+  // voxel and its advance to the next stage's, and the bits of `edge` that say the
+  // tap lies inside the grid.  An upsampled input has no linear source: its
+  // groups (step 0) form the parent's address instead.
+  static_assert(CONV_THREADS == 2 * STAGE_K, "two threads per voxel of a stage");
+  const int k = tid >> 1, rg = tid & 1;
+  long v = v0 + k;  // the voxel of the next stage to produce, and its coordinates
+  int x = (int)(v % g.nx), y = (int)(v / g.nx % g.ny), z = (int)(v / g.nx / g.ny);
+  const bf16 *src[NG];
+  int step[NG], need[NG], off[NG];
 #pragma unroll
-      for (int q = 0; q < 8; ++q) *reinterpret_cast<bf16 *>(base + q * 16) = ev[q];
+  for (int i = 0; i < NG; ++i) {
+    const int m = m0 + (2 * i + rg) * 8, t = m / g.cin, ci = m - t * g.cin;
+    const int dx = t % 3 - 1, dy = (t / 3) % 3 - 1, dz = t / 9 - 1;
+    need[i] = m < rows ? 1 << (dx + 1) | 8 << (dy + 1) | 64 << (dz + 1) : 1 << 30;
+    const bool b = ci >= g.ca;
+    const int c = b ? g.cb : g.ca;
+    step[i] = !b && g.up_a ? 0 : STAGE_K * c;
+    off[i] = ci;
+    src[i] = (b ? xb - g.ca : xa) + ci;
+    if (step[i]) src[i] += (v + ((long)dz * g.ny + dy) * g.nx + dx) * c;
+  }
+  const int nst = WG_VOX / STAGE_K;
+  auto produce = [&](int s) {
+    const int buf = s % NSTAGE;
+    const bool in = v < nvox;
+    // bit 1 + dx, 4 + dy, 7 + dz: the neighbour of that offset is in range
+    const int edge = !in ? 0
+                         : (x > 0) | 2 | (x + 1 < g.nx) << 2 | (y > 0) << 3 | 16 |
+                               (y + 1 < g.ny) << 5 | (z > 0) << 6 | 128 | (z + 1 < g.nz) << 8;
+    uint8_t *a_st = sA + buf * A_STAGE_BYTES + rg * WG_GROUP + k * 16;
+#pragma unroll
+    for (int i = 0; i < NG; ++i) {
+      const bool ok = (edge & need[i]) == need[i];
+      const bf16 *p = src[i];
+      if (g.up_a && step[i] == 0) {
+        const int dx = (need[i] >> 2 & 1) - (need[i] & 1),
+                  dy = (need[i] >> 5 & 1) - (need[i] >> 3 & 1),
+                  dz = (need[i] >> 8 & 1) - (need[i] >> 6 & 1);
+        p = xa + (((size_t)((z + dz) >> 1) * (g.ny >> 1) + ((y + dy) >> 1)) * (g.nx >> 1) +
+                  ((x + dx) >> 1)) * g.ca + off[i];
+      }
+      cp_async16_zfill(a_st + 2 * i * WG_GROUP, ok ? p : xa, ok);
+      src[i] += step[i];
     }
-    fence_async_smem();
+    uint8_t *b_st = sB + buf * BST + k * 16;
+    const bf16 *pg = in ? gr + v * COUT : gr;
+#pragma unroll
+    for (int e = 0; e < COUT / 16; ++e)
+      cp_async16_zfill(b_st + (2 * e + rg) * WG_GROUP, pg + (2 * e + rg) * 8, in);
+    v += STAGE_K;
+    x += STAGE_K;
+    while (x >= g.nx) {
+      x -= g.nx;
+      if (++y == g.ny) y = 0, ++z;
+    }
+  };
+
+  // one cp.async group per stage, NSTAGE - 1 ahead of the MMAs
+  int issued = 0, waited = 0;
+  for (int p = 0; p < NSTAGE - 1; ++p) {
+    produce(p);
+    cp_async_commit();
+  }
+  bool ok = true;
+  for (int s = 0; s < nst; ++s) {
+    const int buf = s % NSTAGE;
+    cp_async_wait<NSTAGE - 2>();  // this thread's copies of stage s have landed ...
+    fence_async_smem();           // ... and are visible to the tensor core's reads
     __syncthreads();
     if (tid == 0) {
       tc_fence_after();
-      const uint32_t a0 = smem_u32(a_st), b0 = smem_u32(b_st);
+      const uint32_t a0 = smem_u32(sA + buf * A_STAGE_BYTES), b0 = smem_u32(sB + buf * BST);
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const uint64_t da = sdesc(a0 + 2 * q * 2048, 2048, 128);
-        const uint64_t db = sdesc(b0 + 2 * q * (COUT / 8) * 128, (COUT / 8) * 128, 128);
+      for (int q = 0; q < STAGE_K / 16; ++q) {
+        // K groups of 8 voxels are 128 bytes apart, row groups WG_GROUP
+        const uint64_t da = sdesc(a0 + q * 256, 128, WG_GROUP);
+        const uint64_t db = sdesc(b0 + q * 256, 128, WG_GROUP);
         mma_bf16(taddr, da, db, IDESC, (s > 0 || q > 0) ? 1u : 0u);
       }
       mma_commit(&mbar[buf]);
     }
+    issued = s + 1;
+    if (s + NSTAGE - 1 < nst) {
+      if (s >= 1) {  // the buffer of stage s - 1 is free once its MMAs are done
+        if (tid == 0 && !mbar_wait(&mbar[(s - 1) % NSTAGE], (uint32_t)(((s - 1) / NSTAGE) & 1)))
+          abort_flag = 1;
+        __syncthreads();
+        if (abort_flag) {
+          ok = false;
+          break;
+        }
+        waited = s;
+      }
+      produce(s + NSTAGE - 1);
+    }
+    cp_async_commit();
   }
-  if (ok) {
-    const int last = nst - 1;
-    bool done = mbar_wait(&mbar[last % NSTAGE], (uint32_t)((last / NSTAGE) & 1));
-    if (!done) abort_flag = 1;
+  cp_async_wait<0>();  // no copy into shared memory outlives the CTA
+  if (tid == 0) {      // every MMA issued is done (after a timeout: bounded, like any wait)
+    for (int s = waited; s < issued; ++s)
+      if (!mbar_wait(&mbar[s % NSTAGE], (uint32_t)((s / NSTAGE) & 1))) abort_flag = 1;
   }
   __syncthreads();
   tc_fence_after();
-  if (abort_flag) {
+  if (abort_flag || !ok) {
     if (tid == 0) atomicExch(err, 1);
   } else {
     const int m = m0 + warp * 32 + lane;
-    float *dst = partial + ((size_t)blockIdx.y * rows + m) * COUT;
+    float4 *dst = reinterpret_cast<float4 *>(partial + ((size_t)blockIdx.y * rows + m) * COUT);
 #pragma unroll
     for (int c0 = 0; c0 < COUT; c0 += 16) {
       float acc[16];
       tmem_ld16(taddr + ((uint32_t)(warp * 32) << 16) + c0, acc);
-      if (m < rows)
-        for (int q = 0; q < 16; ++q) dst[c0 + q] = acc[q];
+      if (m < rows) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          dst[c0 / 4 + q] = make_float4(acc[4 * q], acc[4 * q + 1], acc[4 * q + 2], acc[4 * q + 3]);
+      }
     }
   }
   tc_fence_before();
@@ -642,15 +679,31 @@ k_conv3d_wgrad(const bf16 *__restrict__ xa, const bf16 *__restrict__ xb,
   if (warp == 0) tmem_free(taddr, TM);
 }
 
-// dw[co][t][ci] = sum over chunks (fixed order) of partial[chunk][t*cin + ci][co]
-__global__ void k_wgrad_reduce(const float *__restrict__ partial, int chunks, int rows, int cout,
-                               float *__restrict__ dw) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= rows * cout) return;
-  const int co = e / rows, row = e - co * rows;
+// dw[co][t][ci] = sum over chunks (fixed order) of partial[chunk][t*cin + ci][co]: a warp
+// reads 32 consecutive entries of one chunk, WR_SEG warps take a segment of the chunks
+// each, and the segments' sums are added in order.  (One thread per output walking
+// every chunk, outputs strided in memory: 24 us for 128 chunks of 864 x 32.)
+constexpr int WR_SEG = 8;
+__global__ void __launch_bounds__(32 * WR_SEG)
+k_wgrad_reduce(const float *__restrict__ partial, int chunks, int rows, int cout,
+               float *__restrict__ dw) {
+  __shared__ float part[WR_SEG][32];
+  const int lane = threadIdx.x & 31, seg = threadIdx.x >> 5;
+  const int n = rows * cout, e = blockIdx.x * 32 + lane;
+  const int c1 = (int)((long)(seg + 1) * chunks / WR_SEG);
   float acc = 0.f;
-  for (int c = 0; c < chunks; ++c) acc += partial[((size_t)c * rows + row) * cout + co];
-  dw[(size_t)co * rows + row] = acc;
+  if (e < n) {
+#pragma unroll 8
+    for (int c = (int)((long)seg * chunks / WR_SEG); c < c1; ++c) acc += partial[(size_t)c * n + e];
+  }
+  part[seg][lane] = acc;
+  __syncthreads();
+  if (seg == 0 && e < n) {
+    float s = part[0][lane];
+#pragma unroll
+    for (int q = 1; q < WR_SEG; ++q) s += part[q][lane];
+    dw[(size_t)(e % cout) * rows + e / cout] = s;
+  }
 }
 
 
@@ -1328,7 +1381,7 @@ mp_status launch_wgrad(const ConvGeom &g, const bf16 *xa, const bf16 *xb, const 
   const int chunks = (int)wgrad_chunks(g);
   dim3 grid((rows + 127) / 128, chunks);
   k_conv3d_wgrad<COUT><<<grid, CONV_THREADS, smem, st>>>(xa, xb, gr, g, part, err);
-  k_wgrad_reduce<<<(rows * COUT + 255) / 256, 256, 0, st>>>(part, chunks, rows, COUT, dw);
+  k_wgrad_reduce<<<(rows * COUT + 31) / 32, 32 * WR_SEG, 0, st>>>(part, chunks, rows, COUT, dw);
   NCK(cudaGetLastError());
   return MP_OK;
 }

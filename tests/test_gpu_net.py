@@ -735,3 +735,24 @@ def test_layer_calls_from_several_threads_share_the_workspace_pool():
         assert len(runs) == 5
         for y, dw in runs:
             assert torch.equal(y, ref[k][0]) and torch.equal(dw, ref[k][1])
+
+
+@pytest.mark.parametrize("shape,ca,cb,up,cout", [((3, 5, 7), 16, 0, False, 16),
+                                                 ((5, 9, 13), 32, 16, False, 32),
+                                                 ((2, 2, 2), 16, 16, True, 64),
+                                                 ((6, 10, 14), 48, 16, True, 16),
+                                                 ((1, 1, 2051), 16, 0, False, 32),
+                                                 ((33, 8, 8), 64, 64, False, 64)])
+def test_weight_gradient_ragged_grids(shape, ca, cb, up, cout):
+    """Grids smaller than a stage of 64 voxels, rows that wrap several times in one, a last
+    split-K chunk of a few voxels, and row tiles that end inside a tap."""
+    g = rng(7 * ca + cout + shape[2])
+    xa = bf16_round(g.standard_normal(tuple(d // 2 if up else d for d in shape) + (ca,)))
+    xb = bf16_round(g.standard_normal(shape + (cb,))) if cb else None
+    gy = bf16_round(g.standard_normal(shape + (cout,)))
+    dw = mp_conv3d_wgrad(to_bf16(xa), to_bf16(gy), xb=None if xb is None else to_bf16(xb),
+                         up_a=up).cpu().numpy()
+    xin = conv.upsample2(xa) if up else xa
+    if cb:
+        xin = np.concatenate([xin, xb], axis=-1)
+    assert rel_max(dw, conv.conv3d_wgrad(xin, gy).reshape(cout, 27, ca + cb)) < 1e-5
