@@ -418,8 +418,8 @@ __device__ __forceinline__ double fx_value(unsigned long long *acc, int j, doubl
 #pragma unroll
   for (int q = 0; q < DEFL_REP; ++q) {
     unsigned long long *a = fx_slot(acc, j, q);
-    hi += (long long)a[0];
-    lo += (long long)a[1];
+    hi += (long long)__ldcg(a);  // (other blocks' atomics: past this SM's L1)
+    lo += (long long)__ldcg(a + 1);
     if (clear) a[0] = a[1] = 0ull;
   }
   return ((double)hi + (double)lo / FX_LO) / scale;
@@ -541,19 +541,31 @@ __global__ void k_defl_maxabs(const int *__restrict__ band, int nband, const T *
     atomicMax(mx, (unsigned long long)__double_as_longlong(m));
 }
 
-// sums[j] += sum over the band of (A z_j)_c v_c  ( = (A Z)^T v ), scale from the
-// band maximum of |v| (6 faces of at most beta_max each)
+// What the last block of k_defl_azt forms from the sums: c_j = E_jj^-1 (t_j - s_j) with t from
+// ztb (scale ztb_scale), or E_jj^-1 s_j when ztb is null.  The sums and the band
+// maximum are zeroed for the next projection.
+struct DeflCoef {
+  int m;
+  unsigned long long *ztb;
+  double ztb_scale;
+  const double *einv;
+  double *coef;
+  float *coef32;
+  unsigned long long *mx;
+  unsigned *done;
+};
+
+// s_j = sum over the band of (A z_j)_c v_c  ( = (A Z)^T v ), scale from the band
+// maximum of |v| (6 faces of at most beta_max each), then the coefficients
 template <typename T, typename F>
 __global__ void k_defl_azt(const int *__restrict__ band, int nband, const int *__restrict__ comp,
                            const F *__restrict__ bx, const F *__restrict__ by,
                            const F *__restrict__ bz, Dims d, const T *__restrict__ v,
-                           const unsigned long long *__restrict__ mx, double beta_max,
-                           unsigned long long *acc, double *scale_out) {
+                           double beta_max, unsigned long long *acc, DeflCoef dc) {
   griddep_wait();
-  const double vmax = __longlong_as_double((long long)*mx);
+  const double vmax = __longlong_as_double((long long)*dc.mx);
   const double bound = vmax * 6.0 * beta_max * (double)nband;
   const double scale = bound > 0.0 ? ldexp(1.0, 60) / bound : 1.0;
-  if (blockIdx.x == 0 && threadIdx.x == 0) *scale_out = scale;
   const int stride = gridDim.x * blockDim.x;
   FxCarry carry;
   for (int e0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31); e0 < nband; e0 += stride) {
@@ -572,6 +584,14 @@ __global__ void k_defl_azt(const int *__restrict__ band, int nband, const int *_
     fx_add_warp(acc, ks, ws, scale, carry);
   }
   carry.flush(acc, scale);
+  if (!last_block(dc.done)) return;
+  for (int j = threadIdx.x; j < dc.m; j += blockDim.x) {
+    double s = fx_value(acc, j, scale, true);
+    if (dc.ztb) s = fx_value(dc.ztb, j, dc.ztb_scale, false) - s;
+    dc.coef[j] = dc.einv[j] * s;
+    dc.coef32[j] = (float)dc.coef[j];
+  }
+  if (threadIdx.x == 0) *dc.mx = 0ull;
 }
 
 // sums[j] += sum of v over all cells of component j (|sum| bounded by the caller's scale).
@@ -601,23 +621,14 @@ __global__ void k_defl_zt(const int *__restrict__ comp, const T *__restrict__ v,
   carry.flush(acc, scale);
 }
 
-// c_j = E_jj^-1 (s_j - t_j): s from the sum sa (scale *scale_a, or fixed_scale_a
-// when scale_a is null), t from the sum sb (scale *scale_b), either may be
-// absent.  The per-projection sums (sb, or sa when clear_a) and the band
-// maximum mx are zeroed for the next projection.
-__global__ void k_defl_coef(int m, unsigned long long *sa, const double *scale_a,
-                            double fixed_scale_a, int clear_a, unsigned long long *sb,
-                            const double *scale_b, const double *__restrict__ einv,
-                            double *__restrict__ coef, float *__restrict__ coef32,
-                            unsigned long long *mx) {
-  griddep_wait();
+// c_j = E_jj^-1 s_j from the sums sa (kept)
+__global__ void k_defl_coef(int m, unsigned long long *sa, double scale,
+                            const double *__restrict__ einv, double *__restrict__ coef,
+                            float *__restrict__ coef32, unsigned long long *mx) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j == 0) *mx = 0ull;
   if (j >= m) return;
-  double s = 0.0;
-  if (sa) s = fx_value(sa, j, scale_a ? *scale_a : fixed_scale_a, clear_a != 0);
-  if (sb) s -= fx_value(sb, j, *scale_b, true);
-  coef[j] = einv[j] * s;
+  coef[j] = einv[j] * fx_value(sa, j, scale, false);
   coef32[j] = (float)coef[j];
 }
 
@@ -699,7 +710,7 @@ struct IVec16<2> {
 template <typename T>
 __global__ void __launch_bounds__(VEC_THREADS, 4)
 k_dot_zdefl(const T *__restrict__ r, T *__restrict__ z, const int *__restrict__ comp,
-            const T *__restrict__ coef, size_t n, double *__restrict__ partial) {
+            const T *__restrict__ coef, size_t n, Fin fin) {
   griddep_wait();
   using VT = Vec16<T>;
   using V = typename VT::V;
@@ -736,8 +747,7 @@ k_dot_zdefl(const T *__restrict__ r, T *__restrict__ z, const int *__restrict__ 
     if (m >= 0) z[e] -= coef[m];
     acc = fma(r[e], z[e], acc);
   }
-  double t = block_sum((double)acc);
-  if (threadIdx.x == 0) partial[blockIdx.x] = t;
+  block_finish(block_sum((double)acc), blockIdx.x, fin);
 }
 
 // x_c += coef[comp_c] on every cell of a component (the deflation correction)

@@ -990,6 +990,72 @@ enum { S_RZ = 0, S_RZOLD, S_DQ, S_ALPHA, S_BETA, S_RR, S_BB, S_MEAN, S_TMP,
        S_COUNT };
 enum { OP_STORE = 0, OP_ALPHA, OP_BETA, OP_MEAN };
 
+// What the last block of a reducing kernel does with the kernel's partial sums:
+// the final sum in a fixed order, then an operation on the device scalars and,
+// when host is not null, a copy of the scalars to (mapped) host memory.  A final
+// reduction of its own is a launch of ~2.5 us in a chain of launches, and a
+// copy of the scalars another operation on the stream.  done null: partials only.
+struct Fin {
+  double *partial;
+  unsigned *done;  // blocks finished, zero between kernels
+  double *scal, *host;
+  double count;
+  int op, slot;
+};
+__device__ __forceinline__ void scal_op(double *scal, int op, int slot, double count, double s) {
+  switch (op) {
+    case OP_STORE: scal[slot] = s; break;
+    case OP_ALPHA: scal[S_DQ] = s; scal[S_ALPHA] = scal[S_RZ] / s; break;
+    case OP_BETA:
+      scal[S_RZOLD] = scal[S_RZ];
+      scal[S_RZ] = s;
+      scal[S_BETA] = s / scal[S_RZOLD];
+      break;
+    case OP_MEAN: scal[S_MEAN] = s / count; break;
+  }
+}
+// True in the block that finishes last (all threads call it; the memory written
+// by every block before its call is visible to that block after it).
+__device__ __forceinline__ bool last_block(unsigned *done) {
+  __shared__ int last;
+  __threadfence();
+  __syncthreads();
+  const int lin = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
+  const unsigned nb = gridDim.x * gridDim.y * gridDim.z;
+  if (lin == 0) {
+    last = atomicAdd(done, 1u) == nb - 1u;
+    if (last) *done = 0u;
+  }
+  __syncthreads();
+  if (!last) return false;
+  __threadfence();
+  return true;
+}
+// End of a reducing kernel of 256 threads: t is block_sum's result (thread 0), stored as
+// partial number id.  The final sum has k_reduce's order: 1024 interleaved sums,
+// then its tree.
+__device__ __forceinline__ void block_finish(double t, int id, const Fin &f) {
+  const int lin = threadIdx.x + blockDim.x * threadIdx.y;
+  if (lin == 0) f.partial[id] = t;
+  if (!f.done || !last_block(f.done)) return;
+  __shared__ double red[32];
+  const int np = gridDim.x * gridDim.y * gridDim.z;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    double acc = 0.0;
+    for (int e = lin + 256 * q; e < np; e += 1024) acc += __ldcg(f.partial + e);
+    acc = warp_sum(acc);
+    if ((lin & 31) == 0) red[(lin >> 5) + 8 * q] = acc;
+  }
+  __syncthreads();
+  if (lin < 32) {
+    const double s = warp_sum(red[lin]);
+    if (lin == 0) scal_op(f.scal, f.op, f.slot, f.count, s);
+    __syncwarp();
+    if (f.host && lin < S_COUNT) f.host[lin] = *(volatile double *)(f.scal + lin);
+  }
+}
+
 // Stencil kernels with a reduction walk a column of `zper` planes per
 // thread (grid z = ceil(nz / zper)), so the partial-sum count stays ~2k.
 // q = At d; per-block partial of d.q
@@ -997,7 +1063,8 @@ template <typename T>
 __global__ void k_apply_dot(const T *__restrict__ dv, T *__restrict__ q, const T *__restrict__ bx,
                             const T *__restrict__ by, const T *__restrict__ bz,
                             const T *__restrict__ diag, const T *__restrict__ dd, Dims d,
-                            int zper, double *__restrict__ partial) {
+                            int zper, Fin fin) {
+  griddep_wait();
   int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y;
   int k0 = blockIdx.z * zper, k1 = min(d.nz, k0 + zper);
   T acc = 0;
@@ -1008,8 +1075,7 @@ __global__ void k_apply_dot(const T *__restrict__ dv, T *__restrict__ q, const T
       q[c] = s;
       acc = fma(s, dv[c], acc);
     }
-  double t = block_sum((double)acc);
-  if (thread0()) partial[block_linear_id()] = t;
+  block_finish(block_sum((double)acc), block_linear_id(), fin);
 }
 
 // q = At d (FP32 difference form, op_at's arithmetic per cell) and per-block
@@ -1031,7 +1097,7 @@ template <bool XPBY>
 __global__ void __launch_bounds__(BX * BY)
 k_apply_dot4(const float *__restrict__ dv, float *__restrict__ q, const float *__restrict__ bx,
              const float *__restrict__ by, const float *__restrict__ bz,
-             const float *__restrict__ dd32, Dims d, int zper, double *__restrict__ partial,
+             const float *__restrict__ dd32, Dims d, int zper, Fin fin,
              const float *__restrict__ z, float *__restrict__ dnew,
              const double *__restrict__ scal, int first) {
   griddep_wait();
@@ -1080,8 +1146,7 @@ k_apply_dot4(const float *__restrict__ dv, float *__restrict__ q, const float *_
       }
       *reinterpret_cast<float4 *>(q + c0) = out;
     }
-  const double tot = block_sum((double)acc);
-  if (thread0()) partial[block_linear_id()] = tot;
+  block_finish(block_sum((double)acc), block_linear_id(), fin);
 }
 
 // r = b - At x (scaled), per-block partial of r.r; zero != 0: x = 0, r = b.
@@ -1089,7 +1154,7 @@ template <typename T>
 __global__ void k_residual(const T *__restrict__ x, const T *__restrict__ b, T *__restrict__ r,
                            const T *__restrict__ bx, const T *__restrict__ by,
                            const T *__restrict__ bz, const T *__restrict__ diag, Dims d, int zper,
-                           double *__restrict__ partial, int zero) {
+                           Fin fin, int zero) {
   const T *dd = nullptr;  // diag holds the outflow diagonal
   int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y;
   int k0 = blockIdx.z * zper, k1 = min(d.nz, k0 + zper);
@@ -1101,8 +1166,7 @@ __global__ void k_residual(const T *__restrict__ x, const T *__restrict__ b, T *
       r[c] = v;
       acc = fma((double)v, (double)v, acc);
     }
-  double t = block_sum(acc);
-  if (thread0()) partial[block_linear_id()] = t;
+  block_finish(block_sum(acc), block_linear_id(), fin);
 }
 
 // mixed precision outer residual: r64 = b - At64 x64 (FP64), r32 = fl32(r64)
@@ -1110,7 +1174,7 @@ __global__ void k_residual_mixed(const double *__restrict__ x, const double *__r
                                  float *__restrict__ r32, const double *__restrict__ bx,
                                  const double *__restrict__ by, const double *__restrict__ bz,
                                  const double *__restrict__ diag, Dims d, int zper,
-                                 double *__restrict__ partial, int zero) {
+                                 Fin fin, int zero) {
   int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y;
   int k0 = blockIdx.z * zper, k1 = min(d.nz, k0 + zper);
   double acc = 0.0;
@@ -1121,8 +1185,7 @@ __global__ void k_residual_mixed(const double *__restrict__ x, const double *__r
       r32[c] = (float)v;
       acc = fma(v, v, acc);
     }
-  double t = block_sum(acc);
-  if (thread0()) partial[block_linear_id()] = t;
+  block_finish(block_sum(acc), block_linear_id(), fin);
 }
 
 // Grid-stride vector kernels: fixed grid (deterministic partial order).
@@ -1160,7 +1223,8 @@ __device__ __forceinline__ bool aligned16(const void *a, const void *b = nullptr
 
 template <typename T>
 __global__ void __launch_bounds__(VEC_THREADS, 4)
-k_dot(const T *__restrict__ a, const T *__restrict__ b, size_t n, double *__restrict__ partial) {
+k_dot(const T *__restrict__ a, const T *__restrict__ b, size_t n, Fin fin) {
+  griddep_wait();
   using VT = Vec16<T>;
   using V = typename VT::V;
   constexpr int W = VT::W;
@@ -1179,16 +1243,14 @@ k_dot(const T *__restrict__ a, const T *__restrict__ b, size_t n, double *__rest
     done = nv * W;
   }
   for (size_t e = done + tid; e < n; e += stride) acc = fma(a[e], b[e], acc);
-  double t = block_sum((double)acc);
-  if (threadIdx.x == 0) partial[blockIdx.x] = t;
+  block_finish(block_sum((double)acc), blockIdx.x, fin);
 }
 
 // x += alpha d; r -= alpha q; partial r.r
 template <typename T>
 __global__ void __launch_bounds__(VEC_THREADS, 4)
 k_axpy2(T *__restrict__ x, T *__restrict__ r, const T *__restrict__ dv,
-                        const T *__restrict__ q, size_t n, const double *__restrict__ scal,
-                        double *__restrict__ partial) {
+                        const T *__restrict__ q, size_t n, const double *__restrict__ scal, Fin fin) {
   griddep_wait();
   using VT = Vec16<T>;
   using V = typename VT::V;
@@ -1223,8 +1285,7 @@ k_axpy2(T *__restrict__ x, T *__restrict__ r, const T *__restrict__ dv,
     r[e] = rv;
     acc = fma(rv, rv, acc);
   }
-  double t = block_sum((double)acc);
-  if (threadIdx.x == 0) partial[blockIdx.x] = t;
+  block_finish(block_sum((double)acc), blockIdx.x, fin);
 }
 
 // d = z + beta d (first iteration: d = z)
@@ -1232,6 +1293,7 @@ template <typename T>
 __global__ void __launch_bounds__(VEC_THREADS, 4)
 k_xpby(T *__restrict__ dv, const T *__restrict__ z, size_t n,
                        const double *__restrict__ scal, int first) {
+  griddep_wait();
   using VT = Vec16<T>;
   using V = typename VT::V;
   constexpr int W = VT::W;
@@ -1308,7 +1370,7 @@ __global__ void k_lincomb_f32(float *__restrict__ g, double a, const double *__r
 
 // dst32 = fl32(src64), per-block partial of src.src (FP64)
 __global__ void k_to_f32_norm(const double *__restrict__ src, float *__restrict__ dst, size_t n,
-                              double *__restrict__ partial) {
+                              Fin fin) {
   double acc = 0.0;
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n;
        e += (size_t)gridDim.x * blockDim.x) {
@@ -1316,23 +1378,21 @@ __global__ void k_to_f32_norm(const double *__restrict__ src, float *__restrict_
     dst[e] = (float)v;
     acc = fma(v, v, acc);
   }
-  double t = block_sum(acc);
-  if (threadIdx.x == 0) partial[blockIdx.x] = t;
+  block_finish(block_sum(acc), blockIdx.x, fin);
 }
 
 template <typename T>
-__global__ void k_sum(const T *__restrict__ a, size_t n, double *__restrict__ partial) {
+__global__ void k_sum(const T *__restrict__ a, size_t n, Fin fin) {
   double acc = 0.0;
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n;
        e += (size_t)gridDim.x * blockDim.x)
     acc += (double)a[e];
-  double t = block_sum(acc);
-  if (threadIdx.x == 0) partial[blockIdx.x] = t;
+  block_finish(block_sum(acc), blockIdx.x, fin);
 }
 
 // x -= mean (scal[S_MEAN]); optional partial of the new x.x
 __global__ void k_sub_mean(double *__restrict__ x, size_t n, const double *__restrict__ scal,
-                           double *__restrict__ partial) {
+                           Fin fin) {
   double m = scal[S_MEAN];
   double acc = 0.0;
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n;
@@ -1341,8 +1401,7 @@ __global__ void k_sub_mean(double *__restrict__ x, size_t n, const double *__res
     x[e] = v;
     acc = fma(v, v, acc);
   }
-  double t = block_sum(acc);
-  if (partial != nullptr && threadIdx.x == 0) partial[blockIdx.x] = t;
+  if (fin.partial) block_finish(block_sum(acc), blockIdx.x, fin);
 }
 
 // Single-block final reduction of the partials in a fixed order, then an
@@ -1353,25 +1412,13 @@ __global__ void k_reduce(const double *__restrict__ partial, int np, double *__r
   double acc = 0.0;
   for (int e = threadIdx.x; e < np; e += blockDim.x) acc += partial[e];
   double s = block_sum(acc);
-  if (threadIdx.x == 0) {
-    switch (op) {
-      case OP_STORE: scal[slot] = s; break;
-      case OP_ALPHA: scal[S_DQ] = s; scal[S_ALPHA] = scal[S_RZ] / s; break;
-      case OP_BETA:
-        scal[S_RZOLD] = scal[S_RZ];
-        scal[S_RZ] = s;
-        scal[S_BETA] = s / scal[S_RZOLD];
-        break;
-      case OP_MEAN: scal[S_MEAN] = s / count; break;
-    }
-  }
+  if (threadIdx.x == 0) scal_op(scal, op, slot, count, s);
 }
 
 // --------------------------------------------------------- assembly (A3)
 // bt = h^2 rhs + Jt; per-block partial sum (for the mean)
 __global__ void k_assemble(const double *__restrict__ rhs, const double *__restrict__ Jt,
-                           double *__restrict__ b, size_t n, double h2,
-                           double *__restrict__ partial) {
+                           double *__restrict__ b, size_t n, double h2, Fin fin) {
   double acc = 0.0;
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n;
        e += (size_t)gridDim.x * blockDim.x) {
@@ -1379,15 +1426,13 @@ __global__ void k_assemble(const double *__restrict__ rhs, const double *__restr
     b[e] = v;
     acc += v;
   }
-  double t = block_sum(acc);
-  if (threadIdx.x == 0) partial[blockIdx.x] = t;
+  block_finish(block_sum(acc), blockIdx.x, fin);
 }
 
 // bt = h^2 div_h u* + Jt = h * sum(u_high - u_low) + Jt, fused divergence
 __global__ void k_assemble_u(const double *__restrict__ ux, const double *__restrict__ uy,
                              const double *__restrict__ uz, const double *__restrict__ Jt,
-                             double *__restrict__ b, Dims d, int zper, int kb0, double h,
-                             double *__restrict__ partial) {
+                             double *__restrict__ b, Dims d, int zper, int kb0, double h, Fin fin) {
   // kb0: z-block offset of this launch (a slab of the z-blocks); partial is
   // indexed by the global block
   int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y;
@@ -1402,8 +1447,7 @@ __global__ void k_assemble_u(const double *__restrict__ ux, const double *__rest
       b[c] = v;
       acc += v;
     }
-  double t = block_sum(acc);
-  if (thread0()) partial[block_linear_id() + (size_t)kb0 * gridDim.x * gridDim.y] = t;
+  block_finish(block_sum(acc), block_linear_id() + kb0 * (int)(gridDim.x * gridDim.y), fin);
 }
 
 // div_h u = sum over axes of (u_high - u_low) / h

@@ -135,6 +135,7 @@ struct mp_poisson {
   int nc = 0;
   // reductions
   double *partial = nullptr, *scal = nullptr, *scal_h = nullptr;
+  unsigned *done = nullptr;  // blocks finished of the running reduction, and of a projection's sums
   int npart = 0;
   double bnorm = 0.0;
   mp_stats stats{};
@@ -148,7 +149,7 @@ struct mp_poisson {
   double beta_max = 1.0, ztb_scale = 1.0;
   float fs16 = 1.f;  // scale of the FP16 faces (a power of two)
   int diag_mode = 0;  // per-level arrays formed by k_diag for this geometry (bits: 1 FP64, 2 FP32)
-  double *einv = nullptr, *coef = nullptr, *dscale = nullptr;
+  double *einv = nullptr, *coef = nullptr;
   float *coef32 = nullptr;
   unsigned long long *acc_a = nullptr, *acc_b = nullptr, *acc_ztb = nullptr, *dmax = nullptr;
   int *hint = nullptr;  // pinned host copy of dint
@@ -347,16 +348,16 @@ constexpr int kid(int id64, int id32) {
 // the phase-change mass flux the kernels read (null when none is set)
 const double *mdot_of(const mp_poisson *hd) { return hd->has_mdot ? hd->mdot : nullptr; }
 
-mp_status reduce(mp_poisson *hd, int np, int op, int slot, double count = 0.0) {
-  LAUNCH(hd, K_REDUCE, 0, np * 8.0, k_reduce, 1, 1024, hd->partial, np, hd->scal, op, slot, count);
-  return launch_ok();
+// a reducing kernel's finish: the final sum in its last block, then op on slot;
+// to_host: the scalars copied to scal_h, for the read_scalars that follows
+Fin fin(const mp_poisson *hd, int op, int slot, double count, bool to_host) {
+  return Fin{hd->partial, hd->done, hd->scal, to_host ? hd->scal_h : nullptr, count, op, slot};
 }
-// the same for a reduction whose predecessor on the stream is the kernel that
-// wrote the partials: launched with programmatic serialization (k_reduce waits
-// for that kernel before reading)
-mp_status reduce_after(mp_poisson *hd, int np, int op, int slot) {
-  LAUNCH_PDL(hd, K_REDUCE, 0, np * 8.0, k_reduce, 1, 1024, 0, (const double *)hd->partial, np,
-             hd->scal, op, slot, 0.0);
+// partial sums only
+Fin partials(const mp_poisson *hd) { return Fin{hd->partial, nullptr, nullptr, nullptr, 0.0, 0, 0}; }
+// the final reduction of partials that several launches left
+mp_status reduce(mp_poisson *hd, int np, int op, int slot, double count) {
+  LAUNCH(hd, K_REDUCE, 0, np * 8.0, k_reduce, 1, 1024, hd->partial, np, hd->scal, op, slot, count);
   return launch_ok();
 }
 
@@ -370,14 +371,15 @@ mp_status clear_visits(mp_poisson *hd) {
   return MP_OK;
 }
 
+// Wait for the scalars: the last reducing kernel before the call copied them to
+// scal_h (mapped host memory) itself.
 mp_status read_scalars(mp_poisson *hd) {
-  CK(cudaMemcpyAsync(hd->scal_h, hd->scal, S_COUNT * sizeof(double), cudaMemcpyDeviceToHost,
-                     hd->st));
   CK(cudaStreamSynchronize(hd->st));
   prof_resolve(hd);
   if (hd->scal_h[S_ERR] != 0.0) {  // a bounded device wait gave up: start over clean
     CKS(clear_visits(hd));
     CK(cudaMemsetAsync(hd->scal + S_ERR, 0, sizeof(double), hd->st));
+    hd->scal_h[S_ERR] = 0.0;
     return MP_ERR_TIMEOUT;
   }
   return MP_OK;
@@ -777,21 +779,13 @@ mp_status defl_coef(mp_poisson *hd, const T *v, const F *bx, const F *by, const 
   unsigned long long *acc = with_ztb ? hd->acc_b : hd->acc_a;
   LAUNCH(hd, K_DEFL, 0, nb * (double)sizeof(T), k_defl_maxabs<T>, VEC_BLOCKS, VEC_THREADS,
          hd->band, nb, v, hd->dmax);
-  // k_defl_azt and k_defl_coef follow the kernel launched just before them:
-  // programmatic serialization (both wait for their predecessor first)
+  // follows the kernel launched just before: programmatic serialization
+  const DeflCoef dc{m, with_ztb ? hd->acc_ztb : nullptr, hd->ztb_scale, hd->einv,
+                    hd->coef, hd->coef32, hd->dmax, hd->done + 1};
   auto kazt = k_defl_azt<T, F>;
-  LAUNCH_PDL(hd, K_DEFL, 0, nb * (7.0 * sizeof(T) + 3.0 * sizeof(F) + 28.0), kazt, VEC_BLOCKS,
-             VEC_THREADS, 0, hd->band, nb, hd->comp, bx, by, bz, l0.d, v,
-             (const unsigned long long *)hd->dmax, hd->beta_max, acc, hd->dscale);
-  if (with_ztb)
-    LAUNCH_PDL(hd, K_DEFL, 0, m * 16.0, k_defl_coef, (m + 255) / 256, 256, 0, m, hd->acc_ztb,
-               (const double *)nullptr, hd->ztb_scale, 0, acc, (const double *)hd->dscale,
-               (const double *)hd->einv, hd->coef, hd->coef32, hd->dmax);
-  else
-    LAUNCH_PDL(hd, K_DEFL, 0, m * 16.0, k_defl_coef, (m + 255) / 256, 256, 0, m, acc,
-               (const double *)hd->dscale, 0.0, 1, (unsigned long long *)nullptr,
-               (const double *)nullptr, (const double *)hd->einv, hd->coef, hd->coef32,
-               hd->dmax);
+  LAUNCH_PDL(hd, K_DEFL, 0, nb * (7.0 * sizeof(T) + 3.0 * sizeof(F) + 28.0) + m * 16.0, kazt,
+             VEC_BLOCKS, VEC_THREADS, 0, hd->band, nb, hd->comp, bx, by, bz, l0.d, v, hd->beta_max,
+             acc, dc);
   return launch_ok();
 }
 
@@ -823,24 +817,21 @@ mp_status defl_guess_residuals(mp_poisson *hd, const double *p, double *rguess, 
   const size_t n = hd->n;
   CKS(defl_ztb(hd));
   LAUNCH(hd, K_RESID64, 0, n * 56.0, k_residual<double>, zgrid(l0.d), kBlock, p, hd->b, hd->z,
-         l0.bx, l0.by, l0.bz, l0.diag, l0.d, zper_of(l0.d), hd->partial, 0);
+         l0.bx, l0.by, l0.bz, l0.diag, l0.d, zper_of(l0.d), partials(hd), 0);
   CKS((defl_coef<double, double>(hd, p, l0.bx, l0.by, l0.bz, true)));
   CKS((defl_sub<double, double>(hd, hd->z, l0.bx, l0.by, l0.bz)));
   LAUNCH(hd, K_DOT64, 0, n * 16.0, k_dot<double>, VEC_BLOCKS, VEC_THREADS, hd->z, hd->z, n,
-         hd->partial);
-  CKS(reduce(hd, VEC_BLOCKS, OP_STORE, S_TMP));
+         fin(hd, OP_STORE, S_TMP, 0.0, true));
   CKS(read_scalars(hd));
   *rguess = std::sqrt(hd->scal_h[S_TMP]);
   // zero guess: coef = E^-1 Z^T bt, P bt = bt - At Z coef
   const int m = hd->defl_m;
   LAUNCH(hd, K_DEFL, 0, m * 16.0, k_defl_coef, (m + 255) / 256, 256, m, hd->acc_ztb,
-         (const double *)nullptr, hd->ztb_scale, 0, (unsigned long long *)nullptr,
-         (const double *)nullptr, hd->einv, hd->coef, hd->coef32, hd->dmax);
+         hd->ztb_scale, hd->einv, hd->coef, hd->coef32, hd->dmax);
   CK(cudaMemcpyAsync(hd->z, hd->b, n * sizeof(double), cudaMemcpyDeviceToDevice, hd->st));
   CKS((defl_sub<double, double>(hd, hd->z, l0.bx, l0.by, l0.bz)));
   LAUNCH(hd, K_DOT64, 0, n * 16.0, k_dot<double>, VEC_BLOCKS, VEC_THREADS, hd->z, hd->z, n,
-         hd->partial);
-  CKS(reduce(hd, VEC_BLOCKS, OP_STORE, S_TMP));
+         fin(hd, OP_STORE, S_TMP, 0.0, true));
   CKS(read_scalars(hd));
   *rzero = std::sqrt(hd->scal_h[S_TMP]);
   return MP_OK;
@@ -850,7 +841,7 @@ mp_status defl_guess_residuals(mp_poisson *hd, const double *p, double *rguess, 
 // sums of r . z (the A-DEF2 form of deflated PCG: every search direction is
 // A-orthogonal to the components, so the iteration needs no projection of A d)
 template <typename T, typename F>
-mp_status defl_rz(mp_poisson *hd, const T *r, T *z, const F *bx, const F *by, const F *bz) {
+mp_status defl_rz(mp_poisson *hd, const T *r, T *z, const F *bx, const F *by, const F *bz, int op) {
   CKS((defl_coef<T, F>(hd, z, bx, by, bz, false)));
   const T *coef;
   if constexpr (sizeof(T) == 8)
@@ -858,7 +849,7 @@ mp_status defl_rz(mp_poisson *hd, const T *r, T *z, const F *bx, const F *by, co
   else
     coef = hd->coef32;
   LAUNCH_PDL(hd, K_DEFL_DOT, 0, hd->n * (3.0 * sizeof(T) + 4.0), k_dot_zdefl<T>, VEC_BLOCKS,
-             VEC_THREADS, 0, r, z, (const int *)hd->comp, coef, hd->n, hd->partial);
+             VEC_THREADS, 0, r, z, (const int *)hd->comp, coef, hd->n, fin(hd, op, S_RZ, 0.0, false));
   return launch_ok();
 }
 
@@ -881,8 +872,7 @@ mp_status pcg(mp_poisson *hd, T *x, T *r, T *z, T *dv, T *q, double tol_abs, int
     CKS((defl_coef<T, T>(hd, x, bx, by, bz, true)));
     CKS((defl_sub<T, T>(hd, r, bx, by, bz)));
     LAUNCH(hd, kid<T>(K_DOT64, K_DOT32), 0, 2.0 * nsz, k_dot<T>, VEC_BLOCKS, VEC_THREADS, r, r, n,
-           hd->partial);
-    CKS(reduce(hd, VEC_BLOCKS, OP_STORE, S_RR));
+           fin(hd, OP_STORE, S_RR, 0.0, true));
   }
   int it = 0;
   mp_status st = MP_OK;
@@ -897,21 +887,21 @@ mp_status pcg(mp_poisson *hd, T *x, T *r, T *z, T *dv, T *q, double tol_abs, int
     }
     CKS(run_vcycle<T>(hd, r, z));
     if (defl)
-      CKS((defl_rz<T, T>(hd, r, z, bx, by, bz)));
+      CKS((defl_rz<T, T>(hd, r, z, bx, by, bz, it == 0 ? OP_STORE : OP_BETA)));
     else
       LAUNCH(hd, kid<T>(K_DOT64, K_DOT32), 0, 2.0 * nsz, k_dot<T>, VEC_BLOCKS, VEC_THREADS, r, z,
-             n, hd->partial);
-    CKS(reduce(hd, VEC_BLOCKS, it == 0 ? OP_STORE : OP_BETA, S_RZ));
-    LAUNCH(hd, kid<T>(K_XPBY64, K_XPBY32), 0, (it == 0 ? 2.0 : 3.0) * nsz, k_xpby<T>, VEC_BLOCKS,
-           VEC_THREADS, dv, z, n, hd->scal, it == 0);
-    LAUNCH(hd, kid<T>(K_APPLY64, K_APPLY32), 0, (sizeof(T) == 8 ? 6.0 : 5.0) * nsz,
-           k_apply_dot<T>, zgrid(l0.d), kBlock, dv, q, bx, by, bz, diag, (const T *)nullptr, l0.d,
-           zper_of(l0.d),
-           hd->partial);
-    CKS(reduce(hd, zblocks(l0.d), OP_ALPHA, 0));
-    LAUNCH(hd, kid<T>(K_AXPY64, K_AXPY32), 0, 6.0 * nsz, k_axpy2<T>, VEC_BLOCKS, VEC_THREADS, x,
-           r, dv, q, n, hd->scal, hd->partial);
-    CKS(reduce(hd, VEC_BLOCKS, OP_STORE, S_RR));
+             n, fin(hd, it == 0 ? OP_STORE : OP_BETA, S_RZ, 0.0, false));
+    // each of these follows a kernel: programmatic serialization
+    LAUNCH_PDL(hd, kid<T>(K_XPBY64, K_XPBY32), 0, (it == 0 ? 2.0 : 3.0) * nsz, k_xpby<T>,
+               VEC_BLOCKS, VEC_THREADS, 0, dv, (const T *)z, n, (const double *)hd->scal,
+               it == 0 ? 1 : 0);
+    LAUNCH_PDL(hd, kid<T>(K_APPLY64, K_APPLY32), 0, (sizeof(T) == 8 ? 6.0 : 5.0) * nsz,
+               k_apply_dot<T>, zgrid(l0.d), kBlock, 0, (const T *)dv, q, (const T *)bx,
+               (const T *)by, (const T *)bz, (const T *)diag, (const T *)nullptr, l0.d,
+               zper_of(l0.d), fin(hd, OP_ALPHA, 0, 0.0, false));
+    LAUNCH_PDL(hd, kid<T>(K_AXPY64, K_AXPY32), 0, 6.0 * nsz, k_axpy2<T>, VEC_BLOCKS, VEC_THREADS,
+               0, x, r, (const T *)dv, (const T *)q, n, (const double *)hd->scal,
+               fin(hd, OP_STORE, S_RR, 0.0, true));
     ++it;
     CKS(read_scalars(hd));
     rn = std::sqrt(hd->scal_h[S_RR]);
@@ -934,19 +924,17 @@ mp_status defl_true_residual32(mp_poisson *hd, const double *p, int p_is_zero, d
   const int m = hd->defl_m, nb = hd->defl_nband;
   if (p_is_zero)  // coef = E^-1 Z^T bt
     LAUNCH(hd, K_DEFL, 0, m * 16.0, k_defl_coef, (m + 255) / 256, 256, m, hd->acc_ztb,
-           (const double *)nullptr, hd->ztb_scale, 0, (unsigned long long *)nullptr,
-           (const double *)nullptr, hd->einv, hd->coef, hd->coef32, hd->dmax);
+           hd->ztb_scale, hd->einv, hd->coef, hd->coef32, hd->dmax);
   else
     CKS((defl_coef<double, double>(hd, p, l0.bx, l0.by, l0.bz, true)));
   LAUNCH(hd, K_RESIDMIX, 0, n * (p_is_zero ? 12.0 : 52.0), k_residual_mixed, zgrid(l0.d), kBlock,
-         p, hd->b, hd->r32, l0.bx, l0.by, l0.bz, l0.diag, l0.d, zper_of(l0.d), hd->partial,
+         p, hd->b, hd->r32, l0.bx, l0.by, l0.bz, l0.diag, l0.d, zper_of(l0.d), partials(hd),
          p_is_zero);
   LAUNCH(hd, K_DEFL, 0, nb * 120.0, k_defl_resid_band, VEC_BLOCKS, VEC_THREADS, hd->band, nb,
          hd->comp, l0.bx, l0.by, l0.bz, l0.diag, l0.d, hd->coef,
          p_is_zero ? (const double *)nullptr : p, hd->b, hd->r32);
   LAUNCH(hd, K_DOT32, 0, 4.0 * n, k_dot<float>, VEC_BLOCKS, VEC_THREADS, hd->r32, hd->r32, n,
-         hd->partial);
-  CKS(reduce(hd, VEC_BLOCKS, OP_STORE, S_RR));
+         fin(hd, OP_STORE, S_RR, 0.0, true));
   CKS(read_scalars(hd));
   *rnorm = std::sqrt(hd->scal_h[S_RR]);
   return MP_OK;
@@ -995,8 +983,7 @@ mp_status pcg_mixed(mp_poisson *hd, double *p, double rn, double tol_abs, int ma
         CKS(project_true(rn, 0));
       } else {
         LAUNCH(hd, K_RESIDMIX, 0, n * 52.0, k_residual_mixed, zgrid(l0.d), kBlock, p, hd->b, r,
-               l0.bx, l0.by, l0.bz, l0.diag, l0.d, zper_of(l0.d), hd->partial, 0);
-        CKS(reduce(hd, zblocks(l0.d), OP_STORE, S_RR));
+               l0.bx, l0.by, l0.bz, l0.diag, l0.d, zper_of(l0.d), fin(hd, OP_STORE, S_RR, 0.0, true), 0);
         CKS(read_scalars(hd));
         rn = std::sqrt(hd->scal_h[S_RR]);
       }
@@ -1010,13 +997,13 @@ mp_status pcg_mixed(mp_poisson *hd, double *p, double rn, double tol_abs, int ma
     if (it >= maxit) { st = MP_ERR_NOT_CONVERGED; break; }
     CKS(run_vcycle<float>(hd, r, z));
     if (defl)
-      CKS((defl_rz<float, float>(hd, r, z, l0.bx32, l0.by32, l0.bz32)));
+      CKS((defl_rz<float, float>(hd, r, z, l0.bx32, l0.by32, l0.bz32,
+                                 it == 0 ? OP_STORE : OP_BETA)));
     else
       LAUNCH(hd, K_DOT32, 0, 2.0 * nsz, k_dot<float>, VEC_BLOCKS, VEC_THREADS, r, z, n,
-             hd->partial);
+             fin(hd, it == 0 ? OP_STORE : OP_BETA, S_RZ, 0.0, false));
     // from here to the end of the iteration every launch follows a kernel:
     // programmatic serialization, each kernel waiting for its predecessor
-    CKS(reduce_after(hd, VEC_BLOCKS, it == 0 ? OP_STORE : OP_BETA, S_RZ));
     const bool fused = l0.d.nx % 4 == 0;  // 16-byte rows
     if (fused) {
       // d_new = z + beta d in the operator's loads, stored to the other buffer
@@ -1025,21 +1012,18 @@ mp_status pcg_mixed(mp_poisson *hd, double *p, double rn, double tol_abs, int ma
       LAUNCH_PDL(hd, K_APPLY32, 0, (it == 0 ? 6.0 : 7.0) * nsz, k_apply_dot4<true>, zgrid(dq),
                  kBlock, 0, (const float *)dv, q, (const float *)l0.bx32,
                  (const float *)l0.by32, (const float *)l0.bz32, (const float *)l0.dd32, l0.d,
-                 zper_of(dq), hd->partial, (const float *)z, dnew, (const double *)hd->scal,
+                 zper_of(dq), fin(hd, OP_ALPHA, 0, 0.0, false), (const float *)z, dnew, (const double *)hd->scal,
                  it == 0 ? 1 : 0);
-      CKS(reduce_after(hd, zblocks(dq), OP_ALPHA, 0));
       dv = dnew;
     } else {
       LAUNCH(hd, K_XPBY32, 0, (it == 0 ? 2.0 : 3.0) * nsz, k_xpby<float>, VEC_BLOCKS, VEC_THREADS,
              dv, z, n, hd->scal, it == 0);
       LAUNCH(hd, K_APPLY32, 0, 5.0 * nsz, k_apply_dot<float>, zgrid(l0.d), kBlock, dv, q,
              l0.bx32, l0.by32, l0.bz32, (float *)nullptr, (const float *)l0.dd32, l0.d,
-             zper_of(l0.d), hd->partial);
-      CKS(reduce(hd, zblocks(l0.d), OP_ALPHA, 0));
+             zper_of(l0.d), fin(hd, OP_ALPHA, 0, 0.0, false));
     }
     LAUNCH_PDL(hd, K_AXPY32, 0, 6.0 * nsz, k_axpy2<float>, VEC_BLOCKS, VEC_THREADS, 0, e, r,
-               (const float *)dv, (const float *)q, n, (const double *)hd->scal, hd->partial);
-    CKS(reduce_after(hd, VEC_BLOCKS, OP_STORE, S_RR));
+               (const float *)dv, (const float *)q, n, (const double *)hd->scal, fin(hd, OP_STORE, S_RR, 0.0, true));
     ++it;
     ++since;
     CKS(read_scalars(hd));
@@ -1072,8 +1056,7 @@ mp_status stationary(mp_poisson *hd, T *x, const T *bt, T *r, T *z, double tol_a
     LAUNCH(hd, kid<T>(K_ADD64, K_ADD32), 0, 3.0 * nsz, k_add<T>, VEC_BLOCKS, VEC_THREADS, x, z,
            hd->n);
     LAUNCH(hd, kid<T>(K_RESID64, K_RESID32), 0, 7.0 * nsz, k_residual<T>, zgrid(l0.d), kBlock,
-           x, bt, r, bx, by, bz, diag, l0.d, zper_of(l0.d), hd->partial, 0);
-    CKS(reduce(hd, zblocks(l0.d), OP_STORE, S_RR));
+           x, bt, r, bx, by, bz, diag, l0.d, zper_of(l0.d), fin(hd, OP_STORE, S_RR, 0.0, true), 0);
     ++it;
     CKS(read_scalars(hd));
     rn = std::sqrt(hd->scal_h[S_RR]);
@@ -1085,44 +1068,40 @@ mp_status stationary(mp_poisson *hd, T *x, const T *bt, T *r, T *z, double tol_a
 
 // mean removal of a device FP64 vector (gauge)
 mp_status remove_mean(mp_poisson *hd, double *x) {
-  LAUNCH(hd, K_SUM, 0, hd->n * 8.0, k_sum<double>, VEC_BLOCKS, VEC_THREADS, x, hd->n, hd->partial);
-  CKS(reduce(hd, VEC_BLOCKS, OP_MEAN, 0, (double)hd->n));
+  LAUNCH(hd, K_SUM, 0, hd->n * 8.0, k_sum<double>, VEC_BLOCKS, VEC_THREADS, x, hd->n, fin(hd, OP_MEAN, 0, (double)hd->n, false));
   LAUNCH(hd, K_SUBMEAN, 0, hd->n * 16.0, k_sub_mean, VEC_BLOCKS, VEC_THREADS, x, hd->n, hd->scal,
-         nullptr);
+         Fin{});
   return launch_ok();
 }
 
-// bt (already holding h^2 rhs + Jt with block sums in partial, np blocks)
-// -> subtract mean, store ||bt||^2 in S_BB
+// bt (already holding h^2 rhs + Jt, its mean in S_MEAN) -> subtract the mean,
+// store ||bt||^2 in S_BB
 // With an outflow side the operator is nonsingular: b keeps its mean and only
 // ||bt||^2 is formed.
-mp_status finish_rhs(mp_poisson *hd, int np) {
+mp_status finish_rhs(mp_poisson *hd) {
   if (hd->outflow) {
     LAUNCH(hd, K_DOT64, 0, hd->n * 8.0, k_dot<double>, VEC_BLOCKS, VEC_THREADS, hd->b, hd->b,
-           hd->n, hd->partial);
-    CKS(reduce(hd, VEC_BLOCKS, OP_STORE, S_BB));
+           hd->n, fin(hd, OP_STORE, S_BB, 0.0, true));
     return launch_ok();
   }
-  CKS(reduce(hd, np, OP_MEAN, 0, (double)hd->n));
   LAUNCH(hd, K_SUBMEAN, 0, hd->n * 16.0, k_sub_mean, VEC_BLOCKS, VEC_THREADS, hd->b, hd->n,
-         hd->scal, hd->partial);
-  CKS(reduce(hd, VEC_BLOCKS, OP_STORE, S_BB));
+         hd->scal, fin(hd, OP_STORE, S_BB, 0.0, true));
   return launch_ok();
 }
 
 mp_status assemble_rhs(mp_poisson *hd, const double *rhs) {
   LAUNCH(hd, K_ASSEMBLE, 0, hd->n * 24.0, k_assemble, VEC_BLOCKS, VEC_THREADS, rhs, hd->Jt, hd->b,
-         hd->n, hd->h * hd->h, hd->partial);
+         hd->n, hd->h * hd->h, fin(hd, OP_MEAN, 0, (double)hd->n, false));
   CKS(launch_ok());
-  return finish_rhs(hd, VEC_BLOCKS);
+  return finish_rhs(hd);
 }
 
 mp_status assemble_rhs_u(mp_poisson *hd, const double *ux, const double *uy, const double *uz) {
   Level &l0 = hd->L[0];
   LAUNCH(hd, K_ASSEMBLE_U, 0, hd->n * 40.0, k_assemble_u, zgrid(l0.d), kBlock, ux, uy, uz,
-         hd->Jt, hd->b, l0.d, zper_of(l0.d), 0, hd->h, hd->partial);
+         hd->Jt, hd->b, l0.d, zper_of(l0.d), 0, hd->h, fin(hd, OP_MEAN, 0, (double)hd->n, false));
   CKS(launch_ok());
-  return finish_rhs(hd, zblocks(l0.d));
+  return finish_rhs(hd);
 }
 
 // z-slabs of the host-buffer step: groups of whole z-blocks of zgrid(l0)
@@ -1188,22 +1167,19 @@ mp_status solve_assembled(mp_poisson *hd, double *p, double tol, std::vector<dou
       // q . At q from the FP32 operator on fl32(q): alpha is a scale factor,
       // and 1e-7 relative is ample (an FP64 operator pass is FP64-rate bound)
       LAUNCH(hd, K_RESIDMIX, 0, hd->n * 12.0, k_to_f32_norm, VEC_BLOCKS, VEC_THREADS, p, hd->z32,
-             hd->n, hd->partial);
+             hd->n, partials(hd));
       const Dims dq = chunk_dims(l0.d);
       LAUNCH(hd, K_APPLY32, 0, hd->n * 20.0, k_apply_dot4<false>, zgrid(dq), kBlock,
              (const float *)hd->z32, hd->q32, l0.bx32, l0.by32, l0.bz32, (const float *)l0.dd32,
-             l0.d, zper_of(dq), hd->partial, (const float *)nullptr, (float *)nullptr,
+             l0.d, zper_of(dq), fin(hd, OP_STORE, S_TMP, 0.0, false), (const float *)nullptr, (float *)nullptr,
              (const double *)nullptr, 0);
-      CKS(reduce(hd, zblocks(dq), OP_STORE, S_TMP));
     } else {
       LAUNCH(hd, K_APPLY64, 0, hd->n * 48.0, k_apply_dot<double>, zgrid(l0.d), kBlock, p, hd->q,
              l0.bx, l0.by, l0.bz, l0.diag, (const double *)nullptr, l0.d, zper_of(l0.d),
-             hd->partial);
-      CKS(reduce(hd, zblocks(l0.d), OP_STORE, S_TMP));
+             fin(hd, OP_STORE, S_TMP, 0.0, false));
     }
     LAUNCH(hd, K_DOT64, 0, hd->n * 16.0, k_dot<double>, VEC_BLOCKS, VEC_THREADS, p, hd->b, hd->n,
-           hd->partial);
-    CKS(reduce(hd, VEC_BLOCKS, OP_STORE, S_RZ));
+           fin(hd, OP_STORE, S_RZ, 0.0, true));
     CKS(read_scalars(hd));
     double alpha = hd->scal_h[S_RZ] / hd->scal_h[S_TMP];
     if (!std::isfinite(alpha)) alpha = 0.0;
@@ -1220,11 +1196,10 @@ mp_status solve_assembled(mp_poisson *hd, double *p, double tol, std::vector<dou
     } else {
       if (o.precision == 0)
         LAUNCH(hd, K_RESID64, 0, hd->n * 56.0, k_residual<double>, zgrid(l0.d), kBlock, p, hd->b,
-               hd->r, l0.bx, l0.by, l0.bz, l0.diag, l0.d, zper_of(l0.d), hd->partial, 0);
+               hd->r, l0.bx, l0.by, l0.bz, l0.diag, l0.d, zper_of(l0.d), fin(hd, OP_STORE, S_RR, 0.0, true), 0);
       else
         LAUNCH(hd, K_RESIDMIX, 0, hd->n * 52.0, k_residual_mixed, zgrid(l0.d), kBlock, p,
-               hd->b, hd->r32, l0.bx, l0.by, l0.bz, l0.diag, l0.d, zper_of(l0.d), hd->partial, 0);
-      CKS(reduce(hd, zblocks(l0.d), OP_STORE, S_RR));
+               hd->b, hd->r32, l0.bx, l0.by, l0.bz, l0.diag, l0.d, zper_of(l0.d), fin(hd, OP_STORE, S_RR, 0.0, true), 0);
       CKS(read_scalars(hd));
       rnet = std::sqrt(hd->scal_h[S_RR]);
       if (defl_active(hd) && o.net_check == 0 && std::isfinite(rnet))
@@ -1249,8 +1224,7 @@ mp_status solve_assembled(mp_poisson *hd, double *p, double tol, std::vector<dou
     if (!have_r) {
       LAUNCH(hd, K_RESID64, 0, hd->n * (zero ? 16.0 : 56.0), k_residual<double>, zgrid(l0.d),
              kBlock, p, hd->b, hd->r, l0.bx, l0.by, l0.bz, l0.diag, l0.d, zper_of(l0.d),
-             hd->partial, zero);
-      CKS(reduce(hd, zblocks(l0.d), OP_STORE, S_RR));
+             fin(hd, OP_STORE, S_RR, 0.0, true), zero);
     }
     CKS(read_scalars(hd));
     hd->stats.r0 = std::sqrt(hd->scal_h[S_RR]) * inv_b;
@@ -1268,8 +1242,7 @@ mp_status solve_assembled(mp_poisson *hd, double *p, double tol, std::vector<dou
     if (!have_r && !r_projected) {
       LAUNCH(hd, K_RESIDMIX, 0, hd->n * (zero ? 12.0 : 52.0), k_residual_mixed, zgrid(l0.d),
              kBlock, p, hd->b, hd->r32, l0.bx, l0.by, l0.bz, l0.diag, l0.d, zper_of(l0.d),
-             hd->partial, zero);
-      CKS(reduce(hd, zblocks(l0.d), OP_STORE, S_RR));
+             fin(hd, OP_STORE, S_RR, 0.0, true), zero);
     }
     CKS(read_scalars(hd));
     double rn = std::sqrt(hd->scal_h[S_RR]);
@@ -1297,8 +1270,7 @@ mp_status solve_assembled(mp_poisson *hd, double *p, double tol, std::vector<dou
       LAUNCH(hd, K_ADDF32, 0, hd->n * 24.0, k_add_f32, VEC_BLOCKS, VEC_THREADS, p, hd->e32,
              hd->n);
       LAUNCH(hd, K_RESIDMIX, 0, hd->n * 52.0, k_residual_mixed, zgrid(l0.d), kBlock, p, hd->b,
-             hd->r32, l0.bx, l0.by, l0.bz, l0.diag, l0.d, zper_of(l0.d), hd->partial, 0);
-      CKS(reduce(hd, zblocks(l0.d), OP_STORE, S_RR));
+             hd->r32, l0.bx, l0.by, l0.bz, l0.diag, l0.d, zper_of(l0.d), fin(hd, OP_STORE, S_RR, 0.0, true), 0);
       CKS(read_scalars(hd));
       rn = std::sqrt(hd->scal_h[S_RR]);
       if (hist) hist->push_back(rn * inv_b);
@@ -1310,8 +1282,7 @@ mp_status solve_assembled(mp_poisson *hd, double *p, double tol, std::vector<dou
     if (!hd->outflow) CKS(remove_mean(hd, p));  // gauge of the singular problem
     // final true FP64 residual of the returned p
     LAUNCH(hd, K_RESID64, 0, hd->n * 56.0, k_residual<double>, zgrid(l0.d), kBlock, p, hd->b,
-           hd->r, l0.bx, l0.by, l0.bz, l0.diag, l0.d, zper_of(l0.d), hd->partial, 0);
-    CKS(reduce(hd, zblocks(l0.d), OP_STORE, S_RR));
+           hd->r, l0.bx, l0.by, l0.bz, l0.diag, l0.d, zper_of(l0.d), fin(hd, OP_STORE, S_RR, 0.0, true), 0);
     CKS(read_scalars(hd));
     hd->stats.relres = std::sqrt(hd->scal_h[S_RR]) * inv_b;
   }
@@ -1708,12 +1679,14 @@ mp_status create(mp_poisson *hd, mp_grid g, double h, const mp_bc bc[3]) {
   CKS(dalloc(hd, &hd->Minv, (size_t)hd->nc * hd->nc));
   hd->npart = std::max(std::max(cell_blocks(hd->L[0].d), zblocks(hd->L[0].d)), VEC_BLOCKS);
   CKS(dalloc(hd, &hd->partial, (size_t)hd->npart));
+  CKS(dalloc(hd, &hd->done, (size_t)2));
   CKS(dalloc(hd, &hd->scal, (size_t)S_COUNT));
   if (cudaMallocHost((void **)&hd->scal_h, S_COUNT * sizeof(double)) != cudaSuccess) {
     cudaGetLastError();
     hd->scal_h = nullptr;
     return MP_ERR_OOM;
   }
+  std::memset(hd->scal_h, 0, S_COUNT * sizeof(double));
   CK(cudaMemsetAsync(hd->scal, 0, S_COUNT * sizeof(double), hd->st));
   // deflation workspace
   const size_t nblk = (n + BAND_CELLS - 1) / BAND_CELLS;
@@ -1729,7 +1702,6 @@ mp_status create(mp_poisson *hd, mp_grid g, double h, const mp_bc bc[3]) {
   CKS(dalloc(hd, &hd->einv, (size_t)DEFL_MAX));
   CKS(dalloc(hd, &hd->coef, (size_t)DEFL_MAX));
   CKS(dalloc(hd, &hd->coef32, (size_t)DEFL_MAX));
-  CKS(dalloc(hd, &hd->dscale, 4));
   CKS(dalloc(hd, &hd->acc_a, (size_t)DEFL_MAX * DEFL_REP * 2));
   CKS(dalloc(hd, &hd->acc_b, (size_t)DEFL_MAX * DEFL_REP * 2));
   CKS(dalloc(hd, &hd->acc_ztb, (size_t)DEFL_MAX * DEFL_REP * 2));
@@ -1782,7 +1754,7 @@ mp_status create(mp_poisson *hd, mp_grid g, double h, const mp_bc bc[3]) {
 mp_status deflated_apply(mp_poisson *hd, double *v, double *out) {
   Level &l0 = hd->L[0];
   LAUNCH(hd, K_APPLY64, 0, hd->n * 48.0, k_apply_dot<double>, zgrid(l0.d), kBlock, v, out, l0.bx,
-         l0.by, l0.bz, l0.diag, (const double *)nullptr, l0.d, zper_of(l0.d), hd->partial);
+         l0.by, l0.bz, l0.diag, (const double *)nullptr, l0.d, zper_of(l0.d), partials(hd));
   CKS(launch_ok());
   CKS((defl_coef<double, double>(hd, v, l0.bx, l0.by, l0.bz, false)));
   return defl_sub<double, double>(hd, out, l0.bx, l0.by, l0.bz);
@@ -1790,8 +1762,7 @@ mp_status deflated_apply(mp_poisson *hd, double *v, double *out) {
 
 mp_status dot64(mp_poisson *hd, const double *a, const double *b, double *out) {
   LAUNCH(hd, K_DOT64, 0, hd->n * 16.0, k_dot<double>, VEC_BLOCKS, VEC_THREADS, a, b, hd->n,
-         hd->partial);
-  CKS(reduce(hd, VEC_BLOCKS, OP_STORE, S_TMP));
+         fin(hd, OP_STORE, S_TMP, 0.0, true));
   CKS(read_scalars(hd));
   *out = hd->scal_h[S_TMP];
   return MP_OK;
@@ -2005,11 +1976,12 @@ mp_status project_step_host(mp_poisson *hd, double *ux_h, double *uy_h, double *
     planes(s, k0, cnt);
     LAUNCH(hd, K_ASSEMBLE_U, 0, cnt * plane * 40.0, k_assemble_u, dim3(g.x, g.y, nb), kBlock,
            (const double *)hd->ux, (const double *)hd->uy, (const double *)hd->uz,
-           (const double *)hd->Jt, hd->b, d, q.zper, kb0, hd->h, hd->partial);
+           (const double *)hd->Jt, hd->b, d, q.zper, kb0, hd->h, partials(hd));
   }
   CKS(launch_ok());
   if (hd->opts.initial_guess == 1) CK(cudaStreamWaitEvent(hd->st, solved, 0));
-  CKS(finish_rhs(hd, zblocks(d)));
+  if (!hd->outflow) CKS(reduce(hd, zblocks(d), OP_MEAN, 0, (double)hd->n));
+  CKS(finish_rhs(hd));
   mp_status s = solve_assembled(hd, hd->pst, tol, nullptr);
   if (iterations) *iterations = hd->stats.iterations;
   if (s != MP_OK) return s;
@@ -2053,7 +2025,7 @@ mp_status mp_poisson_apply(mp_handle hd, const double *x, double *y) {
   if (!hd || !x || !y) return MP_ERR_INVALID_ARG;
   Level &l0 = hd->L[0];
   LAUNCH(hd, K_APPLY64, 0, hd->n * 48.0, k_apply_dot<double>, zgrid(l0.d), kBlock, x, y,
-         l0.bx, l0.by, l0.bz, l0.diag, (const double *)nullptr, l0.d, zper_of(l0.d), hd->partial);
+         l0.bx, l0.by, l0.bz, l0.diag, (const double *)nullptr, l0.d, zper_of(l0.d), partials(hd));
   LAUNCH(hd, K_SCALE, 0, hd->n * 16.0, k_scale, VEC_BLOCKS, VEC_THREADS, y, y, hd->n,
          1.0 / (hd->h * hd->h));
   CKS(launch_ok());
