@@ -385,9 +385,9 @@ k_ctail(const __grid_constant__ CtArgs<T> a, const T *rhs, T *xout) {
         int J = w.ly0, K = w.lz0;
         for (int t = tid; t < hy * (v.bz >> 1) * v.P; t += w.act) {
           T sum = 0;
-#pragma unroll 2
-          for (int q = 0; q < 8; ++q)
-            sum += ct_resid(v, w.p, q & 1, 2 * J + ((q >> 1) & 1), 2 * K + (q >> 2));
+#pragma unroll
+          for (int q = 0; q < 4; ++q)  // the children of colour 0 (see k_resid_restrict_h)
+            sum += ct_resid(v, w.p, (q & 1) ^ (q >> 1), 2 * J + (q & 1), 2 * K + (q >> 1));
           const T r = (T)0.5 * sum;
           const int y = (v.y0 >> 1) + J, z = (v.z0 >> 1) + K;
           if (coarsest) {

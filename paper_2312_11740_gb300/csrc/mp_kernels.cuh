@@ -635,9 +635,11 @@ k_tail(TailArgs a, const T *__restrict__ rhs, T *__restrict__ xout) {
     for (int e = threadIdx.x; e < a.lv[l + 1].n; e += TAIL_THREADS) {
       const int I = e % dc.nx, J = (e / dc.nx) % dc.ny, K = e / (dc.nx * dc.ny);
       T sum = 0;
-      for (int q = 0; q < 8; ++q)
+      for (int q = 0; q < 4; ++q) {  // the children of colour 0
+        const int dj = q & 1, dk = q >> 1;
         sum += resid_at(v.x, v.b, v.wx, v.wy, v.wz, (const T *)nullptr, (const T *)v.dd, d,
-                        2 * I + (q & 1), 2 * J + ((q >> 1) & 1), 2 * K + (q >> 2));
+                        2 * I + (dj ^ dk), 2 * J + dj, 2 * K + dk);
+      }
       vc.b[e] = (T)0.5 * sum;
     }
     __syncthreads();
@@ -693,9 +695,11 @@ __device__ __forceinline__ void resid_restrict_cell(const T *__restrict__ x,
                                                     int J, int K) {
   T s = 0;
 #pragma unroll
-  for (int q = 0; q < 8; ++q)
-    s += resid_at(x, b, bx, by, bz, diag, (const T *)nullptr, df, 2 * I + (q & 1), 2 * J + ((q >> 1) & 1),
-                  2 * K + (q >> 2));
+  for (int q = 0; q < 4; ++q) {  // the children of colour 0
+    const int dj = q & 1, dk = q >> 1;
+    s += resid_at(x, b, bx, by, bz, diag, (const T *)nullptr, df, 2 * I + (dj ^ dk), 2 * J + dj,
+                  2 * K + dk);
+  }
   bc[at(dc, I, J, K)] = (T)0.5 * s;
 }
 
@@ -855,7 +859,10 @@ __device__ __forceinline__ float resid_h(const float *__restrict__ x, const floa
   return b[c] - s * inv_fs;
 }
 
-// residual + restriction (half the sum of the 8 children) on the FP16 faces
+// residual + restriction (half the sum of the 8 children) on the FP16 faces.
+// Restriction follows a sweep that ended with colour 1, whose cells' equations
+// have just been solved: their residuals are rounding, and only the four
+// children of colour 0 are formed (here and in every restriction of the V-cycle).
 __global__ void k_resid_restrict_h(const float *__restrict__ x, const float *__restrict__ b,
                                    const __half *__restrict__ hx, const __half *__restrict__ hy,
                                    const __half *__restrict__ hz, const __half *__restrict__ dd16,
@@ -865,20 +872,23 @@ __global__ void k_resid_restrict_h(const float *__restrict__ x, const float *__r
   if (I >= dc.nx || J >= dc.ny) return;
   float s = 0.f;
 #pragma unroll
-  for (int q = 0; q < 8; ++q)
-    s += resid_h(x, b, hx, hy, hz, dd16, inv_fs, df, 2 * I + (q & 1), 2 * J + ((q >> 1) & 1),
-                 2 * K + (q >> 2));
+  for (int q = 0; q < 4; ++q) {
+    const int dj = q & 1, dk = q >> 1;
+    s += resid_h(x, b, hx, hy, hz, dd16, inv_fs, df, 2 * I + (dj ^ dk), 2 * J + dj, 2 * K + dk);
+  }
   bc[at(dc, I, J, K)] = 0.5f * s;
 }
 
-// Residuals bt - At x of the 4-cell x-chunk [i0, i0 + 4) of fine row (j, k),
-// with the FP16 faces and 16-byte loads (resid_h's arithmetic per cell)
+// Residuals bt - At x of the cells i0 + O and i0 + O + 2 (the two of colour 0) of
+// the 4-cell x-chunk [i0, i0 + 4) of fine row (j, k), with the FP16 faces and 16-byte
+// loads (resid_h's arithmetic per cell)
+template <int O>
 __device__ __forceinline__ void resid_h4(const float *__restrict__ x, const float *__restrict__ b,
                                          const __half *__restrict__ hx,
                                          const __half *__restrict__ hy,
                                          const __half *__restrict__ hz,
                                          const __half *__restrict__ dd16, float inv_fs,
-                                         const Dims &d, int i0, int j, int k, float r[4]) {
+                                         const Dims &d, int i0, int j, int k, float r[2]) {
   const size_t c0 = at(d, i0, j, k);
   const size_t cyl = at(d, i0, wlo(j, d.ny), k), cyh = at(d, i0, whi(j, d.ny), k);
   const size_t czl = at(d, i0, j, wlo(k, d.nz)), czh = at(d, i0, j, whi(k, d.nz));
@@ -893,12 +903,19 @@ __device__ __forceinline__ void resid_h4(const float *__restrict__ x, const floa
   const H4 fyh = *reinterpret_cast<const H4 *>(hy + cyh);
   const H4 fz = *reinterpret_cast<const H4 *>(hz + c0);
   const H4 fzh = *reinterpret_cast<const H4 *>(hz + czh);
-  const size_t ce = at(d, whi(i0 + 3, d.nx), j, k);
-  const float fxe = hf(hx, ce), xp = x[ce], xm = x[at(d, wlo(i0, d.nx), j, k)];
+  float fxe = 0.f, xe;  // past the chunk's end: x face and x of i0 + 4 (O = 1), x of i0 - 1 (O = 0)
+  if (O == 1) {
+    const size_t ce = at(d, whi(i0 + 3, d.nx), j, k);
+    fxe = hf(hx, ce);
+    xe = x[ce];
+  } else {
+    xe = x[at(d, wlo(i0, d.nx), j, k)];
+  }
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
+  for (int w = 0; w < 2; ++w) {
+    const int q = O + 2 * w;
     const float v = f4_at(xc, q);
-    const float x_l = q > 0 ? f4_at(xc, q - 1) : xm, x_h = q < 3 ? f4_at(xc, q + 1) : xp;
+    const float x_l = q > 0 ? f4_at(xc, q - 1) : xe, x_h = q < 3 ? f4_at(xc, q + 1) : xe;
     float s = h4_at(fx, q) * (x_l - v);
     s = fmaf(q < 3 ? h4_at(fx, q + 1) : fxe, x_h - v, s);
     s = fmaf(h4_at(fy, q), f4_at(xyl, q) - v, s);
@@ -906,7 +923,7 @@ __device__ __forceinline__ void resid_h4(const float *__restrict__ x, const floa
     s = fmaf(h4_at(fz, q), f4_at(xzl, q) - v, s);
     s = fmaf(h4_at(fzh, q), f4_at(xzh, q) - v, s);
     if (dd16) s = fmaf(-dd_h(dd16, c0 + q), v, s);
-    r[q] = f4_at(bb, q) - s * inv_fs;
+    r[w] = f4_at(bb, q) - s * inv_fs;
   }
 }
 
@@ -920,17 +937,17 @@ __global__ void k_resid_restrict_h4(const float *__restrict__ x, const float *__
   griddep_wait();
   const int m = blockIdx.x * BX + threadIdx.x, J = blockIdx.y * BY + threadIdx.y, K = blockIdx.z;
   if (m >= (df.nx >> 2) || J >= dc.ny) return;
-  float s0 = 0.f, s1 = 0.f, r[4];
-#pragma unroll
-  for (int row = 0; row < 4; ++row) {  // (dj, dk) = (0,0), (1,0), (0,1), (1,1)
-    resid_h4(x, b, hx, hy, hz, dd16, inv_fs, df, 4 * m, 2 * J + (row & 1), 2 * K + (row >> 1), r);
-    s0 += r[0];
-    s0 += r[1];
-    s1 += r[2];
-    s1 += r[3];
-  }
-  bc[at(dc, 2 * m, J, K)] = 0.5f * s0;
-  bc[at(dc, 2 * m + 1, J, K)] = 0.5f * s1;
+  float s0 = 0.f, s1 = 0.f, r[2];
+  const int i0 = 4 * m, j = 2 * J, k = 2 * K;
+  resid_h4<0>(x, b, hx, hy, hz, dd16, inv_fs, df, i0, j, k, r);
+  s0 += r[0], s1 += r[1];
+  resid_h4<1>(x, b, hx, hy, hz, dd16, inv_fs, df, i0, j + 1, k, r);
+  s0 += r[0], s1 += r[1];
+  resid_h4<1>(x, b, hx, hy, hz, dd16, inv_fs, df, i0, j, k + 1, r);
+  s0 += r[0], s1 += r[1];
+  resid_h4<0>(x, b, hx, hy, hz, dd16, inv_fs, df, i0, j + 1, k + 1, r);
+  s0 += r[0], s1 += r[1];
+  *reinterpret_cast<float2 *>(bc + at(dc, 2 * m, J, K)) = make_float2(0.5f * s0, 0.5f * s1);
 }
 
 template <typename T>

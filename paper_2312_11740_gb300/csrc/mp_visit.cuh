@@ -427,9 +427,10 @@ __global__ void __launch_bounds__(VS_THREADS, 1) k_visit(const VisitArgs<T> a) {
       const int rc = dP.q(t), p = t - rc * P, K = dhy.q(rc), J = rc - K * hy;
       T sum = 0;
 #pragma unroll
-      for (int w = 0; w < 8; ++w) {  // (di, dj, dk) = bits of w
-        const int o = w & 1, ly = 2 * J + ((w >> 1) & 1), lz = 2 * K + (w >> 2);
-        const int r = lz * by + ly, k = (y0 + ly + z0 + lz + o) & 1;  // colour
+      for (int w = 0; w < 4; ++w) {  // the children of colour 0
+        constexpr int k = 0;
+        const int o = (w & 1) ^ (w >> 1), ly = 2 * J + (w & 1), lz = 2 * K + (w >> 1);
+        const int r = lz * by + ly;
         const VsAt i = vs_at(r, ly, lz, p, o, P, by);
         const T *xo = X + (1 - k) * nh;
         const F *hxc = HX + k * n1, *hxo = HX + (1 - k) * n1, *hyc = HY + k * n1y,
