@@ -35,6 +35,7 @@ namespace mp {
 namespace cgx = cooperative_groups;
 
 constexpr int CT_MAX_CTAS = 16, CTL_THREADS = 512, CT_MAX_LEVELS = 10, CT_MAX_COARSE = 512;
+constexpr int CT_MAX_TAB = 1024;  // rows and planes of all levels
 constexpr int CT_POLL = 1 << 22;  // polls of one wait (tenths of a second)
 
 template <typename T>
@@ -122,20 +123,33 @@ __host__ __device__ inline int ct_part(int n, int p, int row) {
   return (((row >> 1) + 1) * p - 1) / (n >> 1);
 }
 
+// Quotient t / d from m = ct_magic(d) (round-up reciprocal: exact while t d <
+// 2^32).  d = 1 gives m = 0, read as "the quotient is t".
+__device__ __forceinline__ unsigned ct_magic(unsigned d) { return 0xFFFFFFFFu / d + 1u; }
+__device__ __forceinline__ int ct_div(int t, unsigned m) {
+  return m ? (int)__umulhi((unsigned)t, m) : t;
+}
+
+// This CTA's part of a level, formed once per launch in shared memory (the
+// divisions behind it take about a microsecond and every step of a level
+// needs them): block origin and size, neighbours, and the multipliers of the walks.
+struct CtBlock {
+  int own, cy, cz, y0, by, z0, bz;
+  int ym, yp, zm, zp;            // CTAs of the blocks beside
+  unsigned mP, mh, m0, m1, m2;   // ct_magic of P, by / 2, by, by + 1, by + 2
+};
+
 // One level seen by one CTA.
 template <typename T>
 struct CtView {
   T *X, *B, *ID, *HX, *HY, *HZ, *DD;
-  int nx, ny, nz, P, py, pz, bym, bzm, cy, cz, y0, by, z0, bz;
+  int nx, ny, nz, P, py, pz, bym, bzm, y0, by, z0, bz;
   int n1, nh, n1y, n1z;
   bool own;  // this CTA holds a block
-  __device__ CtView(T *base, const CtLevel<T> &l, int rank) {
+  __device__ CtView(T *base, const CtLevel<T> &l, const CtBlock &k) {
     nx = l.d.nx, ny = l.d.ny, nz = l.d.nz, P = nx >> 1;
     py = l.py, pz = l.pz, bym = l.bym, bzm = l.bzm;
-    own = rank < py * pz;
-    cy = own ? rank % py : 0, cz = own ? rank / py : 0;
-    y0 = ct_cut(ny, py, cy), by = ct_cut(ny, py, cy + 1) - y0;
-    z0 = ct_cut(nz, pz, cz), bz = ct_cut(nz, pz, cz + 1) - z0;
+    own = k.own, y0 = k.y0, by = k.by, z0 = k.z0, bz = k.bz;
     n1 = bym * bzm * P, nh = (bym + 2) * (bzm + 2) * P;
     n1y = (bym + 1) * bzm * P, n1z = bym * (bzm + 1) * P;
     X = base + l.off;
@@ -152,18 +166,19 @@ struct CtView {
   }
 };
 
-// The walk of a thread over its cells: one pair p, rows advancing by rpt.
+// The walk of a thread over its cells: one pair p, rows advancing by rpt.  rows:
+// rows of a plane of the walk, m its ct_magic.
 struct CtWalk {
   int p, act, ly0, lz0, dly, dlz;
   bool works;
-  __device__ CtWalk(int P, int by) {
-    const int tid = threadIdx.x, rpt = CTL_THREADS / P;
+  __device__ CtWalk(int P, unsigned mP, int rows, unsigned m) {
+    const int tid = threadIdx.x, rpt = ct_div(CTL_THREADS, mP);
     act = rpt * P;
     works = tid < act;
-    const int r0 = tid / P;
+    const int r0 = ct_div(tid, mP);
     p = tid - r0 * P;
-    lz0 = r0 / by, ly0 = r0 - lz0 * by;
-    dlz = rpt / by, dly = rpt - dlz * by;
+    lz0 = ct_div(r0, m), ly0 = r0 - lz0 * rows;
+    dlz = ct_div(rpt, m), dly = rpt - dlz * rows;
   }
 };
 
@@ -182,48 +197,65 @@ __device__ __forceinline__ void ct_half(const CtView<T> &v, const CtWalk &w, boo
   T *Xc = v.X + C * v.nh;
   const T *Xo = v.X + (1 - C) * v.nh;
   if (w.works) {
+    // two cells at a time: both cells' operands are loaded before either is stored
+    // (the compiler cannot move a load past a store to shared memory)
     int ly = w.ly0, lz = w.lz0;
-    for (int t = threadIdx.x; t < by * bz * P; t += w.act) {
-      const int f = v.f(w.p, ly, lz), h = f + (2 * lz + v.bym + 3) * P, fy = f + lz * P;
-      const int o = (par + ly + lz) & 1;
-      const int jl = o ? 0 : dlo, jh = o ? dhi : 0;
-      T num = -v.B[C * v.n1 + f];
-      if (!zero) {
-        num = fma(v.HX[C * v.n1 + f], Xo[h + jl], num);
-        num = fma(v.HX[(1 - C) * v.n1 + f + jh], Xo[h + jh], num);
-        num = fma(v.HY[C * v.n1y + fy], Xo[h - P], num);
-        num = fma(v.HY[(1 - C) * v.n1y + fy + P], Xo[h + P], num);
-        num = fma(v.HZ[C * v.n1z + f], Xo[h - sZ], num);
-        num = fma(v.HZ[(1 - C) * v.n1z + f + v.bym * P], Xo[h + sZ], num);
+    for (int t = threadIdx.x; t < by * bz * P; t += 2 * w.act) {
+      int yy[2], zz[2], hh[2];
+      T xx[2];
+      const bool two = t + w.act < by * bz * P;
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        yy[u] = ly, zz[u] = lz;
+        if (u == 0 || two) {
+          const int f = v.f(w.p, ly, lz), h = f + (2 * lz + v.bym + 3) * P, fy = f + lz * P;
+          const int o = (par + ly + lz) & 1;
+          const int jl = o ? 0 : dlo, jh = o ? dhi : 0;
+          T num = -v.B[C * v.n1 + f];
+          if (!zero) {
+            num = fma(v.HX[C * v.n1 + f], Xo[h + jl], num);
+            num = fma(v.HX[(1 - C) * v.n1 + f + jh], Xo[h + jh], num);
+            num = fma(v.HY[C * v.n1y + fy], Xo[h - P], num);
+            num = fma(v.HY[(1 - C) * v.n1y + fy + P], Xo[h + P], num);
+            num = fma(v.HZ[C * v.n1z + f], Xo[h - sZ], num);
+            num = fma(v.HZ[(1 - C) * v.n1z + f + v.bym * P], Xo[h + sZ], num);
+          }
+          xx[u] = num * v.ID[C * v.n1 + f];
+          hh[u] = h;
+        }
+        ly += w.dly, lz += w.dlz;
+        if (ly >= by) ly -= by, ++lz;
       }
-      const T x = num * v.ID[C * v.n1 + f];
-      Xc[h] = x;
-      // boundary rows: to the block beside, or this block's own halo
-      if (ly == 0) {
-        if (v.py == 1) Xc[h + by * P] = x;
-        else if (exchange) ct_send(rem[0] + m + lz * P * W, x, e);
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        if (u == 1 && !two) break;
+        const T x = xx[u];
+        const int h = hh[u], y = yy[u], z = zz[u];
+        Xc[h] = x;
+        // boundary rows: to the block beside, or this block's own halo
+        if (y == 0) {
+          if (v.py == 1) Xc[h + by * P] = x;
+          else if (exchange) ct_send(rem[0] + m + z * P * W, x, e);
+        }
+        if (y == by - 1) {
+          if (v.py == 1) Xc[h - by * P] = x;
+          else if (exchange) ct_send(rem[1] + m + z * P * W, x, e);
+        }
+        if (z == 0) {
+          if (v.pz == 1) Xc[h + bz * sZ] = x;
+          else if (exchange) ct_send(rem[2] + m + y * P * W, x, e);
+        }
+        if (z == bz - 1) {
+          if (v.pz == 1) Xc[h - bz * sZ] = x;
+          else if (exchange) ct_send(rem[3] + m + y * P * W, x, e);
+        }
       }
-      if (ly == by - 1) {
-        if (v.py == 1) Xc[h - by * P] = x;
-        else if (exchange) ct_send(rem[1] + m + lz * P * W, x, e);
-      }
-      if (lz == 0) {
-        if (v.pz == 1) Xc[h + bz * sZ] = x;
-        else if (exchange) ct_send(rem[2] + m + ly * P * W, x, e);
-      }
-      if (lz == bz - 1) {
-        if (v.pz == 1) Xc[h - bz * sZ] = x;
-        else if (exchange) ct_send(rem[3] + m + ly * P * W, x, e);
-      }
-      ly += w.dly, lz += w.dlz;
-      if (ly >= by) ly -= by, ++lz;
     }
   }
   if (exchange) {
     const int ry = v.py > 1 ? 2 * bz : 0, rz = v.pz > 1 ? 2 * by : 0;  // halo rows received
-    const int rpt = w.act / P;
     if (w.works)
-      for (int row = (threadIdx.x - w.p) / P; row < ry + rz; row += rpt) {
+      for (int row = w.lz0 * by + w.ly0; row < ry + rz; row += w.dlz * by + w.dly) {
         int slot, dst;
         if (row < ry) {
           const bool hi = row >= bz;
@@ -280,18 +312,50 @@ k_ctail(const __grid_constant__ CtArgs<T> a, const T *rhs, T *xout) {
   const int nctas = (int)cl.num_blocks();
   extern __shared__ __align__(16) unsigned char ct_raw[];
   T *base = reinterpret_cast<T *>(ct_raw);
-  __shared__ double mean_s;
+  __shared__ CtBlock blk[CT_MAX_LEVELS];
+  // owner and local index of every row y and plane z of a level, by level: part << 16 | local
+  __shared__ int tab[CT_MAX_TAB], tab0[CT_MAX_LEVELS];
   const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(ct_raw);
   const uint32_t mail = sbase + a.mail, flip = a.mail_words * 4;  // half of the words, in bytes
   constexpr int W = sizeof(T) == 8 ? 16 : 8;
   const int last = a.nlev - 1;
-  // this CTA's blocks of the level coefficients.  They were formed with the
-  // geometry, before the kernel this launch follows: read ahead of the wait
-  for (int l = 0; l < last; ++l) {
+  // Nothing up to the wait depends on the kernel this launch follows (the level
+  // coefficients were formed with the geometry), so it overlaps that kernel's end.
+  if (tid < last) {
+    const CtLevel<T> &g = a.lv[tid];
+    CtBlock k;
+    k.own = rank < g.py * g.pz;
+    k.cy = k.own ? rank % g.py : 0, k.cz = k.own ? rank / g.py : 0;
+    k.y0 = ct_cut(g.d.ny, g.py, k.cy), k.by = ct_cut(g.d.ny, g.py, k.cy + 1) - k.y0;
+    k.z0 = ct_cut(g.d.nz, g.pz, k.cz), k.bz = ct_cut(g.d.nz, g.pz, k.cz + 1) - k.z0;
+    k.ym = (k.cy == 0 ? g.py - 1 : k.cy - 1) + k.cz * g.py;
+    k.yp = (k.cy == g.py - 1 ? 0 : k.cy + 1) + k.cz * g.py;
+    k.zm = k.cy + (k.cz == 0 ? g.pz - 1 : k.cz - 1) * g.py;
+    k.zp = k.cy + (k.cz == g.pz - 1 ? 0 : k.cz + 1) * g.py;
+    k.mP = ct_magic(g.d.nx >> 1), k.mh = ct_magic(k.by >> 1), k.m0 = ct_magic(k.by);
+    k.m1 = ct_magic(k.by + 1), k.m2 = ct_magic(k.by + 2);
+    blk[tid] = k;
+    int t0 = 0;
+    for (int l = 0; l < tid; ++l) t0 += a.lv[l].d.ny + a.lv[l].d.nz;
+    tab0[tid] = t0;
+  }
+  for (int e = tid; e < a.mail_words; e += CTL_THREADS)
+    reinterpret_cast<unsigned long long *>(ct_raw + a.mail)[e] = 0ull;
+  __syncthreads();
+  for (int l = 1; l < last; ++l) {
     const CtLevel<T> &g = a.lv[l];
-    const CtView<T> v(base, g, rank);
+    for (int q = tid; q < g.d.ny + g.d.nz; q += CTL_THREADS) {
+      const bool y = q < g.d.ny;
+      const int n = y ? g.d.ny : g.d.nz, p = y ? g.py : g.pz, row = y ? q : q - g.d.ny;
+      const int c = ct_part(n, p, row);
+      tab[tab0[l] + q] = c << 16 | (row - ct_cut(n, p, c));
+    }
+  }
+  for (int l = 0; l < last; ++l) {  // this CTA's blocks of the level coefficients
+    const CtLevel<T> &g = a.lv[l];
+    const CtView<T> v(base, g, blk[l]);
     if (!v.own) continue;
-    const CtWalk w(v.P, v.by + 1);  // rows 0 .. by, planes 0 .. bz: the high faces too
+    const CtWalk w(v.P, blk[l].mP, v.by + 1, blk[l].m1);  // rows 0 .. by, planes 0 .. bz
     if (w.works) {
       int ly = w.ly0, lz = w.lz0;
       for (; lz <= v.bz;) {
@@ -301,43 +365,46 @@ k_ctail(const __grid_constant__ CtArgs<T> a, const T *rhs, T *xout) {
         const bool iny = ly < v.by, inz = lz < v.bz;
         if (inz) {
           const int s = (lz * (v.bym + 1) + ly) * v.P + w.p;
-          v.HY[q * v.n1y + s] = g.by[c];
-          v.HY[(1 - q) * v.n1y + s] = g.by[c + 1];
+          const auto fy = vs_pair(g.by + c);
+          v.HY[q * v.n1y + s] = fy.x;
+          v.HY[(1 - q) * v.n1y + s] = fy.y;
         }
         if (iny) {
           const int s = v.f(w.p, ly, lz);
-          v.HZ[q * v.n1z + s] = g.bz[c];
-          v.HZ[(1 - q) * v.n1z + s] = g.bz[c + 1];
+          const auto fz = vs_pair(g.bz + c);
           if (inz) {
-            v.HX[q * v.n1 + s] = g.bx[c];
-            v.HX[(1 - q) * v.n1 + s] = g.bx[c + 1];
-            v.ID[q * v.n1 + s] = g.idiag[c];
-            v.ID[(1 - q) * v.n1 + s] = g.idiag[c + 1];
+            const auto fx = vs_pair(g.bx + c), id = vs_pair(g.idiag + c);
+            v.HX[q * v.n1 + s] = fx.x;
+            v.HX[(1 - q) * v.n1 + s] = fx.y;
+            v.ID[q * v.n1 + s] = id.x;
+            v.ID[(1 - q) * v.n1 + s] = id.y;
             if (v.DD) {
-              v.DD[q * v.n1 + s] = g.dd[c];
-              v.DD[(1 - q) * v.n1 + s] = g.dd[c + 1];
+              const auto dd = vs_pair(g.dd + c);
+              v.DD[q * v.n1 + s] = dd.x;
+              v.DD[(1 - q) * v.n1 + s] = dd.y;
             }
           }
+          v.HZ[q * v.n1z + s] = fz.x;
+          v.HZ[(1 - q) * v.n1z + s] = fz.y;
         }
         ly += w.dly, lz += w.dlz;
         if (ly >= v.by + 1) ly -= v.by + 1, ++lz;
       }
     }
   }
-  for (int e = tid; e < a.mail_words; e += CTL_THREADS)
-    reinterpret_cast<unsigned long long *>(ct_raw + a.mail)[e] = 0ull;
+  cl.sync();  // every CTA of the cluster has started and cleared its slots
   griddep_wait();
   {
-    const CtView<T> v(base, a.lv[0], rank);
+    const CtView<T> v(base, a.lv[0], blk[0]);
     if (v.own) {
-      const CtWalk w(v.P, v.by);
+      const CtWalk w(v.P, blk[0].mP, v.by, blk[0].m0);
       if (w.works) {
         int ly = w.ly0, lz = w.lz0;
         for (int t = tid; t < v.by * v.bz * v.P; t += w.act) {
           const int q = (v.y0 + ly + v.z0 + lz) & 1, s = v.f(w.p, ly, lz);
-          const size_t c = at(a.lv[0].d, 2 * w.p, v.y0 + ly, v.z0 + lz);
-          v.B[q * v.n1 + s] = rhs[c];
-          v.B[(1 - q) * v.n1 + s] = rhs[c + 1];
+          const auto r = vs_pair(rhs + at(a.lv[0].d, 2 * w.p, v.y0 + ly, v.z0 + lz));
+          v.B[q * v.n1 + s] = r.x;
+          v.B[(1 - q) * v.n1 + s] = r.y;
           ly += w.dly, lz += w.dlz;
           if (ly >= v.by) ly -= v.by, ++lz;
         }
@@ -345,24 +412,21 @@ k_ctail(const __grid_constant__ CtArgs<T> a, const T *rhs, T *xout) {
     }
   }
   bool dead = *(volatile double *)a.err != 0.0;
-  cl.sync();  // every CTA of the cluster has started, loaded its blocks and cleared its slots
+  __syncthreads();
   unsigned e = 0;  // epoch of the last exchange, counted alike by every CTA
 
   // the sweeps of one level: colours c0, 1 - c0; the last exchange of an
   // upward visit is not needed
-  auto sweeps = [&](const CtView<T> &v, auto first, int nu, bool zero, bool keep_last) {
+  auto sweeps = [&](const CtView<T> &v, const CtBlock &k, auto first, int nu, bool zero,
+                    bool keep_last) {
     constexpr int C0 = decltype(first)::value;
     if (v.own) {
-      const CtWalk w(v.P, v.by);
+      const CtWalk w(v.P, k.mP, v.by, k.m0);
       uint32_t rem[4];
-      const int ym = (v.cy == 0 ? v.py - 1 : v.cy - 1) + v.cz * v.py,
-                yp = (v.cy == v.py - 1 ? 0 : v.cy + 1) + v.cz * v.py,
-                zm = v.cy + (v.cz == 0 ? v.pz - 1 : v.cz - 1) * v.py,
-                zp = v.cy + (v.cz == v.pz - 1 ? 0 : v.cz + 1) * v.py;
-      rem[0] = ct_map(mail + (v.bzm * v.P + w.p) * W, ym);
-      rem[1] = ct_map(mail + w.p * W, yp);
-      rem[2] = ct_map(mail + ((2 * v.bzm + v.bym) * v.P + w.p) * W, zm);
-      rem[3] = ct_map(mail + (2 * v.bzm * v.P + w.p) * W, zp);
+      rem[0] = ct_map(mail + (v.bzm * v.P + w.p) * W, k.ym);
+      rem[1] = ct_map(mail + w.p * W, k.yp);
+      rem[2] = ct_map(mail + ((2 * v.bzm + v.bym) * v.P + w.p) * W, k.zm);
+      rem[3] = ct_map(mail + (2 * v.bzm * v.P + w.p) * W, k.zp);
       for (int s = 0; s < nu; ++s) {
         ct_half<T, C0>(v, w, zero && s == 0, e + 2 * s + 1, mail, rem, flip, dead, a.err);
         const bool x = keep_last || s + 1 < nu;
@@ -373,14 +437,15 @@ k_ctail(const __grid_constant__ CtArgs<T> a, const T *rhs, T *xout) {
   };
 
   for (int l = 0; l < last; ++l) {  // down
-    const CtView<T> v(base, a.lv[l], rank);
-    sweeps(v, VsColour<0>{}, a.lv[l].nu1, true, true);
+    const CtView<T> v(base, a.lv[l], blk[l]);
+    sweeps(v, blk[l], VsColour<0>{}, a.lv[l].nu1, true, true);
     const CtLevel<T> &gc = a.lv[l + 1];
     const bool coarsest = l + 1 == last;
     if (v.own) {  // residual, restricted to the coarser block's owner
-      const CtView<T> vc(base, gc, rank);
+      const CtView<T> vc(base, gc, blk[coarsest ? l : l + 1]);
+      const int *ty = tab + tab0[coarsest ? l : l + 1], *tz = ty + vc.ny;
       const int hy = v.by >> 1;
-      const CtWalk w(v.P, hy);
+      const CtWalk w(v.P, blk[l].mP, hy, blk[l].mh);
       if (w.works) {
         int J = w.ly0, K = w.lz0;
         for (int t = tid; t < hy * (v.bz >> 1) * v.P; t += w.act) {
@@ -395,11 +460,9 @@ k_ctail(const __grid_constant__ CtArgs<T> a, const T *rhs, T *xout) {
                 sbase + (gc.off + gc.n + w.p + gc.d.nx * (y + gc.d.ny * z)) * (int)sizeof(T);
             for (int k = 0; k < nctas; ++k) ct_st(ct_map(to, k), r);
           } else {
-            const int oy = ct_part(vc.ny, vc.py, y), oz = ct_part(vc.nz, vc.pz, z);
-            const int ly = y - ct_cut(vc.ny, vc.py, oy), lz = z - ct_cut(vc.nz, vc.pz, oz);
-            const int c = (w.p + y + z) & 1;
-            T *p = vc.B + c * vc.n1 + vc.f(w.p >> 1, ly, lz);
-            ct_st(ct_map((uint32_t)__cvta_generic_to_shared(p), oy + oz * vc.py), r);
+            const int ey = ty[y], ez = tz[z], c = (w.p + y + z) & 1;
+            T *p = vc.B + c * vc.n1 + vc.f(w.p >> 1, ey & 0xffff, ez & 0xffff);
+            ct_st(ct_map((uint32_t)__cvta_generic_to_shared(p), (ey >> 16) + (ez >> 16) * vc.py), r);
           }
           J += w.dly, K += w.dlz;
           if (J >= hy) J -= hy, ++K;
@@ -408,32 +471,35 @@ k_ctail(const __grid_constant__ CtArgs<T> a, const T *rhs, T *xout) {
     }
     cl.sync();
   }
-  {  // coarsest: x = Minv (-(b - mean b)) in FP64, rows spread over the cluster's warps
+  {  // coarsest: x = -Minv (b - mean b) in FP64, rows spread over the cluster's warps.
+    // Minv 1 = 1 for a singular operator (M 1 = 1), so the mean is added to the
+    // product instead of removed from b, and every warp forms it along the way
     const CtLevel<T> &g = a.lv[last];
     const int n = g.n;
     T *X = base + g.off, *B = X + n;
-    double acc0 = 0.0;
-    for (int q = tid; q < n; q += CTL_THREADS) acc0 += (double)B[q];
-    const double sum = block_sum(acc0);
-    if (tid == 0) mean_s = a.singular ? sum / n : 0.0;
-    __syncthreads();
-    const double mean = mean_s;
     const int lane = tid & 31;
     for (int r = rank * (CTL_THREADS / 32) + (tid >> 5); r < n; r += nctas * (CTL_THREADS / 32)) {
-      double acc = 0.0;
-      for (int c = lane; c < n; c += 32)
-        acc = fma(__ldg(a.Minv + (size_t)r * n + c), (double)B[c] - mean, acc);
-      const T x = (T)(-warp_sum(acc));
-      if (lane < nctas) ct_st(ct_map((uint32_t)__cvta_generic_to_shared(X + r), lane), x);
+      double acc = 0.0, sum = 0.0;
+#pragma unroll 4
+      for (int c = lane; c < n; c += 32) {
+        const double bc = (double)B[c];
+        acc = fma(__ldg(a.Minv + (size_t)r * n + c), bc, acc);
+        sum += bc;
+      }
+      acc = warp_sum(acc);
+      sum = a.singular ? warp_sum(sum) / n : 0.0;
+      if (lane < nctas) ct_st(ct_map((uint32_t)__cvta_generic_to_shared(X + r), lane), (T)(sum - acc));
     }
     cl.sync();
   }
   for (int l = last - 1; l >= 0; --l) {  // up
-    const CtView<T> v(base, a.lv[l], rank);
+    const CtView<T> v(base, a.lv[l], blk[l]);
     const CtLevel<T> &gc = a.lv[l + 1];
     if (v.own) {  // the parents' corrections, halo rows included (faces of the block, not corners)
-      const CtView<T> vc(base, gc, rank);
-      const CtWalk w(v.P, v.by + 2);
+      const int lc = l + 1 == last ? l : l + 1;
+      const CtView<T> vc(base, gc, blk[lc]);
+      const int *ty = tab + tab0[lc], *tz = ty + vc.ny;
+      const CtWalk w(v.P, blk[l].mP, v.by + 2, blk[l].m2);
       if (w.works) {
         int hy = w.ly0, hz = w.lz0;
         for (; hz < v.bz + 2;) {
@@ -447,11 +513,10 @@ k_ctail(const __grid_constant__ CtArgs<T> a, const T *rhs, T *xout) {
             if (l + 1 == last) {
               x = base[gc.off + w.p + gc.d.nx * (J + gc.d.ny * K)];
             } else {
-              const int oy = ct_part(vc.ny, vc.py, J), oz = ct_part(vc.nz, vc.pz, K);
-              const int ly = J - ct_cut(vc.ny, vc.py, oy), lz = K - ct_cut(vc.nz, vc.pz, oz);
-              const int c = (w.p + J + K) & 1;
-              T *p = vc.X + c * vc.nh + vc.h(w.p >> 1, ly, lz);
-              x = ct_ld(ct_map((uint32_t)__cvta_generic_to_shared(p), oy + oz * vc.py), T());
+              const int ey2 = ty[J], ez2 = tz[K], c = (w.p + J + K) & 1;
+              T *p = vc.X + c * vc.nh + vc.h(w.p >> 1, ey2 & 0xffff, ez2 & 0xffff);
+              x = ct_ld(ct_map((uint32_t)__cvta_generic_to_shared(p),
+                               (ey2 >> 16) + (ez2 >> 16) * vc.py), T());
             }
             const int s = v.h(w.p, hy - 1, hz - 1);
             v.X[s] += x;
@@ -463,25 +528,28 @@ k_ctail(const __grid_constant__ CtArgs<T> a, const T *rhs, T *xout) {
       }
       __syncthreads();
     }
-    sweeps(v, VsColour<1>{}, a.lv[l].nu2, false, false);
+    // at the top level: this CTA reads no other's shared memory any more
+    if (l == 0) cl.barrier_arrive();
+    sweeps(v, blk[l], VsColour<1>{}, a.lv[l].nu2, false, false);
     if (l > 0) cl.sync();  // the finer level reads this one's x
   }
-  const CtView<T> v(base, a.lv[0], rank);
+  const CtView<T> v(base, a.lv[0], blk[0]);
   if (v.own) {
-    const CtWalk w(v.P, v.by);
+    const CtWalk w(v.P, blk[0].mP, v.by, blk[0].m0);
     if (w.works) {
       int ly = w.ly0, lz = w.lz0;
       for (int t = tid; t < v.by * v.bz * v.P; t += w.act) {
         const int q = (v.y0 + ly + v.z0 + lz) & 1, s = v.h(w.p, ly, lz);
         const size_t c = at(a.lv[0].d, 2 * w.p, v.y0 + ly, v.z0 + lz);
-        xout[c] = v.X[q * v.nh + s];
-        xout[c + 1] = v.X[(1 - q) * v.nh + s];
+        vs_put(xout + c, v.X[q * v.nh + s], v.X[(1 - q) * v.nh + s]);
         ly += w.dly, lz += w.dlz;
         if (ly >= v.by) ly -= v.by, ++lz;
       }
     }
   }
-  cl.sync();  // no CTA leaves while another may still write to its shared memory
+  // No CTA leaves while another may still read its shared memory.  (Boundary rows are
+  // written to it only until the last exchange, which it has received.)
+  cl.barrier_wait();
 }
 
 }  // namespace mp

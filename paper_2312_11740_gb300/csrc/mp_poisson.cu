@@ -87,6 +87,7 @@ constexpr int TAIL32_NU_MAX = 4;  // sweeps per level in the one-CTA FP32 tail
 // largest level of the cluster tail: above it a half-sweep takes longer on the
 // cluster's SMs than a launch or a level visit spread over all of them (FP64: the
 // pipe's rate)
+constexpr size_t CT_STATIC = 6144;  // static shared memory of the cluster tail (at most)
 constexpr size_t CT_TOP32 = 65536, CT_TOP64 = 16384;
 // Smallest level of the fused sweep and largest of an FP32 visit.  A level that
 // stays in L2 streams its faces for every colour from there: measured per CG
@@ -1559,9 +1560,11 @@ mp_status ctail_setup(mp_poisson *hd, CtPlan *out) {
       p.mail = (int)(elems * sizeof(T));
       p.mail_words = 2 * slots * (sizeof(T) == 8 ? 2 : 1);
       p.bytes = (size_t)p.mail + (size_t)p.mail_words * 8;
-      if (p.bytes + 1024 > (size_t)optin) continue;  // (a little is static)
+      int rows = 0;
+      for (int l = top; l < nl - 1; ++l) rows += hd->L[l].d.ny + hd->L[l].d.nz;
+      if (rows > CT_MAX_TAB || p.bytes + CT_STATIC > (size_t)optin) continue;
       if (cudaFuncSetAttribute(k_ctail<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               optin - 1024) != cudaSuccess) {
+                               optin - (int)CT_STATIC) != cudaSuccess) {
         cudaGetLastError();
         return MP_OK;
       }
