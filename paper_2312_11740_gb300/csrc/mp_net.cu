@@ -364,6 +364,8 @@ k_conv3d_halo(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
   // iteration (empty past the last stage), so that stage s's gathers are the
   // group NS - 2 behind the newest at the top of iteration s
   int produced = 0, waited_full = 0, committed = 0, waited_done = 0;
+  // (a single-layer call launches this kernel while its weights are still being packed)
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   for (int p = 0; p < NS - 1; ++p) {
     if (produced < nst) {
       produce(produced);
@@ -455,7 +457,7 @@ k_conv3d_halo(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
     // drain (bounded): copies still in flight into shared memory, MMAs still reading it
     for (int s = waited_full; s < produced; ++s) mbar_wait(&full[s % NS], (uint32_t)((s / NS) & 1));
     for (int s = waited_done; s < committed; ++s) mbar_wait(&done[s % NS], (uint32_t)((s / NS) & 1));
-    atomicExch(a.err, 1);
+    *(volatile int *)a.err = 1;
   }
   tc_fence_before();
   __syncthreads();
@@ -659,7 +661,7 @@ k_conv3d_wgrad(const bf16 *__restrict__ xa, const bf16 *__restrict__ xb,
   __syncthreads();
   tc_fence_after();
   if (abort_flag || !ok) {
-    if (tid == 0) atomicExch(err, 1);
+    if (tid == 0) *(volatile int *)err = 1;
   } else {
     const int m = m0 + warp * 32 + lane;
     float4 *dst = reinterpret_cast<float4 *>(partial + ((size_t)blockIdx.y * rows + m) * COUT);
@@ -1226,6 +1228,26 @@ mp_status ws_pool(cudaMemPool_t *out) {
   *out = ws_pools[dev];
   return MP_OK;
 }
+// Status word of a thread's single-layer calls, in mapped host memory: a kernel
+// writes it only when a wait gave up, so a call needs neither a memset nor a copy
+// (each a few us of a call).  The calls wait for their work, so one per thread does.
+struct StatusWord {
+  int *p = nullptr;
+  ~StatusWord() {
+    if (p) cudaFreeHost(p);
+  }
+};
+mp_status status_word(int **out) {
+  static thread_local StatusWord w;
+  if (!w.p && cudaHostAlloc((void **)&w.p, 64, cudaHostAllocPortable) != cudaSuccess) {
+    cudaGetLastError();
+    w.p = nullptr;
+    return MP_ERR_OOM;
+  }
+  *(volatile int *)w.p = 0;
+  *out = w.p;
+  return MP_OK;
+}
 // return what the current device's pool keeps and no call uses
 void ws_trim() {
   int dev = 0;
@@ -1309,7 +1331,7 @@ int take_wait_failure() {
 template <int NC>
 mp_status launch_halo(const ConvGeom &g, const CUtensorMap &ma, const CUtensorMap &mb,
                       const bf16 *xa, const bf16 *wimg, const float *bias, int cout, bf16 *y,
-                      float *y32, int relu, int *err, cudaStream_t st) {
+                      float *y32, int relu, int *err, cudaStream_t st, bool after_pack) {
   const int smem = h_smem_bytes<NC>();
   static bool attr = false;
   if (!attr) {
@@ -1341,20 +1363,33 @@ mp_status launch_halo(const ConvGeom &g, const CUtensorMap &ma, const CUtensorMa
   const long items = (long)a.ntiles * a.nsplit;
   long grid = std::min<long>(items, (long)sm_count() * h_ctas_per_sm<NC>());
   grid = std::max<long>(a.nsplit, grid - grid % a.nsplit);
-  k_conv3d_halo<NC><<<(int)grid, CONV_THREADS, smem, st>>>(ma, mb, a);
-  NCK(cudaGetLastError());
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3(CONV_THREADS);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute la[1];
+  la[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  la[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = la;
+  cfg.numAttrs = after_pack ? 1 : 0;  // after the packing kernel: overlap its end
+  NCK(cudaLaunchKernelEx(&cfg, k_conv3d_halo<NC>, ma, mb, a));
   return MP_OK;
 }
 
 // forward convolution through k_conv3d_halo; wimg packed by k_pack_img for nc_of(cout)
 mp_status conv_fwd(const ConvGeom &g, const CUtensorMap &ma, const CUtensorMap &mb,
                    const bf16 *xa, const bf16 *wimg, const float *bias, int cout, bf16 *y,
-                   float *y32, int relu, int *err, cudaStream_t st) {
+                   float *y32, int relu, int *err, cudaStream_t st, bool after_pack = false) {
   switch (nc_of(cout)) {
-    case 16: return launch_halo<16>(g, ma, mb, xa, wimg, bias, cout, y, y32, relu, err, st);
-    case 32: return launch_halo<32>(g, ma, mb, xa, wimg, bias, cout, y, y32, relu, err, st);
-    case 48: return launch_halo<48>(g, ma, mb, xa, wimg, bias, cout, y, y32, relu, err, st);
-    case 64: return launch_halo<64>(g, ma, mb, xa, wimg, bias, cout, y, y32, relu, err, st);
+    case 16:
+      return launch_halo<16>(g, ma, mb, xa, wimg, bias, cout, y, y32, relu, err, st, after_pack);
+    case 32:
+      return launch_halo<32>(g, ma, mb, xa, wimg, bias, cout, y, y32, relu, err, st, after_pack);
+    case 48:
+      return launch_halo<48>(g, ma, mb, xa, wimg, bias, cout, y, y32, relu, err, st, after_pack);
+    case 64:
+      return launch_halo<64>(g, ma, mb, xa, wimg, bias, cout, y, y32, relu, err, st, after_pack);
   }
   return MP_ERR_INVALID_ARG;
 }
@@ -1583,22 +1618,19 @@ mp_status mp_conv3d_fwd(int nx, int ny, int nz, const void *xa, int ca, int up_a
   CUtensorMap ma, mb;
   NCKS(make_maps(g, (const bf16 *)xa, (const bf16 *)xb, &ma, &mb));
   const size_t nw = (size_t)cout * 27 * g.cin;
-  // one block: the packed weights (a multiple of 16 bytes), then the status word
   cudaMemPool_t pool;
+  int *err = nullptr;
   NCKS(ws_pool(&pool));
-  bf16 *img = nullptr;
-  NCK(cudaMallocFromPoolAsync((void **)&img, nw * sizeof(bf16) + sizeof(int), pool, st));
-  int *err = reinterpret_cast<int *>(img + nw);
-  NCK(cudaMemsetAsync(err, 0, sizeof(int), st));
+  NCKS(status_word(&err));
+  bf16 *img = nullptr;  // packed weights
+  NCK(cudaMallocFromPoolAsync((void **)&img, nw * sizeof(bf16), pool, st));
   k_pack_img<bf16><<<grid_for(nw), 256, 0, st>>>((const bf16 *)w, cout, g.cin, 0, nc_of(cout), img);
   mp_status s = conv_fwd(g, ma, mb, (const bf16 *)xa, img, bias, cout, (bf16 *)y, y32, relu, err,
-                         st);
-  int h = 0;
-  if (s == MP_OK) NCK(cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, st));
+                         st, true);
   NCK(cudaFreeAsync(img, st));
   NCK(cudaStreamSynchronize(st));
   if (s != MP_OK) return s;
-  return h ? MP_ERR_TIMEOUT : MP_OK;
+  return *(volatile int *)err ? MP_ERR_TIMEOUT : MP_OK;
 }
 
 mp_status mp_conv3d_wgrad(int nx, int ny, int nz, const void *xa, int ca, int up_a,
@@ -1611,20 +1643,18 @@ mp_status mp_conv3d_wgrad(int nx, int ny, int nz, const void *xa, int ca, int up
   cudaStream_t st = (cudaStream_t)stream;
   ConvGeom geo{nx, ny, nz, ca, cb, up_a ? 1 : 0, ca + cb};
   cudaMemPool_t pool;
+  int *err = nullptr;
   NCKS(ws_pool(&pool));
-  const size_t np = wgrad_partial_floats(geo, cout);
+  NCKS(status_word(&err));
   float *part = nullptr;
-  NCK(cudaMallocFromPoolAsync((void **)&part, np * sizeof(float) + sizeof(int), pool, st));
-  int *err = reinterpret_cast<int *>(part + np);
-  NCK(cudaMemsetAsync(err, 0, sizeof(int), st));
+  NCK(cudaMallocFromPoolAsync((void **)&part, wgrad_partial_floats(geo, cout) * sizeof(float), pool,
+                              st));
   mp_status s = conv_wgrad(geo, (const bf16 *)xa, (const bf16 *)xb, (const bf16 *)g, cout, part,
                            dw, err, st);
-  int h = 0;
-  if (s == MP_OK) NCK(cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, st));
   NCK(cudaFreeAsync(part, st));
   NCK(cudaStreamSynchronize(st));
   if (s != MP_OK) return s;
-  return h ? MP_ERR_TIMEOUT : MP_OK;
+  return *(volatile int *)err ? MP_ERR_TIMEOUT : MP_OK;
 }
 
 mp_status mp_net_create(mp_net_handle *out, int nx, int ny, int nz, void *stream) {
