@@ -220,8 +220,12 @@ __device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t b
       : "memory");
 }
 
+// Threads of a CTA: one issues the TMA loads and the MMAs; all gather upsampled inputs and run
+// the epilogue (a warp reads the 32 TMEM lanes of its index mod 4; the two
+// halves of the CTA take two output planes each).
+constexpr int HALO_THREADS = 256;
 template <int NC>
-__global__ void __launch_bounds__(CONV_THREADS, h_ctas_per_sm<NC>())
+__global__ void __launch_bounds__(HALO_THREADS, h_ctas_per_sm<NC>())
 k_conv3d_halo(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
               const HaloArgs a) {
   constexpr int NS = h_nstage<NC>();
@@ -238,8 +242,18 @@ k_conv3d_halo(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
   __shared__ __align__(8) uint64_t full[NS], done[NS];
   __shared__ uint32_t tslot;
   __shared__ int abort_flag;
+  // upsampled inputs: per halo voxel its coordinates in the halo (8 bits each) and its
+  // parent's offset from the parent of the tile's origin (tile origins are even)
+  __shared__ int2 htab[HVOX];
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (a.up_a)
+    for (int v = tid; v < HVOX; v += HALO_THREADS) {
+      const int hx = v % HX, hy = (v / HX) % HY, hz = v / (HX * HY);
+      htab[v] = make_int2(hx | hy << 8 | hz << 16,
+                          (((hz - 1) >> 1) * (a.ny >> 1) + ((hy - 1) >> 1)) * (a.nx >> 1) +
+                              ((hx - 1) >> 1));
+    }
   if (tid == 0) {
     for (int s = 0; s < NS; ++s) {
       mbar_init(&full[s]);
@@ -305,12 +319,15 @@ k_conv3d_halo(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
       const int cc = 16 * c + 8 * g;
       if (!(a.up_a && cc < a.ca)) continue;
       uint8_t *dst = st + g * HPLANE;
-      for (int v = tid; v < HVOX; v += CONV_THREADS) {
-        const int hx = v % HX, hy = (v / HX) % HY, hz = v / (HX * HY);
-        const int gx = x0 - 1 + hx, gy = y0 - 1 + hy, gz = z0 - 1 + hz;
-        if (gx >= 0 && gy >= 0 && gz >= 0 && gx < a.nx && gy < a.ny && gz < a.nz)
-          cp_async16(dst + v * 16,
-                     a.xa + (((size_t)(gz >> 1) * any + (gy >> 1)) * anx + (gx >> 1)) * a.ca + cc);
+      const bf16 *src =
+          a.xa + (((size_t)(z0 >> 1) * any + (y0 >> 1)) * anx + (x0 >> 1)) * a.ca + cc;
+#pragma unroll 3
+      for (int v = tid; v < HVOX; v += HALO_THREADS) {
+        const int2 h = htab[v];
+        const int gx = x0 - 1 + (h.x & 255), gy = y0 - 1 + (h.x >> 8 & 255), gz = z0 - 1 + (h.x >> 16);
+        if ((unsigned)gx < (unsigned)a.nx && (unsigned)gy < (unsigned)a.ny &&
+            (unsigned)gz < (unsigned)a.nz)
+          cp_async16(dst + v * 16, src + (long)h.y * a.ca);
         else
           *reinterpret_cast<uint4 *>(dst + v * 16) = make_uint4(0, 0, 0, 0);
       }
@@ -322,19 +339,19 @@ k_conv3d_halo(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
     int x0, y0, z0;
     tile_origin(lt, x0, y0, z0);
     tc_fence_after();
-    const int r = warp * 32 + lane;
+    const int r = (warp & 3) * 32 + lane;
     const int gx = x0 + (r & 7), gy = y0 + (r >> 3);
     const uint32_t acc = (uint32_t)((lt & 1) * HT_Z * NC);
-    const int co0 = split * NC;
+    const int co0 = split * NC, zhalf = (warp >> 2) * (HT_Z / 2);
 #pragma unroll 1
-    for (int zp = 0; zp < HT_Z; ++zp) {
+    for (int zp = zhalf; zp < zhalf + HT_Z / 2; ++zp) {
       const int gz = z0 + zp;
       const bool inside = gx < a.nx && gy < a.ny && gz < a.nz;
       const size_t vox = ((size_t)gz * a.ny + gy) * a.nx + gx;
 #pragma unroll
       for (int c0 = 0; c0 < NC; c0 += 16) {
         float v[16];
-        tmem_ld16(taddr + ((uint32_t)(warp * 32) << 16) + acc + zp * NC + c0, v);
+        tmem_ld16(taddr + ((uint32_t)((warp & 3) * 32) << 16) + acc + zp * NC + c0, v);
         if (inside) {
 #pragma unroll
           for (int q = 0; q < 16; ++q) {
@@ -378,7 +395,7 @@ k_conv3d_halo(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
     const int buf = s % NS;
     cp_async_wait<NS - 2>();  // this thread's gathers of stage s have landed ...
     fence_async_smem();       // ... and are visible to the tensor core's reads
-    // one thread polls the barriers (127 pollers would load the shared-memory
+    // one thread polls the barriers (255 pollers would load the shared-memory
     // pipe that feeds the tensor core); the others wait at the CTA barrier
     if (tid == 0) {
       if (!(s == 0 && a.fail_first) && mbar_wait(&full[buf], (uint32_t)((s / NS) & 1)))
@@ -1365,7 +1382,7 @@ mp_status launch_halo(const ConvGeom &g, const CUtensorMap &ma, const CUtensorMa
   grid = std::max<long>(a.nsplit, grid - grid % a.nsplit);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3(CONV_THREADS);
+  cfg.blockDim = dim3(HALO_THREADS);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute la[1];
