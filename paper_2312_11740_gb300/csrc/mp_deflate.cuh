@@ -555,12 +555,42 @@ struct DeflCoef {
   unsigned *done;
 };
 
+// The band's rows of A Z, once per geometry: a band cell that touches one
+// component (almost all do) gets that component and its (A z_j)_c; one that
+// touches several ROW_MANY, none ROW_NONE.  A projection then reads 12 bytes of
+// a cell's row instead of gathering its six faces and seven components, and does
+// one FP64 product per cell instead of seven products and sums (this part's FP64
+// rate bounds the pass).
+constexpr int ROW_NONE = -1, ROW_MANY = -2;
+template <typename F>
+__global__ void k_defl_rows(const int *__restrict__ band, int nband, const int *__restrict__ comp,
+                            const F *__restrict__ bx, const F *__restrict__ by,
+                            const F *__restrict__ bz, Dims d, int *__restrict__ row_k,
+                            double *__restrict__ row_w) {
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < nband; e += gridDim.x * blockDim.x) {
+    int ks[7], k = ROW_NONE;
+    double ws[7], w = 0.0;
+    band_row(bx, by, bz, comp, d, (size_t)band[e], ks, ws);
+#pragma unroll
+    for (int f = 0; f < 7; ++f)
+      if (ks[f] >= 0) {
+        if (k == ROW_NONE) k = ks[f];
+        if (ks[f] != k) k = ROW_MANY;
+        w += ws[f];
+      }
+    row_k[e] = k;
+    row_w[e] = w;
+  }
+}
+
 // s_j = sum over the band of (A z_j)_c v_c  ( = (A Z)^T v ), scale from the band
-// maximum of |v| (6 faces of at most beta_max each), then the coefficients
+// maximum of |v| (6 faces of at most beta_max each), then the coefficients.
+// row_k, row_w: k_defl_rows' result, or null (a band too large to keep them).
 template <typename T, typename F>
 __global__ void k_defl_azt(const int *__restrict__ band, int nband, const int *__restrict__ comp,
                            const F *__restrict__ bx, const F *__restrict__ by,
                            const F *__restrict__ bz, Dims d, const T *__restrict__ v,
+                           const int *__restrict__ row_k, const double *__restrict__ row_w,
                            double beta_max, unsigned long long *acc, DeflCoef dc) {
   griddep_wait();
   const double vmax = __longlong_as_double((long long)*dc.mx);
@@ -570,18 +600,35 @@ __global__ void k_defl_azt(const int *__restrict__ band, int nband, const int *_
   FxCarry carry;
   for (int e0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31); e0 < nband; e0 += stride) {
     const int e = e0 + (threadIdx.x & 31);
-    int ks[7];
-    double ws[7];
-#pragma unroll
-    for (int f = 0; f < 7; ++f) ks[f] = -1, ws[f] = 0.0;
+    int k = ROW_NONE;
+    double val = 0.0;
+    size_t c = 0;
     if (e < nband) {
-      const size_t c = (size_t)band[e];
-      band_row(bx, by, bz, comp, d, c, ks, ws);
-      const double vc = (double)v[c];
-#pragma unroll
-      for (int f = 0; f < 7; ++f) ws[f] *= vc;
+      c = (size_t)band[e];
+      k = row_k ? row_k[e] : ROW_MANY;
+      if (k >= 0) val = row_w[e] * (double)v[c];
     }
-    fx_add_warp(acc, ks, ws, scale, carry);
+    if (__any_sync(0xffffffffu, k == ROW_MANY)) {  // the warp's cells from their faces
+      int ks[7];
+      double ws[7];
+#pragma unroll
+      for (int f = 0; f < 7; ++f) ks[f] = -1, ws[f] = 0.0;
+      if (e < nband) {
+        band_row(bx, by, bz, comp, d, c, ks, ws);
+        const double vc = (double)v[c];
+#pragma unroll
+        for (int f = 0; f < 7; ++f) ws[f] *= vc;
+      }
+      fx_add_warp(acc, ks, ws, scale, carry);
+      continue;
+    }
+    // the contributions to the warp's leading component in a fixed shuffle tree, the
+    // others per lane (as fx_add_warp)
+    const unsigned has = __ballot_sync(0xffffffffu, k >= 0);
+    if (has == 0u) continue;
+    const int lead = __shfl_sync(0xffffffffu, k, __ffs(has) - 1);
+    carry.add(acc, lead, warp_sum(k == lead ? val : 0.0), scale);
+    if (k >= 0 && k != lead) fx_add(acc, k, val, scale);
   }
   carry.flush(acc, scale);
   if (!last_block(dc.done)) return;

@@ -153,6 +153,9 @@ struct mp_poisson {
   double *einv = nullptr, *coef = nullptr;
   float *coef32 = nullptr;
   unsigned long long *acc_a = nullptr, *acc_b = nullptr, *acc_ztb = nullptr, *dmax = nullptr;
+  int *row_k = nullptr;     // the band's rows of A Z (up to row_cap cells)
+  double *row_w = nullptr;
+  size_t row_cap = 0;
   int *hint = nullptr;  // pinned host copy of dint
   mp_net_handle net = nullptr;  // learned initial guess (initial_guess = 2)
   int net_factor = 1;           // solver grid / network grid (1 or 2)
@@ -745,6 +748,9 @@ mp_status deflation_setup(mp_poisson *hd) {
          hd->comp, l0.bx, l0.by, l0.bz, l0.d, hd->acc_a, escale);
   LAUNCH(hd, K_DEFL, 0, m * 8.0, k_defl_einv, (m + 255) / 256, 256, m, hd->acc_a, escale,
          hd->einv);
+  if ((size_t)nband <= hd->row_cap)
+    LAUNCH(hd, K_DEFL, 0, nband * 72.0, k_defl_rows<double>, VEC_BLOCKS, VEC_THREADS, hd->band, nband,
+           hd->comp, l0.bx, l0.by, l0.bz, l0.d, hd->row_k, hd->row_w);
   CKS(launch_ok());
   hd->defl_m = m;
   hd->defl_nband = nband;
@@ -784,9 +790,11 @@ mp_status defl_coef(mp_poisson *hd, const T *v, const F *bx, const F *by, const 
   const DeflCoef dc{m, with_ztb ? hd->acc_ztb : nullptr, hd->ztb_scale, hd->einv,
                     hd->coef, hd->coef32, hd->dmax, hd->done + 1};
   auto kazt = k_defl_azt<T, F>;
+  const bool rows = (size_t)nb <= hd->row_cap;
   LAUNCH_PDL(hd, K_DEFL, 0, nb * (7.0 * sizeof(T) + 3.0 * sizeof(F) + 28.0) + m * 16.0, kazt,
-             VEC_BLOCKS, VEC_THREADS, 0, hd->band, nb, hd->comp, bx, by, bz, l0.d, v, hd->beta_max,
-             acc, dc);
+             VEC_BLOCKS, VEC_THREADS, 0, hd->band, nb, hd->comp, bx, by, bz, l0.d, v,
+             rows ? (const int *)hd->row_k : nullptr, rows ? (const double *)hd->row_w : nullptr,
+             hd->beta_max, acc, dc);
   return launch_ok();
 }
 
@@ -1696,6 +1704,9 @@ mp_status create(mp_poisson *hd, mp_grid g, double h, const mp_bc bc[3]) {
   CKS(dalloc(hd, &hd->lab, n));
   CKS(dalloc(hd, &hd->comp, n));
   CKS(dalloc(hd, &hd->band, n));
+  hd->row_cap = n / 8 + 65536;
+  CKS(dalloc(hd, &hd->row_k, hd->row_cap));
+  CKS(dalloc(hd, &hd->row_w, hd->row_cap));
   hd->tcap = (int)std::min<size_t>(n / 64 + 1024, (size_t)1 << 30);
   CKS(dalloc(hd, &hd->troots, (size_t)hd->tcap));
   CKS(dalloc(hd, &hd->cnt, nblk));
