@@ -276,12 +276,17 @@ __global__ void k_rank_roots(const int *__restrict__ roots, const int *__restric
   }
 }
 
-// comp[c] = id of c's root (roots already hold their id), -1 for liquid
-__global__ void k_comp_from_roots(const int *__restrict__ lab, int *comp, size_t n) {
-  for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < n;
-       c += (size_t)gridDim.x * blockDim.x) {
-    const int r = lab[c];
-    comp[c] = r < 0 ? -1 : comp[r];
+// comp[c] = id of c's root (roots already hold their id), -1 for liquid; mask: one
+// bit per cell, set in gas (a projection reads comp only where it is)
+__global__ void k_comp_from_roots(const int *__restrict__ lab, int *comp, size_t n,
+                                  unsigned *__restrict__ mask) {
+  // (whole warps, blocks of a multiple of 32 cells: lane 0's cell starts a mask word)
+  for (size_t c0 = blockIdx.x * (size_t)blockDim.x; c0 < n; c0 += (size_t)gridDim.x * blockDim.x) {
+    const size_t c = c0 + threadIdx.x;
+    const int r = c < n ? lab[c] : -1;
+    if (c < n) comp[c] = r < 0 ? -1 : comp[r];
+    const unsigned m = __ballot_sync(0xffffffffu, r >= 0);
+    if ((threadIdx.x & 31) == 0 && c < n) mask[c >> 5] = m;
   }
 }
 
@@ -757,7 +762,7 @@ struct IVec16<2> {
 template <typename T>
 __global__ void __launch_bounds__(VEC_THREADS, 4)
 k_dot_zdefl(const T *__restrict__ r, T *__restrict__ z, const int *__restrict__ comp,
-            const T *__restrict__ coef, size_t n, Fin fin) {
+            const unsigned *__restrict__ mask, const T *__restrict__ coef, size_t n, Fin fin) {
   griddep_wait();
   using VT = Vec16<T>;
   using V = typename VT::V;
@@ -774,18 +779,17 @@ k_dot_zdefl(const T *__restrict__ r, T *__restrict__ z, const int *__restrict__ 
     for (size_t e = tid; e < nv; e += stride) {
       const V x = rv[e];
       V y = zv[e];
-      const typename IVec16<W>::V ce = cv[e];
-      bool any = false;
+      if ((mask[e * W >> 5] >> (e * W & 31)) & ((1u << W) - 1u)) {  // gas among the W cells
+        const typename IVec16<W>::V ce = cv[e];
 #pragma unroll
-      for (int q = 0; q < W; ++q) {
-        const int m = IVec16<W>::at(ce, q);
-        if (m >= 0) {
-          VT::set(y, q, VT::at(y, q) - coef[m]);
-          any = true;
+        for (int q = 0; q < W; ++q) {
+          const int m = IVec16<W>::at(ce, q);
+          if (m >= 0) VT::set(y, q, VT::at(y, q) - coef[m]);
         }
-        acc = fma(VT::at(x, q), VT::at(y, q), acc);
+        zv[e] = y;
       }
-      if (any) zv[e] = y;
+#pragma unroll
+      for (int q = 0; q < W; ++q) acc = fma(VT::at(x, q), VT::at(y, q), acc);
     }
     done = nv * W;
   }

@@ -1097,18 +1097,30 @@ __global__ void k_apply_dot(const T *__restrict__ dv, T *__restrict__ q, const T
 
 // q = At d (FP32 difference form, op_at's arithmetic per cell) and per-block
 // partials of d.q, with 16-byte rows (nx a multiple of 4): a thread owns a
-// 4-cell x-chunk in each of its zper planes and loads it as vectors.
+// 4-cell x-chunk and marches its zper planes, keeping the chunk's d of three
+// planes and the z faces between them, so a plane's own chunk is loaded once.
 // XPBY: the CG direction update d = z + beta d (k_xpby's operation, d = z on
 // the first iteration) fused in: every value of d the stencil needs is formed
 // from z and the old direction dv, and the thread's own chunk of the new
 // direction is stored to dnew (a second buffer: other blocks still read dv).
-__device__ __forceinline__ float4 xpby4(const float *__restrict__ z, const float *__restrict__ d,
-                                        size_t c, float beta, int first) {
-  const float4 zz = *reinterpret_cast<const float4 *>(z + c);
-  if (first) return zz;
-  const float4 dd = *reinterpret_cast<const float4 *>(d + c);
-  return make_float4(fmaf(beta, dd.x, zz.x), fmaf(beta, dd.y, zz.y), fmaf(beta, dd.z, zz.z),
-                     fmaf(beta, dd.w, zz.w));
+// e (XPBY, may be null): the pending solution update e += alpha dv of the previous
+// iteration, taken here because dv is already in registers (one read of d less
+// than in a pass of its own).
+// What bounds it: HBM.  256^3, XPBY with e: 36 B/cell in 104 us (5.7 TB/s); without
+// e, reloading the planes, 28 B/cell took 96 us.
+struct XpbyChunk {
+  float4 d, old;  // the new direction, and dv's values
+};
+__device__ __forceinline__ XpbyChunk xpby4(const float *__restrict__ z, const float *__restrict__ d,
+                                           size_t c, float beta, int first) {
+  XpbyChunk r;
+  r.d = *reinterpret_cast<const float4 *>(z + c);
+  r.old = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (first) return r;
+  r.old = *reinterpret_cast<const float4 *>(d + c);
+  r.d = make_float4(fmaf(beta, r.old.x, r.d.x), fmaf(beta, r.old.y, r.d.y),
+                    fmaf(beta, r.old.z, r.d.z), fmaf(beta, r.old.w, r.d.w));
+  return r;
 }
 template <bool XPBY>
 __global__ void __launch_bounds__(BX * BY)
@@ -1116,12 +1128,13 @@ k_apply_dot4(const float *__restrict__ dv, float *__restrict__ q, const float *_
              const float *__restrict__ by, const float *__restrict__ bz,
              const float *__restrict__ dd32, Dims d, int zper, Fin fin,
              const float *__restrict__ z, float *__restrict__ dnew,
-             const double *__restrict__ scal, int first) {
+             const double *__restrict__ scal, int first, float *__restrict__ e) {
   griddep_wait();
   const float beta = XPBY && !first ? (float)scal[S_BETA] : 0.f;
-  auto ld4 = [&](size_t c) -> float4 {
+  const float alpha = XPBY && e ? (float)scal[S_ALPHA] : 0.f;  // (the previous iteration's)
+  auto ld4 = [&](size_t c) -> XpbyChunk {
     if (XPBY) return xpby4(z, dv, c, beta, first);
-    return *reinterpret_cast<const float4 *>(dv + c);
+    return XpbyChunk{*reinterpret_cast<const float4 *>(dv + c), make_float4(0.f, 0.f, 0.f, 0.f)};
   };
   auto ld1 = [&](size_t c) -> float {
     if (XPBY) return first ? z[c] : fmaf(beta, dv[c], z[c]);
@@ -1130,39 +1143,52 @@ k_apply_dot4(const float *__restrict__ dv, float *__restrict__ q, const float *_
   const int t = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y;
   const int k0 = blockIdx.z * zper, k1 = min(d.nz, k0 + zper);
   float acc = 0.f;
-  if (t < (d.nx >> 2) && j < d.ny)
+  if (t < (d.nx >> 2) && j < d.ny && k0 < k1) {
+    const int i0 = 4 * t;
+    float4 xzl = ld4(at(d, i0, j, wlo(k0, d.nz))).d;
+    XpbyChunk cur = ld4(at(d, i0, j, k0));
+    float4 fz = *reinterpret_cast<const float4 *>(bz + at(d, i0, j, k0));
     for (int k = k0; k < k1; ++k) {
-      const int i0 = 4 * t;
       const size_t c0 = at(d, i0, j, k);
       const size_t cyl = at(d, i0, wlo(j, d.ny), k), cyh = at(d, i0, whi(j, d.ny), k);
-      const size_t czl = at(d, i0, j, wlo(k, d.nz)), czh = at(d, i0, j, whi(k, d.nz));
+      const size_t czh = at(d, i0, j, whi(k, d.nz));
       const size_t ce = at(d, whi(i0 + 3, d.nx), j, k);
-      const float4 xc = ld4(c0);
-      const float4 xyl = ld4(cyl), xyh = ld4(cyh), xzl = ld4(czl), xzh = ld4(czh);
+      const XpbyChunk up = ld4(czh);
+      const float4 xc = cur.d, xzh = up.d;
+      const float4 xyl = ld4(cyl).d, xyh = ld4(cyh).d;
       if (XPBY) *reinterpret_cast<float4 *>(dnew + c0) = xc;
+      if (XPBY && e) {
+        float4 ev = *reinterpret_cast<float4 *>(e + c0);
+        ev = make_float4(fmaf(alpha, cur.old.x, ev.x), fmaf(alpha, cur.old.y, ev.y),
+                         fmaf(alpha, cur.old.z, ev.z), fmaf(alpha, cur.old.w, ev.w));
+        *reinterpret_cast<float4 *>(e + c0) = ev;
+      }
       const float4 fx = *reinterpret_cast<const float4 *>(bx + c0);
       const float4 fy = *reinterpret_cast<const float4 *>(by + c0);
       const float4 fyh = *reinterpret_cast<const float4 *>(by + cyh);
-      const float4 fz = *reinterpret_cast<const float4 *>(bz + c0);
       const float4 fzh = *reinterpret_cast<const float4 *>(bz + czh);
       const float fxe = bx[ce], xp = ld1(ce), xm = ld1(at(d, wlo(i0, d.nx), j, k));
       float4 out;
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float v = f4_at(xc, e);
-        const float x_l = e > 0 ? f4_at(xc, e - 1) : xm, x_h = e < 3 ? f4_at(xc, e + 1) : xp;
-        float s = f4_at(fx, e) * (x_l - v);
-        s = fmaf(e < 3 ? f4_at(fx, e + 1) : fxe, x_h - v, s);
-        s = fmaf(f4_at(fy, e), f4_at(xyl, e) - v, s);
-        s = fmaf(f4_at(fyh, e), f4_at(xyh, e) - v, s);
-        s = fmaf(f4_at(fz, e), f4_at(xzl, e) - v, s);
-        s = fmaf(f4_at(fzh, e), f4_at(xzh, e) - v, s);
-        if (dd32) s = fmaf(-dd32[c0 + e], v, s);
-        if (e == 0) out.x = s; else if (e == 1) out.y = s; else if (e == 2) out.z = s; else out.w = s;
+      for (int u = 0; u < 4; ++u) {
+        const float v = f4_at(xc, u);
+        const float x_l = u > 0 ? f4_at(xc, u - 1) : xm, x_h = u < 3 ? f4_at(xc, u + 1) : xp;
+        float s = f4_at(fx, u) * (x_l - v);
+        s = fmaf(u < 3 ? f4_at(fx, u + 1) : fxe, x_h - v, s);
+        s = fmaf(f4_at(fy, u), f4_at(xyl, u) - v, s);
+        s = fmaf(f4_at(fyh, u), f4_at(xyh, u) - v, s);
+        s = fmaf(f4_at(fz, u), f4_at(xzl, u) - v, s);
+        s = fmaf(f4_at(fzh, u), f4_at(xzh, u) - v, s);
+        if (dd32) s = fmaf(-dd32[c0 + u], v, s);
+        if (u == 0) out.x = s; else if (u == 1) out.y = s; else if (u == 2) out.z = s; else out.w = s;
         acc = fmaf(s, v, acc);
       }
       *reinterpret_cast<float4 *>(q + c0) = out;
+      xzl = xc;
+      cur = up;
+      fz = fzh;
     }
+  }
   block_finish(block_sum((double)acc), block_linear_id(), fin);
 }
 
@@ -1263,8 +1289,9 @@ k_dot(const T *__restrict__ a, const T *__restrict__ b, size_t n, Fin fin) {
   block_finish(block_sum((double)acc), blockIdx.x, fin);
 }
 
-// x += alpha d; r -= alpha q; partial r.r
-template <typename T>
+// x += alpha d; r -= alpha q; partial r.r.  X false: only r (the update of x is
+// left to the next k_apply_dot4 or k_add_f32).
+template <typename T, bool X>
 __global__ void __launch_bounds__(VEC_THREADS, 4)
 k_axpy2(T *__restrict__ x, T *__restrict__ r, const T *__restrict__ dv,
                         const T *__restrict__ q, size_t n, const double *__restrict__ scal, Fin fin) {
@@ -1277,27 +1304,41 @@ k_axpy2(T *__restrict__ x, T *__restrict__ r, const T *__restrict__ dv,
   const size_t tid = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
   const size_t stride = (size_t)gridDim.x * blockDim.x;
   size_t done = 0;
-  if (aligned16(x, r, dv, q)) {
+  if (X ? aligned16(x, r, dv, q) : aligned16(r, q)) {
     const size_t nv = n / W;
     V *xv = reinterpret_cast<V *>(x), *rv = reinterpret_cast<V *>(r);
     const V *dvv = reinterpret_cast<const V *>(dv), *qv = reinterpret_cast<const V *>(q);
-    for (size_t e = tid; e < nv; e += stride) {
-      V xe = xv[e], re = rv[e];
-      const V de = dvv[e], qe = qv[e];
+    // U vectors at a time (both loaded before either is stored) in the order of one
+    // at a time: without x there are two loads per vector, too few in flight
+    constexpr int U = X ? 1 : 4;
+    for (size_t e0 = tid; e0 < nv; e0 += U * stride) {
+      V xe[U], de[U], re[U], qe[U];
 #pragma unroll
-      for (int k = 0; k < W; ++k) {
-        VT::set(xe, k, fma(alpha, VT::at(de, k), VT::at(xe, k)));
-        const T rk = fma(-alpha, VT::at(qe, k), VT::at(re, k));
-        VT::set(re, k, rk);
-        acc = fma(rk, rk, acc);
+      for (int u = 0; u < U; ++u) {
+        const size_t e = e0 + u * stride;
+        if (u > 0 && e >= nv) break;
+        re[u] = rv[e], qe[u] = qv[e];
+        if (X) xe[u] = xv[e], de[u] = dvv[e];
       }
-      xv[e] = xe;
-      rv[e] = re;
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const size_t e = e0 + u * stride;
+        if (u > 0 && e >= nv) break;
+#pragma unroll
+        for (int k = 0; k < W; ++k) {
+          if (X) VT::set(xe[u], k, fma(alpha, VT::at(de[u], k), VT::at(xe[u], k)));
+          const T rk = fma(-alpha, VT::at(qe[u], k), VT::at(re[u], k));
+          VT::set(re[u], k, rk);
+          acc = fma(rk, rk, acc);
+        }
+        if (X) xv[e] = xe[u];
+        rv[e] = re[u];
+      }
     }
     done = nv * W;
   }
   for (size_t e = done + tid; e < n; e += stride) {
-    x[e] = fma(alpha, dv[e], x[e]);
+    if (X) x[e] = fma(alpha, dv[e], x[e]);
     T rv = fma(-alpha, q[e], r[e]);
     r[e] = rv;
     acc = fma(rv, rv, acc);
@@ -1344,17 +1385,24 @@ __global__ void k_add(T *__restrict__ x, const T *__restrict__ y, size_t n) {
     x[e] += y[e];
 }
 
-// x64 += e32, then e32 = 0 (accumulation of an FP32 correction in FP64)
-// x += (double) e, e = 0: four cells per step (16-byte e, two 16-byte x
-// accesses) when both arrays start 16-byte aligned (x may be a caller's
-// view), then the tail
-__global__ void k_add_f32(double *__restrict__ x, float *__restrict__ e, size_t n) {
-  const bool vec = ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(e)) & 15) == 0;
+// x64 += e32, then e32 = 0 (accumulation of an FP32 correction in FP64): four cells
+// per step (16-byte e, two 16-byte x accesses) when the arrays start 16-byte aligned
+// (x may be a caller's view), then the tail.  dv (may be null): the pending e +=
+// alpha dv comes first.
+__global__ void k_add_f32(double *__restrict__ x, float *__restrict__ e, size_t n,
+                          const float *__restrict__ dv, const double *__restrict__ scal) {
+  const bool vec = aligned16(x, e, dv);
+  const float alpha = dv ? (float)scal[S_ALPHA] : 0.f;
   const size_t n4 = vec ? n / 4 : 0, stride = (size_t)gridDim.x * blockDim.x;
   for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < n4; q += stride) {
     float4 *ep = reinterpret_cast<float4 *>(e) + q;
     double2 *xp = reinterpret_cast<double2 *>(x) + 2 * q;
-    const float4 v = *ep;
+    float4 v = *ep;
+    if (dv) {
+      const float4 d = reinterpret_cast<const float4 *>(dv)[q];
+      v = make_float4(fmaf(alpha, d.x, v.x), fmaf(alpha, d.y, v.y), fmaf(alpha, d.z, v.z),
+                      fmaf(alpha, d.w, v.w));
+    }
     double2 a = xp[0], c = xp[1];
     a.x += (double)v.x;
     a.y += (double)v.y;
@@ -1365,7 +1413,7 @@ __global__ void k_add_f32(double *__restrict__ x, float *__restrict__ e, size_t 
     *ep = make_float4(0.f, 0.f, 0.f, 0.f);
   }
   for (size_t k = 4 * n4 + blockIdx.x * (size_t)blockDim.x + threadIdx.x; k < n; k += stride) {
-    x[k] += (double)e[k];
+    x[k] += (double)(dv ? fmaf(alpha, dv[k], e[k]) : e[k]);
     e[k] = 0.f;
   }
 }

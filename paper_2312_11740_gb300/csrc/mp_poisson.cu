@@ -136,6 +136,7 @@ struct mp_poisson {
   int nc = 0;
   // reductions
   double *partial = nullptr, *scal = nullptr, *scal_h = nullptr;
+  int apply_zper = 1;        // planes per thread of k_apply_dot4
   unsigned *done = nullptr;  // blocks finished of the running reduction, and of a projection's sums
   int npart = 0;
   double bnorm = 0.0;
@@ -153,6 +154,7 @@ struct mp_poisson {
   double *einv = nullptr, *coef = nullptr;
   float *coef32 = nullptr;
   unsigned long long *acc_a = nullptr, *acc_b = nullptr, *acc_ztb = nullptr, *dmax = nullptr;
+  unsigned *gmask = nullptr;  // gas cells, one bit each
   int *row_k = nullptr;     // the band's rows of A Z (up to row_cap cells)
   double *row_w = nullptr;
   size_t row_cap = 0;
@@ -233,6 +235,23 @@ Dims chunk_dims(const Dims &d) {
   Dims q = d;
   q.nx = d.nx / 4;
   return q;
+}
+// Planes per thread of k_apply_dot4, which loads a plane more on either side of
+// its own: the least (waves of resident blocks) x (planes + 2).  slots: blocks
+// resident at once.
+int zper_apply(const Dims &dq, int slots) {
+  const long plane = (long)((dq.nx + BX - 1) / BX) * ((dq.ny + BY - 1) / BY);
+  long best = 0;
+  int zper = 1;
+  for (int zp = 1; zp <= dq.nz; ++zp) {
+    const long blocks = plane * ((dq.nz + zp - 1) / zp);
+    const long cost = (blocks + slots - 1) / slots * (zp + 2);
+    if (best == 0 || cost < best) best = cost, zper = zp;
+  }
+  return zper;
+}
+dim3 apply_grid(const Dims &dq, int zper) {
+  return dim3((dq.nx + BX - 1) / BX, (dq.ny + BY - 1) / BY, (dq.nz + zper - 1) / zper);
 }
 int zblocks(const Dims &d) {
   dim3 g = zgrid(d);
@@ -727,7 +746,7 @@ mp_status deflation_setup(mp_poisson *hd) {
          hd->roots, hd->dint, lim, (const int *)(hd->dint + 3), hd->tcap);
   LAUNCH(hd, K_DEFL_LABEL, 0, DEFL_MAX * 8.0, k_rank_roots, 1, 1024, hd->roots, hd->dint, hd->comp);
   LAUNCH(hd, K_DEFL_LABEL, 0, n * 12.0, k_comp_from_roots, VEC_BLOCKS, VEC_THREADS, hd->lab, hd->comp,
-         n);
+         n, hd->gmask);
   CK(cudaMemcpyAsync(hd->hint, hd->dint, 4 * sizeof(int), cudaMemcpyDeviceToHost, hd->st));
   CK(cudaStreamSynchronize(hd->st));
   const int m = hd->hint[0];
@@ -858,7 +877,8 @@ mp_status defl_rz(mp_poisson *hd, const T *r, T *z, const F *bx, const F *by, co
   else
     coef = hd->coef32;
   LAUNCH_PDL(hd, K_DEFL_DOT, 0, hd->n * (3.0 * sizeof(T) + 4.0), k_dot_zdefl<T>, VEC_BLOCKS,
-             VEC_THREADS, 0, r, z, (const int *)hd->comp, coef, hd->n, fin(hd, op, S_RZ, 0.0, false));
+             VEC_THREADS, 0, r, z, (const int *)hd->comp, (const unsigned *)hd->gmask, coef, hd->n,
+             fin(hd, op, S_RZ, 0.0, false));
   return launch_ok();
 }
 
@@ -908,7 +928,8 @@ mp_status pcg(mp_poisson *hd, T *x, T *r, T *z, T *dv, T *q, double tol_abs, int
                k_apply_dot<T>, zgrid(l0.d), kBlock, 0, (const T *)dv, q, (const T *)bx,
                (const T *)by, (const T *)bz, (const T *)diag, (const T *)nullptr, l0.d,
                zper_of(l0.d), fin(hd, OP_ALPHA, 0, 0.0, false));
-    LAUNCH_PDL(hd, kid<T>(K_AXPY64, K_AXPY32), 0, 6.0 * nsz, k_axpy2<T>, VEC_BLOCKS, VEC_THREADS,
+    auto kaxpy = k_axpy2<T, true>;
+    LAUNCH_PDL(hd, kid<T>(K_AXPY64, K_AXPY32), 0, 6.0 * nsz, kaxpy, VEC_BLOCKS, VEC_THREADS,
                0, x, r, (const T *)dv, (const T *)q, n, (const double *)hd->scal,
                fin(hd, OP_STORE, S_RR, 0.0, true));
     ++it;
@@ -982,12 +1003,15 @@ mp_status pcg_mixed(mp_poisson *hd, double *p, double rn, double tol_abs, int ma
     CKS(project_true(rn, p_zero ? 1 : 0));
   }
   double rn_rep = rn, rec = rn;
+  bool pending = false;  // e += alpha d of the last iteration still to be added
   CK(cudaMemsetAsync(e, 0, n * sizeof(float), hd->st));
   while (true) {
     if (since > 0 && (rec <= std::fmax(o.inner_rtol * rn_rep, 0.5 * tol_abs) ||
                       since >= o.inner_max || it >= maxit)) {
       // reliable update: p += e32 (e32 = 0), r32 = bt - At p from FP64
-      LAUNCH(hd, K_ADDF32, 0, n * 24.0, k_add_f32, VEC_BLOCKS, VEC_THREADS, p, e, n);
+      LAUNCH(hd, K_ADDF32, 0, n * (pending ? 28.0 : 24.0), k_add_f32, VEC_BLOCKS, VEC_THREADS, p, e, n,
+             pending ? (const float *)dv : nullptr, (const double *)hd->scal);
+      pending = false;
       if (defl) {
         CKS(project_true(rn, 0));
       } else {
@@ -1018,11 +1042,11 @@ mp_status pcg_mixed(mp_poisson *hd, double *p, double rn, double tol_abs, int ma
       // d_new = z + beta d in the operator's loads, stored to the other buffer
       const Dims dq = chunk_dims(l0.d);
       float *dnew = dv == hd->d32 ? hd->d32b : hd->d32;
-      LAUNCH_PDL(hd, K_APPLY32, 0, (it == 0 ? 6.0 : 7.0) * nsz, k_apply_dot4<true>, zgrid(dq),
+      LAUNCH_PDL(hd, K_APPLY32, 0, (it == 0 ? 6.0 : pending ? 9.0 : 7.0) * nsz, k_apply_dot4<true>, apply_grid(dq, hd->apply_zper),
                  kBlock, 0, (const float *)dv, q, (const float *)l0.bx32,
                  (const float *)l0.by32, (const float *)l0.bz32, (const float *)l0.dd32, l0.d,
-                 zper_of(dq), fin(hd, OP_ALPHA, 0, 0.0, false), (const float *)z, dnew, (const double *)hd->scal,
-                 it == 0 ? 1 : 0);
+                 hd->apply_zper, fin(hd, OP_ALPHA, 0, 0.0, false), (const float *)z, dnew, (const double *)hd->scal,
+                 it == 0 ? 1 : 0, pending ? e : (float *)nullptr);
       dv = dnew;
     } else {
       LAUNCH(hd, K_XPBY32, 0, (it == 0 ? 2.0 : 3.0) * nsz, k_xpby<float>, VEC_BLOCKS, VEC_THREADS,
@@ -1031,8 +1055,13 @@ mp_status pcg_mixed(mp_poisson *hd, double *p, double rn, double tol_abs, int ma
              l0.bx32, l0.by32, l0.bz32, (float *)nullptr, (const float *)l0.dd32, l0.d,
              zper_of(l0.d), fin(hd, OP_ALPHA, 0, 0.0, false));
     }
-    LAUNCH_PDL(hd, K_AXPY32, 0, 6.0 * nsz, k_axpy2<float>, VEC_BLOCKS, VEC_THREADS, 0, e, r,
-               (const float *)dv, (const float *)q, n, (const double *)hd->scal, fin(hd, OP_STORE, S_RR, 0.0, true));
+    // with the fused form the update e += alpha d waits for the next iteration's
+    // operator (or the next reliable update), which reads this d anyway
+    pending = fused;
+    auto kaxpy = fused ? k_axpy2<float, false> : k_axpy2<float, true>;
+    LAUNCH_PDL(hd, K_AXPY32, 0, (fused ? 3.0 : 6.0) * nsz, kaxpy, VEC_BLOCKS, VEC_THREADS, 0, e, r,
+               (const float *)dv, (const float *)q, n, (const double *)hd->scal,
+               fin(hd, OP_STORE, S_RR, 0.0, true));
     ++it;
     ++since;
     CKS(read_scalars(hd));
@@ -1178,10 +1207,10 @@ mp_status solve_assembled(mp_poisson *hd, double *p, double tol, std::vector<dou
       LAUNCH(hd, K_RESIDMIX, 0, hd->n * 12.0, k_to_f32_norm, VEC_BLOCKS, VEC_THREADS, p, hd->z32,
              hd->n, partials(hd));
       const Dims dq = chunk_dims(l0.d);
-      LAUNCH(hd, K_APPLY32, 0, hd->n * 20.0, k_apply_dot4<false>, zgrid(dq), kBlock,
+      LAUNCH(hd, K_APPLY32, 0, hd->n * 20.0, k_apply_dot4<false>, apply_grid(dq, hd->apply_zper), kBlock,
              (const float *)hd->z32, hd->q32, l0.bx32, l0.by32, l0.bz32, (const float *)l0.dd32,
-             l0.d, zper_of(dq), fin(hd, OP_STORE, S_TMP, 0.0, false), (const float *)nullptr, (float *)nullptr,
-             (const double *)nullptr, 0);
+             l0.d, hd->apply_zper, fin(hd, OP_STORE, S_TMP, 0.0, false), (const float *)nullptr, (float *)nullptr,
+             (const double *)nullptr, 0, (float *)nullptr);
     } else {
       LAUNCH(hd, K_APPLY64, 0, hd->n * 48.0, k_apply_dot<double>, zgrid(l0.d), kBlock, p, hd->q,
              l0.bx, l0.by, l0.bz, l0.diag, (const double *)nullptr, l0.d, zper_of(l0.d),
@@ -1277,7 +1306,7 @@ mp_status solve_assembled(mp_poisson *hd, double *p, double tol, std::vector<dou
       total += 1;
       ++outer;
       LAUNCH(hd, K_ADDF32, 0, hd->n * 24.0, k_add_f32, VEC_BLOCKS, VEC_THREADS, p, hd->e32,
-             hd->n);
+             hd->n, (const float *)nullptr, (const double *)nullptr);
       LAUNCH(hd, K_RESIDMIX, 0, hd->n * 52.0, k_residual_mixed, zgrid(l0.d), kBlock, p, hd->b,
              hd->r32, l0.bx, l0.by, l0.bz, l0.diag, l0.d, zper_of(l0.d), fin(hd, OP_STORE, S_RR, 0.0, true), 0);
       CKS(read_scalars(hd));
@@ -1703,6 +1732,7 @@ mp_status create(mp_poisson *hd, mp_grid g, double h, const mp_bc bc[3]) {
   const size_t nblk = (n + BAND_CELLS - 1) / BAND_CELLS;
   CKS(dalloc(hd, &hd->lab, n));
   CKS(dalloc(hd, &hd->comp, n));
+  CKS(dalloc(hd, &hd->gmask, n / 32 + 1));
   CKS(dalloc(hd, &hd->band, n));
   hd->row_cap = n / 8 + 65536;
   CKS(dalloc(hd, &hd->row_k, hd->row_cap));
@@ -1750,6 +1780,13 @@ mp_status create(mp_poisson *hd, mp_grid g, double h, const mp_bc bc[3]) {
   }
   // fused FP32 sweep: levels above the one-CTA tail with nx a multiple of 8
   CKS(visit_setup(hd));
+  {
+    int dev = 0, sms = 0, occ = 0;
+    CK(cudaGetDevice(&dev));
+    CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_apply_dot4<true>, BX * BY, 0));
+    hd->apply_zper = zper_apply(chunk_dims(hd->L[0].d), std::max(1, sms * occ));
+  }
   CKS(fused_setup(hd));
   CKS(ctail_setup<float>(hd, &hd->ct32));
   CKS(ctail_setup<double>(hd, &hd->ct64));
