@@ -130,6 +130,7 @@ __global__ void __launch_bounds__(CT_THREADS) k_ccl_tile(const double *__restric
                                                          int *__restrict__ lab, Dims d, int *err,
                                                          int limit, int *__restrict__ troots,
                                                          int *ntroots, int cap) {
+  griddep_wait();
   __shared__ int L[CT_CELLS];
   const int tx = blockIdx.x * CT_X, ty = blockIdx.y * CT_Y, tz = blockIdx.z * CT_Z;
   // local index li = x + CT_X (y + CT_Y z); cells outside the grid are liquid
@@ -185,6 +186,7 @@ __global__ void __launch_bounds__(CT_THREADS) k_ccl_tile(const double *__restric
 // neighbour across the face (wrapping on periodic axes only)
 __global__ void __launch_bounds__(CT_THREADS) k_ccl_faces(int *lab, Dims d, int per, int *err,
                                                           int limit) {
+  griddep_wait();
   const int tx = blockIdx.x * CT_X, ty = blockIdx.y * CT_Y, tz = blockIdx.z * CT_Z;
   const int xe = min(CT_X, d.nx - tx), ye = min(CT_Y, d.ny - ty), ze = min(CT_Z, d.nz - tz);
   // the face cells of the tile: x = xe-1 (ye * ze), y = ye-1 (xe * ze), z = ze-1 (xe * ye)
@@ -224,6 +226,7 @@ __global__ void __launch_bounds__(CT_THREADS) k_ccl_faces(int *lab, Dims d, int 
 __global__ void k_ccl_flatten_roots(int *lab, const int *__restrict__ troots,
                                     const int *__restrict__ ntroots, int cap, int *err,
                                     int *roots, int *nroots, int limit) {
+  griddep_wait();
   const int nt = *ntroots;
   if (nt > cap) return;
   for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < nt; q += gridDim.x * blockDim.x) {
@@ -239,6 +242,7 @@ __global__ void k_ccl_flatten_roots(int *lab, const int *__restrict__ troots,
 
 __global__ void k_ccl_flatten(int *lab, size_t n, int *err, int *roots, int *nroots, int limit,
                               const int *__restrict__ ntroots, int cap) {
+  griddep_wait();
   if (*ntroots <= cap) {
     for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < n;
          c += (size_t)gridDim.x * blockDim.x) {
@@ -263,6 +267,7 @@ __global__ void k_ccl_flatten(int *lab, size_t n, int *err, int *roots, int *nro
 // roots' cell order whatever order the roots were appended in).  One block.
 __global__ void k_rank_roots(const int *__restrict__ roots, const int *__restrict__ nroots,
                              int *__restrict__ comp) {
+  griddep_wait();
   __shared__ int sr[DEFL_MAX];
   const int m = *nroots;
   if (m > DEFL_MAX) return;  // deflation is off for this geometry
@@ -280,6 +285,7 @@ __global__ void k_rank_roots(const int *__restrict__ roots, const int *__restric
 // bit per cell, set in gas (a projection reads comp only where it is)
 __global__ void k_comp_from_roots(const int *__restrict__ lab, int *comp, size_t n,
                                   unsigned *__restrict__ mask) {
+  griddep_wait();
   // (whole warps, blocks of a multiple of 32 cells: lane 0's cell starts a mask word)
   for (size_t c0 = blockIdx.x * (size_t)blockDim.x; c0 < n; c0 += (size_t)gridDim.x * blockDim.x) {
     const size_t c = c0 + threadIdx.x;
@@ -322,6 +328,7 @@ __global__ void __launch_bounds__(BAND_THREADS) k_band_count(const int *__restri
 // Each pass stages SCAN_TILE counts in shared memory (coalesced), every thread
 // sums 8 consecutive ones, and a two-level warp-shuffle scan gives the offsets.
 __global__ void __launch_bounds__(SCAN_THREADS) k_scan_counts(int *cnt, int nb, int *total) {
+  griddep_wait();
   __shared__ int tile[SCAN_TILE];
   __shared__ int wsum[32];
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
@@ -372,6 +379,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_counts(int *cnt, int nb, 
 __global__ void __launch_bounds__(BAND_THREADS) k_band_assign(const unsigned char *__restrict__ flag,
                                                               size_t n, const int *__restrict__ off,
                                                               int *__restrict__ band) {
+  griddep_wait();
   __shared__ int wcount[BAND_THREADS / 32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const size_t base = (size_t)blockIdx.x * BAND_CELLS;
@@ -518,6 +526,7 @@ template <typename F>
 __global__ void k_defl_E(const int *__restrict__ band, int nband, const int *__restrict__ comp,
                          const F *__restrict__ bx, const F *__restrict__ by,
                          const F *__restrict__ bz, Dims d, unsigned long long *acc, double scale) {
+  griddep_wait();
   const int stride = gridDim.x * blockDim.x;
   FxCarry carry;
   for (int e0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31); e0 < nband; e0 += stride) {
@@ -572,6 +581,7 @@ __global__ void k_defl_rows(const int *__restrict__ band, int nband, const int *
                             const F *__restrict__ bx, const F *__restrict__ by,
                             const F *__restrict__ bz, Dims d, int *__restrict__ row_k,
                             double *__restrict__ row_w) {
+  griddep_wait();
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < nband; e += gridDim.x * blockDim.x) {
     int ks[7], k = ROW_NONE;
     double ws[7], w = 0.0;
@@ -732,6 +742,7 @@ __global__ void k_defl_resid_band(const int *__restrict__ band, int nband,
                                   const double *__restrict__ diag, Dims d,
                                   const double *__restrict__ coef, const double *__restrict__ p,
                                   const double *__restrict__ b, float *__restrict__ r32) {
+  griddep_wait();
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < nband; e += gridDim.x * blockDim.x) {
     const size_t c = (size_t)band[e];
     int i, j, k;
@@ -814,6 +825,7 @@ __global__ void k_defl_add_z(double *__restrict__ x, const int *__restrict__ com
 // E -> 1/E (fixed-point sums with a fixed scale; the sums are zeroed)
 __global__ void k_defl_einv(int m, unsigned long long *acc, double scale,
                             double *__restrict__ einv) {
+  griddep_wait();
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= m) return;
   const double e = fx_value(acc, j, scale, true);

@@ -82,6 +82,7 @@ __device__ __forceinline__ bool gas(double v) { return __double_as_longlong(v) >
 // and square root are costly on this part, and the band is a thin shell.
 __global__ void k_curvature(const double *__restrict__ phi, double *__restrict__ kap, Dims d,
                             double h, int per) {
+  griddep_wait();
   int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y, k = blockIdx.z;
   if (i >= d.nx || j >= d.ny) return;
   bool px = per & 1, py = per & 2, pz = per & 4;
@@ -147,6 +148,7 @@ __device__ __forceinline__ double gfm_jump(double pa, double pb, double ka, doub
 __global__ void k_faces(const double *__restrict__ phi, double *__restrict__ bx,
                         double *__restrict__ by, double *__restrict__ bz, Dims d, double rl,
                         double rg, double irl, double irg, int per) {
+  griddep_wait();
   int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y, k = blockIdx.z;
   if (i >= d.nx || j >= d.ny) return;
   size_t c = at(d, i, j, k);
@@ -188,6 +190,7 @@ __global__ void k_jump(const double *__restrict__ phi, const double *__restrict_
                        const double *__restrict__ bz, double *__restrict__ Jt, Dims d,
                        double sig, const double *__restrict__ mdot, double rl, double rg,
                        double h) {
+  griddep_wait();
   int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y, k = blockIdx.z;
   if (i >= d.nx || j >= d.ny) return;
   size_t c = at(d, i, j, k);
@@ -256,6 +259,7 @@ __global__ void k_diag(const double *__restrict__ bx, const double *__restrict__
                        __half *__restrict__ by16, __half *__restrict__ bz16, float fs, Dims d,
                        BndPlanes bp, double *__restrict__ dd, float *__restrict__ dd32,
                        __half *__restrict__ dd16) {
+  griddep_wait();
   int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y, k = blockIdx.z;
   if (i >= d.nx || j >= d.ny) return;
   size_t c = at(d, i, j, k);
@@ -295,6 +299,7 @@ __global__ void k_diag(const double *__restrict__ bx, const double *__restrict__
 __global__ void k_coarsen_faces(const double *__restrict__ fx, const double *__restrict__ fy,
                                 const double *__restrict__ fz, Dims df, double *__restrict__ cx,
                                 double *__restrict__ cy, double *__restrict__ cz, Dims dc) {
+  griddep_wait();
   int I = blockIdx.x * BX + threadIdx.x, J = blockIdx.y * BY + threadIdx.y, K = blockIdx.z;
   if (I >= dc.nx || J >= dc.ny) return;
   int i = 2 * I, j = 2 * J, k = 2 * K;
@@ -314,6 +319,7 @@ __global__ void k_coarsen_faces(const double *__restrict__ fx, const double *__r
 __global__ void k_dense_build(const double *__restrict__ bx, const double *__restrict__ by,
                               const double *__restrict__ bz, const double *__restrict__ diag,
                               double *__restrict__ M, Dims d, int singular) {
+  griddep_wait();
   const int n = d.nx * d.ny * d.nz;
   const int c = blockIdx.x * blockDim.x + threadIdx.x, r = blockIdx.y;
   if (c >= n) return;
@@ -1218,6 +1224,7 @@ __global__ void k_residual_mixed(const double *__restrict__ x, const double *__r
                                  const double *__restrict__ by, const double *__restrict__ bz,
                                  const double *__restrict__ diag, Dims d, int zper,
                                  Fin fin, int zero) {
+  griddep_wait();
   int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * BY + threadIdx.y;
   int k0 = blockIdx.z * zper, k1 = min(d.nz, k0 + zper);
   double acc = 0.0;

@@ -735,17 +735,17 @@ mp_status deflation_setup(mp_poisson *hd) {
   const dim3 ct_grid((l0.d.nx + CT_X - 1) / CT_X, (l0.d.ny + CT_Y - 1) / CT_Y,
                      (l0.d.nz + CT_Z - 1) / CT_Z);
   const int lim = hd->opts.label_limit;
-  LAUNCH(hd, K_DEFL_LABEL, 0, n * 12.0, k_ccl_tile, ct_grid, CT_THREADS, hd->phi, hd->lab, l0.d,
+  LAUNCH_PDL(hd, K_DEFL_LABEL, 0, n * 12.0, k_ccl_tile, ct_grid, CT_THREADS, 0, hd->phi, hd->lab, l0.d,
          hd->dint + 2, lim, hd->troots, hd->dint + 3, hd->tcap);
-  LAUNCH(hd, K_DEFL_LABEL, 0, n * 4.0, k_ccl_faces, ct_grid, CT_THREADS, hd->lab, l0.d, hd->per,
+  LAUNCH_PDL(hd, K_DEFL_LABEL, 0, n * 4.0, k_ccl_faces, ct_grid, CT_THREADS, 0, hd->lab, l0.d, hd->per,
          hd->dint + 2, lim);
-  LAUNCH(hd, K_DEFL_LABEL, 0, hd->tcap * 8.0, k_ccl_flatten_roots, VEC_BLOCKS, VEC_THREADS, hd->lab,
+  LAUNCH_PDL(hd, K_DEFL_LABEL, 0, hd->tcap * 8.0, k_ccl_flatten_roots, VEC_BLOCKS, VEC_THREADS, 0, hd->lab,
          (const int *)hd->troots, (const int *)(hd->dint + 3), hd->tcap, hd->dint + 2, hd->roots,
          hd->dint, lim);
-  LAUNCH(hd, K_DEFL_LABEL, 0, n * 8.0, k_ccl_flatten, VEC_BLOCKS, VEC_THREADS, hd->lab, n, hd->dint + 2,
+  LAUNCH_PDL(hd, K_DEFL_LABEL, 0, n * 8.0, k_ccl_flatten, VEC_BLOCKS, VEC_THREADS, 0, hd->lab, n, hd->dint + 2,
          hd->roots, hd->dint, lim, (const int *)(hd->dint + 3), hd->tcap);
-  LAUNCH(hd, K_DEFL_LABEL, 0, DEFL_MAX * 8.0, k_rank_roots, 1, 1024, hd->roots, hd->dint, hd->comp);
-  LAUNCH(hd, K_DEFL_LABEL, 0, n * 12.0, k_comp_from_roots, VEC_BLOCKS, VEC_THREADS, hd->lab, hd->comp,
+  LAUNCH_PDL(hd, K_DEFL_LABEL, 0, DEFL_MAX * 8.0, k_rank_roots, 1, 1024, 0, hd->roots, hd->dint, hd->comp);
+  LAUNCH_PDL(hd, K_DEFL_LABEL, 0, n * 12.0, k_comp_from_roots, VEC_BLOCKS, VEC_THREADS, 0, hd->lab, hd->comp,
          n, hd->gmask);
   CK(cudaMemcpyAsync(hd->hint, hd->dint, 4 * sizeof(int), cudaMemcpyDeviceToHost, hd->st));
   CK(cudaStreamSynchronize(hd->st));
@@ -753,8 +753,8 @@ mp_status deflation_setup(mp_poisson *hd) {
   if (hd->hint[2] != 0 || m <= 0 || m > DEFL_MAX) return MP_OK;
   LAUNCH(hd, K_DEFL_LABEL, 0, n * 5.0, k_band_count, nblk, BAND_THREADS, hd->comp, l0.d, n, hd->cnt,
          hd->bflag);
-  LAUNCH(hd, K_DEFL_LABEL, 0, nblk * 8.0, k_scan_counts, 1, SCAN_THREADS, hd->cnt, nblk, hd->dint + 1);
-  LAUNCH(hd, K_DEFL_LABEL, 0, n * 1.0, k_band_assign, nblk, BAND_THREADS, hd->bflag, n, hd->cnt,
+  LAUNCH_PDL(hd, K_DEFL_LABEL, 0, nblk * 8.0, k_scan_counts, 1, SCAN_THREADS, 0, hd->cnt, nblk, hd->dint + 1);
+  LAUNCH_PDL(hd, K_DEFL_LABEL, 0, n * 1.0, k_band_assign, nblk, BAND_THREADS, 0, hd->bflag, n, hd->cnt,
          hd->band);
   CK(cudaMemcpyAsync(hd->hint, hd->dint, 4 * sizeof(int), cudaMemcpyDeviceToHost, hd->st));
   CK(cudaStreamSynchronize(hd->st));
@@ -763,12 +763,12 @@ mp_status deflation_setup(mp_poisson *hd) {
   // E_jj = -sum of the boundary faces (fixed point: |E| <= 6 beta_max nband)
   const double escale = std::ldexp(1.0, 60) / (6.0 * hd->beta_max * (double)nband + 1.0);
   CK(cudaMemsetAsync(hd->acc_a, 0, defl_acc_bytes(m), hd->st));
-  LAUNCH(hd, K_DEFL, 0, nband * 60.0, k_defl_E<double>, VEC_BLOCKS, VEC_THREADS, hd->band, nband,
+  LAUNCH_PDL(hd, K_DEFL, 0, nband * 60.0, k_defl_E<double>, VEC_BLOCKS, VEC_THREADS, 0, hd->band, nband,
          hd->comp, l0.bx, l0.by, l0.bz, l0.d, hd->acc_a, escale);
-  LAUNCH(hd, K_DEFL, 0, m * 8.0, k_defl_einv, (m + 255) / 256, 256, m, hd->acc_a, escale,
+  LAUNCH_PDL(hd, K_DEFL, 0, m * 8.0, k_defl_einv, (m + 255) / 256, 256, 0, m, hd->acc_a, escale,
          hd->einv);
   if ((size_t)nband <= hd->row_cap)
-    LAUNCH(hd, K_DEFL, 0, nband * 72.0, k_defl_rows<double>, VEC_BLOCKS, VEC_THREADS, hd->band, nband,
+    LAUNCH_PDL(hd, K_DEFL, 0, nband * 72.0, k_defl_rows<double>, VEC_BLOCKS, VEC_THREADS, 0, hd->band, nband,
            hd->comp, l0.bx, l0.by, l0.bz, l0.d, hd->row_k, hd->row_w);
   CKS(launch_ok());
   hd->defl_m = m;
@@ -957,10 +957,10 @@ mp_status defl_true_residual32(mp_poisson *hd, const double *p, int p_is_zero, d
            hd->ztb_scale, hd->einv, hd->coef, hd->coef32, hd->dmax);
   else
     CKS((defl_coef<double, double>(hd, p, l0.bx, l0.by, l0.bz, true)));
-  LAUNCH(hd, K_RESIDMIX, 0, n * (p_is_zero ? 12.0 : 52.0), k_residual_mixed, zgrid(l0.d), kBlock,
+  LAUNCH_PDL(hd, K_RESIDMIX, 0, n * (p_is_zero ? 12.0 : 52.0), k_residual_mixed, zgrid(l0.d), kBlock, 0,
          p, hd->b, hd->r32, l0.bx, l0.by, l0.bz, l0.diag, l0.d, zper_of(l0.d), partials(hd),
          p_is_zero);
-  LAUNCH(hd, K_DEFL, 0, nb * 120.0, k_defl_resid_band, VEC_BLOCKS, VEC_THREADS, hd->band, nb,
+  LAUNCH_PDL(hd, K_DEFL, 0, nb * 120.0, k_defl_resid_band, VEC_BLOCKS, VEC_THREADS, 0, hd->band, nb,
          hd->comp, l0.bx, l0.by, l0.bz, l0.diag, l0.d, hd->coef,
          p_is_zero ? (const double *)nullptr : p, hd->b, hd->r32);
   LAUNCH(hd, K_DOT32, 0, 4.0 * n, k_dot<float>, VEC_BLOCKS, VEC_THREADS, hd->r32, hd->r32, n,
@@ -1015,7 +1015,7 @@ mp_status pcg_mixed(mp_poisson *hd, double *p, double rn, double tol_abs, int ma
       if (defl) {
         CKS(project_true(rn, 0));
       } else {
-        LAUNCH(hd, K_RESIDMIX, 0, n * 52.0, k_residual_mixed, zgrid(l0.d), kBlock, p, hd->b, r,
+        LAUNCH_PDL(hd, K_RESIDMIX, 0, n * 52.0, k_residual_mixed, zgrid(l0.d), kBlock, 0, p, hd->b, r,
                l0.bx, l0.by, l0.bz, l0.diag, l0.d, zper_of(l0.d), fin(hd, OP_STORE, S_RR, 0.0, true), 0);
         CKS(read_scalars(hd));
         rn = std::sqrt(hd->scal_h[S_RR]);
@@ -1236,7 +1236,7 @@ mp_status solve_assembled(mp_poisson *hd, double *p, double tol, std::vector<dou
         LAUNCH(hd, K_RESID64, 0, hd->n * 56.0, k_residual<double>, zgrid(l0.d), kBlock, p, hd->b,
                hd->r, l0.bx, l0.by, l0.bz, l0.diag, l0.d, zper_of(l0.d), fin(hd, OP_STORE, S_RR, 0.0, true), 0);
       else
-        LAUNCH(hd, K_RESIDMIX, 0, hd->n * 52.0, k_residual_mixed, zgrid(l0.d), kBlock, p,
+        LAUNCH_PDL(hd, K_RESIDMIX, 0, hd->n * 52.0, k_residual_mixed, zgrid(l0.d), kBlock, 0, p,
                hd->b, hd->r32, l0.bx, l0.by, l0.bz, l0.diag, l0.d, zper_of(l0.d), fin(hd, OP_STORE, S_RR, 0.0, true), 0);
       CKS(read_scalars(hd));
       rnet = std::sqrt(hd->scal_h[S_RR]);
@@ -1278,8 +1278,8 @@ mp_status solve_assembled(mp_poisson *hd, double *p, double tol, std::vector<dou
   } else {
     // FP64 iterative refinement around an FP32 inner solve
     if (!have_r && !r_projected) {
-      LAUNCH(hd, K_RESIDMIX, 0, hd->n * (zero ? 12.0 : 52.0), k_residual_mixed, zgrid(l0.d),
-             kBlock, p, hd->b, hd->r32, l0.bx, l0.by, l0.bz, l0.diag, l0.d, zper_of(l0.d),
+      LAUNCH_PDL(hd, K_RESIDMIX, 0, hd->n * (zero ? 12.0 : 52.0), k_residual_mixed, zgrid(l0.d),
+             kBlock, 0, p, hd->b, hd->r32, l0.bx, l0.by, l0.bz, l0.diag, l0.d, zper_of(l0.d),
              fin(hd, OP_STORE, S_RR, 0.0, true), zero);
     }
     CKS(read_scalars(hd));
@@ -1307,7 +1307,7 @@ mp_status solve_assembled(mp_poisson *hd, double *p, double tol, std::vector<dou
       ++outer;
       LAUNCH(hd, K_ADDF32, 0, hd->n * 24.0, k_add_f32, VEC_BLOCKS, VEC_THREADS, p, hd->e32,
              hd->n, (const float *)nullptr, (const double *)nullptr);
-      LAUNCH(hd, K_RESIDMIX, 0, hd->n * 52.0, k_residual_mixed, zgrid(l0.d), kBlock, p, hd->b,
+      LAUNCH_PDL(hd, K_RESIDMIX, 0, hd->n * 52.0, k_residual_mixed, zgrid(l0.d), kBlock, 0, p, hd->b,
              hd->r32, l0.bx, l0.by, l0.bz, l0.diag, l0.d, zper_of(l0.d), fin(hd, OP_STORE, S_RR, 0.0, true), 0);
       CKS(read_scalars(hd));
       rn = std::sqrt(hd->scal_h[S_RR]);
@@ -1356,8 +1356,8 @@ mp_status diag_fields(mp_poisson *hd, int mode) {
     auto kd = mode == 1 ? k_diag<1> : (mode == 2 ? k_diag<2> : k_diag<3>);
     BndPlanes bp{};
     for (int q = 0; q < 6; ++q) bp.p[q] = lv.bnd[q];
-    LAUNCH(hd, K_DIAG, (int)l, lv.n * (mode == 1 ? 48.0 : (mode == 2 ? 58.0 : 66.0)), kd,
-           cell_grid(lv.d), kBlock, lv.bx, lv.by, lv.bz, lv.diag, lv.idiag, lv.bx32, lv.by32,
+    LAUNCH_PDL(hd, K_DIAG, (int)l, lv.n * (mode == 1 ? 48.0 : (mode == 2 ? 58.0 : 66.0)), kd,
+           cell_grid(lv.d), kBlock, 0, lv.bx, lv.by, lv.bz, lv.diag, lv.idiag, lv.bx32, lv.by32,
            lv.bz32, lv.idiag32, lv.bx16, lv.by16, lv.bz16, hd->fs16, lv.d, bp, lv.dd, lv.dd32,
            lv.dd16);
     CKS(launch_ok());
@@ -1376,11 +1376,11 @@ mp_status geometry(mp_poisson *hd, const double *phi, double rho_l, double rho_g
   Level &l0 = hd->L[0];
   CK(cudaMemcpyAsync(hd->phi, phi, hd->n * sizeof(double), cudaMemcpyDeviceToDevice, hd->st));
   const double n0 = (double)hd->n;
-  LAUNCH(hd, K_CURV, 0, n0 * 16.0, k_curvature, cell_grid(l0.d), kBlock, hd->phi, hd->kap, l0.d,
+  LAUNCH_PDL(hd, K_CURV, 0, n0 * 16.0, k_curvature, cell_grid(l0.d), kBlock, 0, hd->phi, hd->kap, l0.d,
          hd->h, hd->per);
-  LAUNCH(hd, K_FACES, 0, n0 * 32.0, k_faces, cell_grid(l0.d), kBlock, hd->phi, l0.bx, l0.by,
+  LAUNCH_PDL(hd, K_FACES, 0, n0 * 32.0, k_faces, cell_grid(l0.d), kBlock, 0, hd->phi, l0.bx, l0.by,
          l0.bz, l0.d, rho_l, rho_g, 1.0 / rho_l, 1.0 / rho_g, hd->per);
-  LAUNCH(hd, K_JUMP, 0, n0 * (hd->has_mdot ? 56.0 : 48.0), k_jump, cell_grid(l0.d), kBlock,
+  LAUNCH_PDL(hd, K_JUMP, 0, n0 * (hd->has_mdot ? 56.0 : 48.0), k_jump, cell_grid(l0.d), kBlock, 0,
          hd->phi, hd->kap, l0.bx, l0.by, l0.bz, hd->Jt, l0.d, sigma, mdot_of(hd), rho_l, rho_g,
          hd->h);
   CKS(launch_ok());
@@ -1391,7 +1391,7 @@ mp_status geometry(mp_poisson *hd, const double *phi, double rho_l, double rho_g
     Level &lv = hd->L[l];
     if (l > 0) {
       Level &lf = hd->L[l - 1];
-      LAUNCH(hd, K_COARSEN, (int)l, lv.n * 120.0, k_coarsen_faces, cell_grid(lv.d), kBlock, lf.bx,
+      LAUNCH_PDL(hd, K_COARSEN, (int)l, lv.n * 120.0, k_coarsen_faces, cell_grid(lv.d), kBlock, 0, lf.bx,
              lf.by, lf.bz, lf.d, lv.bx, lv.by, lv.bz, lv.d);
     }
   }
@@ -1419,7 +1419,7 @@ mp_status geometry(mp_poisson *hd, const double *phi, double rho_l, double rho_g
   Level &lc = hd->L.back();
   const int lcl = (int)hd->L.size() - 1;
   const double nc = (double)hd->nc;
-  LAUNCH(hd, K_DENSE, lcl, nc * nc * 8.0, k_dense_build, dim3((hd->nc + 127) / 128, hd->nc), 128,
+  LAUNCH_PDL(hd, K_DENSE, lcl, nc * nc * 8.0, k_dense_build, dim3((hd->nc + 127) / 128, hd->nc), 128, 0,
          lc.bx, lc.by, lc.bz, lc.diag, hd->Maug, lc.d, hd->outflow == 0 ? 1 : 0);
   // the inverse, GJ_B columns per launch, between the two halves of Maug and
   // into Minv at the last step
@@ -1929,7 +1929,7 @@ mp_status mp_poisson_set_mass_flux(mp_handle hd, const double *mdot_dev) {
   hd->has_mdot = mdot_dev != nullptr;
   // the jump source of the current geometry, with or without the flux jump
   Level &l0 = hd->L[0];
-  LAUNCH(hd, K_JUMP, 0, hd->n * (hd->has_mdot ? 56.0 : 48.0), k_jump, cell_grid(l0.d), kBlock,
+  LAUNCH_PDL(hd, K_JUMP, 0, hd->n * (hd->has_mdot ? 56.0 : 48.0), k_jump, cell_grid(l0.d), kBlock, 0,
          hd->phi, hd->kap, l0.bx, l0.by, l0.bz, hd->Jt, l0.d, hd->sigma, mdot_of(hd), hd->rho_l,
          hd->rho_g, hd->h);
   CKS(launch_ok());
