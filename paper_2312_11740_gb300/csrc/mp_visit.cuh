@@ -6,7 +6,9 @@
 // one launch per sweep a 64^3 level took ~8 us a sweep and a 128^3 one ~19,
 // whatever they moved.  A level whose iterate, right-hand side and face
 // coefficients fit the chip's shared memory (FP32 to about 2.1 M cells, FP64 to
-// about 0.6 M) is read once, swept in shared memory and written once.
+// about 0.6 M) is read once, swept in shared memory and written once.  64^3 FP32:
+// 1.37 us a half-sweep and ~5 us a launch; under 256^3 64 us per V-cycle for
+// the level's two visits, transfers included (167 for its sweeps alone before).
 //
 // Blocks: the level is cut in y and z (whole x rows) into py x pz blocks, one
 // CTA each, at most one CTA per SM, launched cooperatively: the CTAs wait on
