@@ -390,6 +390,14 @@ mp_status mp_poisson_rhs_noalloc(long long ncells, const double *rhs_dev, const 
 mp_status mp_poisson_deflated_energy(mp_handle hd, const float *q_dev, const float *t_dev,
                                      float *gq_dev, double *loss_out);
 
+/* Defines: no paper passage (test support for the error path of the bounded
+ * waits).  Test only: the next n V-cycles of this process run with the poll limit
+ * of their waits (level visits and cluster tail) at zero, so the first wait of a
+ * CTA for a neighbour's rows gives up; nothing waits longer than usual.  The
+ * solve that runs such a V-cycle returns MP_ERR_TIMEOUT and its handle stays
+ * usable.  n = 0 cancels. */
+mp_status mp_poisson_test_wait_timeout(int n);
+
 /* Defines: no paper passage (resource release).
  * Free everything the handle owns.  NULL is ignored. */
 void mp_poisson_destroy(mp_handle hd);

@@ -106,6 +106,7 @@ SIGNATURES = {
     "mp_poisson_set_profiling": (_I, [_P, _I]),
     "mp_poisson_get_profile": (_I, [_P, ctypes.POINTER(mp_kernel_prof), _I, _IP]),
     "mp_poisson_rhs_noalloc": (_I, [ctypes.c_longlong, _P, _P, _P, _P]),
+    "mp_poisson_test_wait_timeout": (_I, [_I]),
     "mp_poisson_destroy": (None, [_P]),
     "mp_poisson_set_net": (_I, [_P, _P]),
     "mp_poisson_get_components": (_I, [_P, _P, _IP]),

@@ -17,7 +17,9 @@
 // the slowest CTA and costs ~0.8 us, inside a level.  Slots alternate with the epoch's
 // parity, so a word is overwritten only after its reader has sent its own next
 // message.  Cluster barriers separate levels.  Waits are bounded: a CTA that gives
-// up sets *err and finishes without waiting (its result is not used).
+// up sets *err and finishes without waiting (its result is not used).  It still
+// sends and is sent to, so the last barrier follows the last exchange of the top
+// level in every CTA: none leaves while another may write to its shared memory.
 //
 // Shared-memory arrays are split by colour as in mp_visit.cuh; a level's strides
 // come from its largest block, so a cell's address in its owner's shared memory
@@ -56,6 +58,7 @@ struct CtArgs {
   int singular;   // mean-project the coarsest right-hand side
   int mail;       // byte offset of the exchange slots
   int mail_words;  // 8-byte words of both parities
+  int polls;       // polls of one wait (CT_POLL)
   double *err;
 };
 
@@ -189,7 +192,7 @@ struct CtWalk {
 template <typename T, int C>
 __device__ __forceinline__ void ct_half(const CtView<T> &v, const CtWalk &w, bool zero, unsigned e,
                                         uint32_t mail, const uint32_t rem[4], uint32_t flip,
-                                        bool &dead, double *err) {
+                                        bool &dead, int polls, double *err) {
   constexpr int W = sizeof(T) == 8 ? 16 : 8;  // bytes of a slot
   const int P = v.P, by = v.by, bz = v.bz, sZ = (v.bym + 2) * P;
   const int dlo = w.p == 0 ? P - 1 : -1, dhi = w.p == P - 1 ? 1 - P : 1;
@@ -272,7 +275,7 @@ __device__ __forceinline__ void ct_half(const CtView<T> &v, const CtWalk &w, boo
         }
         T x = 0;
         bool got = false;
-        for (int it = 0; !got && !dead && it < CT_POLL; ++it)
+        for (int it = 0; !got && !dead && it < polls; ++it)
           got = ct_recv(mail + m + slot * W, e, x);
         if (!got) {
           if (!dead) *(volatile double *)err = 1.0;
@@ -418,9 +421,11 @@ k_ctail(const __grid_constant__ CtArgs<T> a, const T *rhs, T *xout) {
   unsigned e = 0;  // epoch of the last exchange, counted alike by every CTA
 
   // the sweeps of one level: colours c0, 1 - c0; the last exchange of an
-  // upward visit is not needed
+  // upward visit is not needed.  leave (the kernel's last sweeps): arrive at the
+  // last cluster barrier once this CTA has sent and received everything, which
+  // leaves the last half-sweep to cover the other CTAs' arrival
   auto sweeps = [&](const CtView<T> &v, const CtBlock &k, auto first, int nu, bool zero,
-                    bool keep_last) {
+                    bool keep_last, bool leave) {
     constexpr int C0 = decltype(first)::value;
     if (v.own) {
       const CtWalk w(v.P, k.mP, v.by, k.m0);
@@ -430,17 +435,21 @@ k_ctail(const __grid_constant__ CtArgs<T> a, const T *rhs, T *xout) {
       rem[2] = ct_map(mail + ((2 * v.bzm + v.bym) * v.P + w.p) * W, k.zm);
       rem[3] = ct_map(mail + (2 * v.bzm * v.P + w.p) * W, k.zp);
       for (int s = 0; s < nu; ++s) {
-        ct_half<T, C0>(v, w, zero && s == 0, e + 2 * s + 1, mail, rem, flip, dead, a.err);
+        ct_half<T, C0>(v, w, zero && s == 0, e + 2 * s + 1, mail, rem, flip, dead, a.polls, a.err);
         const bool x = keep_last || s + 1 < nu;
-        ct_half<T, 1 - C0>(v, w, false, x ? e + 2 * s + 2 : 0u, mail, rem, flip, dead, a.err);
+        if (leave && s + 1 == nu) cl.barrier_arrive();
+        ct_half<T, 1 - C0>(v, w, false, x ? e + 2 * s + 2 : 0u, mail, rem, flip, dead, a.polls,
+                           a.err);
       }
+    } else if (leave) {
+      cl.barrier_arrive();
     }
     e += 2 * nu;
   };
 
   for (int l = 0; l < last; ++l) {  // down
     const CtView<T> v(base, a.lv[l], blk[l]);
-    sweeps(v, blk[l], VsColour<0>{}, a.lv[l].nu1, true, true);
+    sweeps(v, blk[l], VsColour<0>{}, a.lv[l].nu1, true, true, false);
     const CtLevel<T> &gc = a.lv[l + 1];
     const bool coarsest = l + 1 == last;
     if (v.own) {  // residual, restricted to the coarser block's owner
@@ -530,9 +539,7 @@ k_ctail(const __grid_constant__ CtArgs<T> a, const T *rhs, T *xout) {
       }
       __syncthreads();
     }
-    // at the top level: this CTA reads no other's shared memory any more
-    if (l == 0) cl.barrier_arrive();
-    sweeps(v, blk[l], VsColour<1>{}, a.lv[l].nu2, false, false);
+    sweeps(v, blk[l], VsColour<1>{}, a.lv[l].nu2, false, false, l == 0);
     if (l > 0) cl.sync();  // the finer level reads this one's x
   }
   const CtView<T> v(base, a.lv[0], blk[0]);
@@ -549,9 +556,7 @@ k_ctail(const __grid_constant__ CtArgs<T> a, const T *rhs, T *xout) {
       }
     }
   }
-  // No CTA leaves while another may still read its shared memory.  (Boundary rows are
-  // written to it only until the last exchange, which it has received.)
-  cl.barrier_wait();
+  cl.barrier_wait();  // every CTA is past its last access to another's shared memory
 }
 
 }  // namespace mp

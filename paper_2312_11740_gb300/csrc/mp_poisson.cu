@@ -10,6 +10,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -191,6 +192,7 @@ struct mp_poisson {
   unsigned *epoch = nullptr;
   size_t mail_words = 0;
   unsigned long long epochs_used = 0, epochs_cycle = 0;
+  bool no_polls = false;  // the running V-cycle's waits give up at once (a test asked)
   bool capturing = false;
   std::vector<int> cap_ids, cap_levels;
 };
@@ -449,6 +451,7 @@ mp_status ctail_launch(mp_poisson *hd, const T *rhs, T *x) {
   a.singular = hd->outflow == 0;
   a.mail = pl.mail;
   a.mail_words = pl.mail_words;
+  a.polls = hd->no_polls ? 0 : CT_POLL;
   a.err = hd->scal + S_ERR;
   double bytes = 0.0;
   for (int q = 0; q < a.nlev; ++q) {
@@ -511,6 +514,7 @@ mp_status visit_launch(mp_poisson *hd, int l, const T *rhs, T *x) {
   a.py = pl.py, a.pz = pl.pz, a.bym = pl.bym, a.bzm = pl.bzm;
   a.fs = hd->fs16, a.inv_fs = 1.f / hd->fs16;
   a.mail = hd->mail, a.epoch = hd->epoch, a.err = hd->scal + S_ERR;
+  a.polls = hd->no_polls ? 0 : VS_POLL;
   const int id = kid<T>(K_VISIT64, K_RBGS32F);
   // b and the faces once; x written (up: also read), the coarser level's vector
   const double face = sizeof(T) == 8 ? 4.0 * 8.0 : 3.0 * 2.0;
@@ -667,6 +671,16 @@ void destroy_graphs(mp_poisson *hd) {
   hd->graphs.clear();
 }
 
+// V-cycles that are still to run with their waits' poll limit at zero
+// (mp_poisson_test_wait_timeout)
+std::atomic<int> g_wait_timeouts{0};
+bool take_wait_timeout() {
+  int v = g_wait_timeouts.load();
+  while (v > 0 && !g_wait_timeouts.compare_exchange_weak(v, v - 1)) {
+  }
+  return v > 0;
+}
+
 // A whole V-cycle from the finest level.  Without per-launch profiling it is
 // captured once into a CUDA graph (per precision and buffer pair) and
 // replayed: the cycle is a fixed sequence of ~100 launches, most of them on
@@ -674,7 +688,12 @@ void destroy_graphs(mp_poisson *hd) {
 template <typename T>
 mp_status run_vcycle(mp_poisson *hd, const T *rhs, T *x) {
   hd->epochs_used += hd->epochs_cycle;
-  if (hd->prof_on) return vcycle<T>(hd, 0, rhs, x);
+  hd->no_polls = take_wait_timeout();
+  if (hd->prof_on || hd->no_polls) {
+    const mp_status s = vcycle<T>(hd, 0, rhs, x);
+    hd->no_polls = false;
+    return s;
+  }
   mp_poisson::Graph *g = nullptr;
   for (auto &e : hd->graphs)
     if (e.type == (int)sizeof(T) && e.rhs == rhs && e.x == x) g = &e;
@@ -1916,6 +1935,12 @@ mp_status mp_poisson_deflated_energy(mp_handle hd, const float *q_dev, const flo
   }
   CK(cudaStreamSynchronize(hd->st));
   prof_resolve(hd);
+  return MP_OK;
+}
+
+mp_status mp_poisson_test_wait_timeout(int n) {
+  if (n < 0) return MP_ERR_INVALID_ARG;
+  g_wait_timeouts.store(n);
   return MP_OK;
 }
 

@@ -60,6 +60,7 @@ struct VisitArgs {
   float fs, inv_fs;
   unsigned long long *mail;  // exchange slots
   unsigned *epoch;           // [0] base of this launch, [1] CTAs done
+  int polls;                 // polls of one wait (VS_POLL)
   double *err;               // set when a wait gave up
 };
 
@@ -394,7 +395,7 @@ __global__ void __launch_bounds__(VS_THREADS, 1) k_visit(const VisitArgs<T> a) {
             dst[u] = ((hi ? bz + 1 : 0) * (by + 2) + j + 1) * P + q;
           }
         }
-        for (int it = 0; wait && it < VS_POLL; ++it) {
+        for (int it = 0; wait && it < a.polls; ++it) {
 #pragma unroll
           for (int u = 0; u < VS_BATCH; ++u) w[u].load(src[u]);
 #pragma unroll

@@ -970,3 +970,32 @@ def test_deflation_of_gas_threads(n, precision):
         out.append(p)
         s.close()
     assert float(torch.linalg.norm(out[0] - out[1]) / torch.linalg.norm(out[1])) < 1e-7
+
+
+@pytest.mark.parametrize("shape,bc,precision,opts", [
+    ((32, 32, 32), (P, P, N), 1, {}), ((56, 24, 40), (P, P, N), 1, {}),
+    ((24, 20, 16), (N, N, N), 0, {}), ((64, 64, 64), (P, P, N), 0, {}),
+    ((96, 64, 80), (P, P, N), 1, {}), ((48, 64, 96), (D, N, P), 0, {}),
+    ((40, 12, 28), (P, P, P), 0, {"coarse_cluster": 0}),
+    ((64, 64, 64), (P, N, ND), 1, {"smoother": 0, "method": 1, "max_iters": 5})])
+def test_solver_wait_timeout_is_reported_and_the_handle_stays_usable(shape, bc, precision, opts):
+    """The bounded waits of the level visits and of the cluster tail: with the test switch every
+    wait of the next V-cycle gives up at once.  The tail gives up by itself (the first three grids
+    and the last: equal and unequal blocks) or starts behind a visit that has; the solve reports
+    MP_ERR_TIMEOUT, and the next one gives the bits of the one before."""
+    phi, rhs, h = _smoother_case(shape, bc)
+    s = Poisson(phi, h, bc, 1.0, 1e-3, 0.05, precision=precision, **opts)
+    solve = lambda: s.solve(rhs, tol=TOL, allow_not_converged="max_iters" in opts)  # noqa: E731
+    p, it, hist = solve()
+    for _ in range(2):
+        assert _lib.load().mp_poisson_test_wait_timeout(1) == _lib.MP_OK
+        with pytest.raises(MPError) as err:
+            solve()
+        assert err.value.status == _lib.MP_ERR_TIMEOUT
+        q, it2, hist2 = solve()
+        assert torch.equal(p, q) and it == it2 and list(hist) == list(hist2)
+    assert _lib.load().mp_poisson_test_wait_timeout(1) == _lib.MP_OK
+    assert _lib.load().mp_poisson_test_wait_timeout(0) == _lib.MP_OK  # cancelled
+    solve()
+    assert _lib.load().mp_poisson_test_wait_timeout(-1) == _lib.MP_ERR_INVALID_ARG
+    s.close()
