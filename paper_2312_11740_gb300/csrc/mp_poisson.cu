@@ -682,9 +682,10 @@ bool take_wait_timeout() {
 }
 
 // A whole V-cycle from the finest level.  Without per-launch profiling it is
-// captured once into a CUDA graph (per precision and buffer pair) and
-// replayed: the cycle is a fixed sequence of ~100 launches, most of them on
-// small coarse levels where launch latency, not bandwidth, sets the time.
+// captured once into a CUDA graph (per precision and buffer pair; dropped when
+// the options or the scale of the FP16 faces change) and replayed: the cycle is a
+// fixed sequence of launches, many of them on small coarse levels where launch
+// latency, not bandwidth, sets the time.
 template <typename T>
 mp_status run_vcycle(mp_poisson *hd, const T *rhs, T *x) {
   hd->epochs_used += hd->epochs_cycle;
@@ -1405,7 +1406,9 @@ mp_status geometry(mp_poisson *hd, const double *phi, double rho_l, double rho_g
   CKS(launch_ok());
   // faces never exceed 1 / min(rho): scale them so the largest sits in (2^13, 2^14]
   hd->beta_max = std::max(1.0 / rho_l, 1.0 / rho_g);
-  hd->fs16 = (float)std::ldexp(1.0, 14 - (int)std::ceil(std::log2(hd->beta_max)));
+  const float fs = (float)std::ldexp(1.0, 14 - (int)std::ceil(std::log2(hd->beta_max)));
+  if (fs != hd->fs16) destroy_graphs(hd);  // the FP32 cycle's launches hold the scale by value
+  hd->fs16 = fs;
   for (size_t l = 0; l < hd->L.size(); ++l) {
     Level &lv = hd->L[l];
     if (l > 0) {

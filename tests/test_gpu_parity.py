@@ -999,3 +999,29 @@ def test_solver_wait_timeout_is_reported_and_the_handle_stays_usable(shape, bc, 
     solve()
     assert _lib.load().mp_poisson_test_wait_timeout(-1) == _lib.MP_ERR_INVALID_ARG
     s.close()
+
+
+@pytest.mark.parametrize("shape,bc,opts", [
+    ((96, 64, 80), (P, P, N), {}), ((56, 24, 40), (P, P, N), {"coarse_cluster": 0}),
+    ((56, 24, 40), (P, P, N), {"coarse_cluster": 0, "smoother": 0}),
+    ((48, 64, 72), (P, D, N), {"smoother": 0}),
+    ((160, 192, 160), (P, N, N), {})])
+def test_set_geometry_with_another_density_scale(shape, bc, opts):
+    """The FP16 faces of the mixed-precision levels carry a scale that follows the densities.  A
+    handle that has solved at one density ratio and takes a geometry of another (and back) gives
+    the bits of a fresh handle, whatever kernels smooth the levels: visits, fused sweeps, launches
+    per colour."""
+    phi, rhs, h = _smoother_case(shape, bc)
+    new = lambda rg: Poisson(phi, h, bc, 1.0, rg, 0.05, precision=1, **opts)  # noqa: E731
+    ref = {}
+    for rg in (1e-3, 1e-1):
+        s = new(rg)
+        ref[rg] = s.solve(rhs, tol=TOL)
+        s.close()
+    s = new(1e-3)
+    for rg in (1e-3, 1e-1, 1e-3):
+        s.set_geometry(phi, 1.0, rg, 0.05)
+        p, it, hist = s.solve(rhs, tol=TOL)
+        assert it == ref[rg][1] and list(hist) == list(ref[rg][2])
+        assert torch.equal(p, ref[rg][0])
+    s.close()
