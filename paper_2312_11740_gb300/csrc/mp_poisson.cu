@@ -1471,6 +1471,10 @@ template <typename T>
 mp_status visit_plan(VisitPlan *out, const Dims &d, bool dd, int sms, size_t limit) {
   *out = VisitPlan{};
   if (d.nx % 2 || d.ny % 2 || d.nz % 2) return MP_OK;
+  // k_visit gives a thread one pair of every row it walks.  (No level that a handle takes
+  // and a visit would fit is wider: at most MAX_COARSE unknowns on the coarsest level
+  // make a level of nx > 1024 one of more than 10^6 cells.)
+  if (d.nx > 2 * VS_THREADS) return MP_OK;
   const int uy = d.ny / 2, uz = d.nz / 2;
   double best = 0.0;
   for (int py = 1; py <= std::min(uy, sms); ++py)
