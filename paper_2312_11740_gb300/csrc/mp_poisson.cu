@@ -1816,10 +1816,11 @@ mp_status create(mp_poisson *hd, mp_grid g, double h, const mp_bc bc[3]) {
   CKS(fused_setup(hd));
   CKS(ctail_setup<float>(hd, &hd->ct32));
   CKS(ctail_setup<double>(hd, &hd->ct64));
+  // (the limit is the kernel's, not the handle's: every handle sets the same one)
   CK(cudaFuncSetAttribute(k_tail<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                          (int)std::max<size_t>(hd->tail64_bytes, 1)));
+                          (int)TAIL_BUDGET64));
   CK(cudaFuncSetAttribute(k_tail<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                          (int)std::max<size_t>(hd->tail32_bytes, 1)));
+                          (int)TAIL_BUDGET32));
   // the zero fills of dalloc run on the legacy default stream, which a
   // non-blocking caller stream does not wait for: finish them here
   CK(cudaDeviceSynchronize());

@@ -1025,3 +1025,24 @@ def test_set_geometry_with_another_density_scale(shape, bc, opts):
         assert it == ref[rg][1] and list(hist) == list(ref[rg][2])
         assert torch.equal(p, ref[rg][0])
     s.close()
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_a_smaller_handle_leaves_the_coarse_tail_of_a_larger_one_usable(precision):
+    """The one-CTA coarse tail's shared memory differs from handle to handle: a handle made after
+    another, with a smaller tail, does not take the first one's away."""
+    out = []
+    for other in (False, True):
+        phi, rhs, h = _smoother_case((32, 32, 32), (P, P, N))
+        s = Poisson(phi, h, (P, P, N), 1.0, 1e-3, 0.05, precision=precision, coarse_cluster=0)
+        if other:
+            phi8, rhs8, h8 = _smoother_case((8, 8, 8), (P, P, N))
+            t = Poisson(phi8, h8, (P, P, N), 1.0, 1e-3, 0.05, precision=precision,
+                        coarse_cluster=0)
+            t.solve(rhs8, tol=TOL)
+        p, it, _ = s.solve(rhs, tol=TOL)
+        out.append((p, it))
+        if other:
+            t.close()
+        s.close()
+    assert out[0][1] == out[1][1] and torch.equal(out[0][0], out[1][0])
