@@ -1046,3 +1046,39 @@ def test_a_smaller_handle_leaves_the_coarse_tail_of_a_larger_one_usable(precisio
             t.close()
         s.close()
     assert out[0][1] == out[1][1] and torch.equal(out[0][0], out[1][0])
+
+
+@pytest.mark.parametrize("cases", [
+    [((64, 64, 64), 0), ((64, 64, 64), 0)], [((64, 64, 64), 0), ((96, 64, 80), 1)],
+    [((96, 64, 80), 1), ((32, 32, 32), 1), ((48, 64, 96), 0)]])
+def test_solvers_on_several_streams_and_threads_at_once(cases):
+    """Handles on streams and threads of their own, whose level visits each want (nearly) every
+    SM and whose cluster tails a whole cluster: the bits of the same solves one after the other."""
+    import threading
+    jobs = []
+    for shape, precision in cases:
+        phi, rhs, h = _smoother_case(shape, (P, P, N))
+        st = torch.cuda.Stream()
+        torch.cuda.synchronize()
+        s = Poisson(phi, h, (P, P, N), 1.0, 1e-3, 0.05, precision=precision, stream=st)
+        guesses = [torch.zeros_like(rhs) for _ in range(10)]
+        jobs.append((s, rhs, guesses, s.solve(rhs, tol=TOL)))
+    torch.cuda.synchronize()
+    out = [[] for _ in jobs]
+
+    def work(k):
+        torch.cuda.set_device(0)
+        s, rhs, guesses, _ = jobs[k]
+        for p in guesses:
+            out[k].append(s.solve(rhs, p, tol=TOL))
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(len(jobs))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    for k, (s, _, _, (p0, it0, h0)) in enumerate(jobs):
+        assert len(out[k]) == 10
+        for p, it, hist in out[k]:
+            assert it == it0 and list(hist) == list(h0) and torch.equal(p, p0)
+        s.close()
