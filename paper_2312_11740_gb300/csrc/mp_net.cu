@@ -1250,18 +1250,30 @@ mp_status ws_pool(cudaMemPool_t *out) {
 // Status word of a thread's single-layer calls, in mapped host memory: a kernel
 // writes it only when a wait gave up, so a call needs neither a memset nor a copy
 // (each a few us of a call).  The calls wait for their work, so one per thread does.
+// Allocating and freeing it would invalidate a global-mode stream capture of another
+// thread (a thread may end at any time), hence the relaxed capture mode around both.
+struct RelaxedCapture {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
 struct StatusWord {
   int *p = nullptr;
   ~StatusWord() {
-    if (p) cudaFreeHost(p);
+    if (!p) return;
+    RelaxedCapture relaxed;
+    cudaFreeHost(p);
   }
 };
 mp_status status_word(int **out) {
   static thread_local StatusWord w;
-  if (!w.p && cudaHostAlloc((void **)&w.p, 64, cudaHostAllocPortable) != cudaSuccess) {
-    cudaGetLastError();
-    w.p = nullptr;
-    return MP_ERR_OOM;
+  if (!w.p) {
+    RelaxedCapture relaxed;
+    if (cudaHostAlloc((void **)&w.p, 64, cudaHostAllocPortable) != cudaSuccess) {
+      cudaGetLastError();
+      w.p = nullptr;
+      return MP_ERR_OOM;
+    }
   }
   *(volatile int *)w.p = 0;
   *out = w.p;

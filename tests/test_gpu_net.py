@@ -756,3 +756,35 @@ def test_weight_gradient_ragged_grids(shape, ca, cb, up, cout):
     if cb:
         xin = np.concatenate([xin, xb], axis=-1)
     assert rel_max(dw, conv.conv3d_wgrad(xin, gy).reshape(cout, 27, ca + cb)) < 1e-5
+
+
+@pytest.mark.parametrize("mode", ["global", "thread_local"])
+def test_a_thread_that_made_a_layer_call_may_end_during_a_capture(mode):
+    """The end of a thread gives back what its layer calls kept, and leaves the stream capture of
+    another thread intact."""
+    import threading
+    g = torch.Generator(device="cuda").manual_seed(4)
+    x = torch.randn(16, 16, 16, 16, generator=g, device="cuda").bfloat16()
+    w = (0.05 * torch.randn(16, 27, 16, generator=g, device="cuda")).bfloat16()
+    ref = mp_conv3d_fwd(x, w, 16)
+    called, end, out = threading.Event(), threading.Event(), []
+
+    def work():
+        torch.cuda.set_device(0)
+        out.append(mp_conv3d_fwd(x, w, 16))
+        called.set()
+        end.wait(60)
+    t = threading.Thread(target=work)
+    t.start()
+    assert called.wait(60)
+    a = torch.zeros(1024, device="cuda")
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, capture_error_mode=mode):
+        a.add_(1)
+        end.set()
+        t.join()
+        a.add_(1)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert a[0].item() == 2 and torch.equal(out[0], ref)
