@@ -315,7 +315,11 @@ mp_status mp_poisson_get_stats(mp_handle hd, mp_stats *st);
  * this geometry (no gas, or more than 4096 components). */
 mp_status mp_poisson_get_components(mp_handle hd, int *comp_dev, int *m);
 
-/* Per-(kernel, level) launch record, filled by mp_poisson_get_profile. */
+/* Per-(kernel, level) launch record, filled by mp_poisson_get_profile.
+ * "rbgs_f32_fused" stands for the FP32 sweeps that share a launch: one sweep a launch on
+ * levels of at least 4e6 cells, one visit (all its sweeps, with the restriction behind
+ * or the prolongation in front) on levels of at most 6e5; FP64 visits are
+ * "level_visit_f64". */
 typedef struct {
   char name[40];        /* kernel name, e.g. "rbgs_f32" */
   int level;            /* multigrid level (0 = finest) */

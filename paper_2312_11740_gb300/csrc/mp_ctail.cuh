@@ -38,7 +38,7 @@ namespace mp {
 
 namespace cgx = cooperative_groups;
 
-constexpr int CT_MAX_CTAS = 16, CTL_THREADS = 512, CT_MAX_LEVELS = 10, CT_MAX_COARSE = 512;
+constexpr int CT_MAX_CTAS = 16, CTL_THREADS = 512, CT_MAX_LEVELS = 10;
 constexpr int CT_MAX_TAB = 1024;  // rows and planes of all levels
 constexpr int CT_POLL = 1 << 22;  // polls of one wait (tenths of a second)
 

@@ -65,9 +65,6 @@ __device__ __forceinline__ double block_sum(double v) {
 __device__ __forceinline__ int block_linear_id() {
   return blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
 }
-__device__ __forceinline__ bool thread0() {
-  return threadIdx.x == 0 && threadIdx.y == 0 && threadIdx.z == 0;
-}
 
 // phi > 0 (gas) tested on the bit pattern: an integer comparison instead of
 // an FP64 one (FP64 instructions are the scarce resource of the setup kernels)

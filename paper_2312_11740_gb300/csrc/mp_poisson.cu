@@ -68,11 +68,14 @@ struct Level {
 
 enum KernelId {
   K_CURV, K_FACES, K_JUMP, K_DIAG, K_COARSEN, K_DENSE, K_GJ,
-  K_RBGS64, K_RBGS32, K_RBGS32F, K_VISIT64, K_TAIL64, K_TAIL32, K_CTAIL64, K_CTAIL32, K_RESTR64, K_RESTR32, K_PROL64, K_PROL32, K_COARSE64, K_COARSE32,
+  K_RBGS64, K_RBGS32, K_RBGS32F, K_VISIT64, K_TAIL64, K_TAIL32, K_CTAIL64, K_CTAIL32, K_RESTR64,
+  K_RESTR32, K_PROL64, K_PROL32, K_COARSE64, K_COARSE32,
   K_APPLY64, K_APPLY32, K_RESID64, K_RESID32, K_RESIDMIX, K_DOT64, K_DOT32, K_AXPY64, K_AXPY32,
   K_XPBY64, K_XPBY32, K_ADD64, K_ADD32, K_ADDF32, K_SUM, K_SUBMEAN, K_REDUCE, K_ASSEMBLE,
   K_ASSEMBLE_U, K_PROJECT, K_DIV, K_SCALE, K_DEFL, K_DEFL_LABEL, K_DEFL_DOT, K_COUNT
 };
+// rbgs_f32_fused: k_rbgs_fused (levels of at least FUSED_MIN cells, a sweep a launch) and
+// k_visit<float> (levels of at most VISIT_TOP32, a visit a launch)
 const char *const kKernelNames[K_COUNT] = {
   "curvature", "gfm_faces", "jump", "diag", "coarsen_faces", "dense_build", "gauss_jordan",
   "rbgs_f64", "rbgs_f32", "rbgs_f32_fused", "level_visit_f64", "coarse_tail_f64", "coarse_tail_f32",
@@ -356,13 +359,6 @@ void launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cuda
       launch_pdl(kern, (grid), (block), (smem), (hd)->st, __VA_ARGS__);     \
     prof_end((hd), (id), (level), (double)(bytes));                         \
   } while (0)
-// the same with dynamic shared memory
-#define LAUNCH_SMEM(hd, id, level, bytes, kern, grid, block, smem, ...) \
-  do {                                                                  \
-    prof_begin((hd), (id), (level));                                    \
-    kern<<<(grid), (block), (smem), (hd)->st>>>(__VA_ARGS__);           \
-    prof_end((hd), (id), (level), (double)(bytes));                     \
-  } while (0)
 
 template <typename T>
 constexpr int kid(int id64, int id32) {
@@ -379,7 +375,9 @@ Fin fin(const mp_poisson *hd, int op, int slot, double count, bool to_host) {
   return Fin{hd->partial, hd->done, hd->scal, to_host ? hd->scal_h : nullptr, count, op, slot};
 }
 // partial sums only
-Fin partials(const mp_poisson *hd) { return Fin{hd->partial, nullptr, nullptr, nullptr, 0.0, 0, 0}; }
+Fin partials(const mp_poisson *hd) {
+  return Fin{hd->partial, nullptr, nullptr, nullptr, 0.0, 0, 0};
+}
 // the final reduction of partials that several launches left
 mp_status reduce(mp_poisson *hd, int np, int op, int slot, double count) {
   LAUNCH(hd, K_REDUCE, 0, np * 8.0, k_reduce, 1, 1024, hd->partial, np, hd->scal, op, slot, count);
@@ -594,8 +592,8 @@ mp_status vcycle(mp_poisson *hd, int l, const T *rhs, T *x) {
       if constexpr (sizeof(T) == 4) {
         if (lv.d.nx % 4 == 0)  // 16-byte rows (level buffers are 256-byte aligned)
           LAUNCH_PDL(hd, krb, l, bytes, k_rbgs_h4,
-                     dim3((lv.d.nx / 4 + BX - 1) / BX, (lv.d.ny + BY - 1) / BY, lv.d.nz), kBlock,
-                     0, x, rhs, lv.bx16, lv.by16, lv.bz16, (const __half *)lv.dd16, lv.d, colour, zero,
+                     dim3((lv.d.nx / 4 + BX - 1) / BX, (lv.d.ny + BY - 1) / BY, lv.d.nz), kBlock, 0,
+                     x, rhs, lv.bx16, lv.by16, lv.bz16, (const __half *)lv.dd16, lv.d, colour, zero,
                      hd->fs16);
         else
           LAUNCH_PDL(hd, krb, l, bytes, k_rbgs_h, hg, kBlock, 0, x, rhs, lv.bx16, lv.by16,
@@ -755,27 +753,29 @@ mp_status deflation_setup(mp_poisson *hd) {
   const dim3 ct_grid((l0.d.nx + CT_X - 1) / CT_X, (l0.d.ny + CT_Y - 1) / CT_Y,
                      (l0.d.nz + CT_Z - 1) / CT_Z);
   const int lim = hd->opts.label_limit;
-  LAUNCH_PDL(hd, K_DEFL_LABEL, 0, n * 12.0, k_ccl_tile, ct_grid, CT_THREADS, 0, hd->phi, hd->lab, l0.d,
-         hd->dint + 2, lim, hd->troots, hd->dint + 3, hd->tcap);
-  LAUNCH_PDL(hd, K_DEFL_LABEL, 0, n * 4.0, k_ccl_faces, ct_grid, CT_THREADS, 0, hd->lab, l0.d, hd->per,
-         hd->dint + 2, lim);
-  LAUNCH_PDL(hd, K_DEFL_LABEL, 0, hd->tcap * 8.0, k_ccl_flatten_roots, VEC_BLOCKS, VEC_THREADS, 0, hd->lab,
-         (const int *)hd->troots, (const int *)(hd->dint + 3), hd->tcap, hd->dint + 2, hd->roots,
-         hd->dint, lim);
-  LAUNCH_PDL(hd, K_DEFL_LABEL, 0, n * 8.0, k_ccl_flatten, VEC_BLOCKS, VEC_THREADS, 0, hd->lab, n, hd->dint + 2,
-         hd->roots, hd->dint, lim, (const int *)(hd->dint + 3), hd->tcap);
-  LAUNCH_PDL(hd, K_DEFL_LABEL, 0, DEFL_MAX * 8.0, k_rank_roots, 1, 1024, 0, hd->roots, hd->dint, hd->comp);
-  LAUNCH_PDL(hd, K_DEFL_LABEL, 0, n * 12.0, k_comp_from_roots, VEC_BLOCKS, VEC_THREADS, 0, hd->lab, hd->comp,
-         n, hd->gmask);
+  LAUNCH_PDL(hd, K_DEFL_LABEL, 0, n * 12.0, k_ccl_tile, ct_grid, CT_THREADS, 0, hd->phi, hd->lab,
+             l0.d, hd->dint + 2, lim, hd->troots, hd->dint + 3, hd->tcap);
+  LAUNCH_PDL(hd, K_DEFL_LABEL, 0, n * 4.0, k_ccl_faces, ct_grid, CT_THREADS, 0, hd->lab, l0.d,
+             hd->per, hd->dint + 2, lim);
+  LAUNCH_PDL(hd, K_DEFL_LABEL, 0, hd->tcap * 8.0, k_ccl_flatten_roots, VEC_BLOCKS, VEC_THREADS, 0,
+             hd->lab, (const int *)hd->troots, (const int *)(hd->dint + 3), hd->tcap, hd->dint + 2,
+             hd->roots, hd->dint, lim);
+  LAUNCH_PDL(hd, K_DEFL_LABEL, 0, n * 8.0, k_ccl_flatten, VEC_BLOCKS, VEC_THREADS, 0, hd->lab, n,
+             hd->dint + 2, hd->roots, hd->dint, lim, (const int *)(hd->dint + 3), hd->tcap);
+  LAUNCH_PDL(hd, K_DEFL_LABEL, 0, DEFL_MAX * 8.0, k_rank_roots, 1, 1024, 0, hd->roots, hd->dint,
+             hd->comp);
+  LAUNCH_PDL(hd, K_DEFL_LABEL, 0, n * 12.0, k_comp_from_roots, VEC_BLOCKS, VEC_THREADS, 0, hd->lab,
+             hd->comp, n, hd->gmask);
   CK(cudaMemcpyAsync(hd->hint, hd->dint, 4 * sizeof(int), cudaMemcpyDeviceToHost, hd->st));
   CK(cudaStreamSynchronize(hd->st));
   const int m = hd->hint[0];
   if (hd->hint[2] != 0 || m <= 0 || m > DEFL_MAX) return MP_OK;
   LAUNCH(hd, K_DEFL_LABEL, 0, n * 5.0, k_band_count, nblk, BAND_THREADS, hd->comp, l0.d, n, hd->cnt,
          hd->bflag);
-  LAUNCH_PDL(hd, K_DEFL_LABEL, 0, nblk * 8.0, k_scan_counts, 1, SCAN_THREADS, 0, hd->cnt, nblk, hd->dint + 1);
-  LAUNCH_PDL(hd, K_DEFL_LABEL, 0, n * 1.0, k_band_assign, nblk, BAND_THREADS, 0, hd->bflag, n, hd->cnt,
-         hd->band);
+  LAUNCH_PDL(hd, K_DEFL_LABEL, 0, nblk * 8.0, k_scan_counts, 1, SCAN_THREADS, 0, hd->cnt, nblk,
+             hd->dint + 1);
+  LAUNCH_PDL(hd, K_DEFL_LABEL, 0, n * 1.0, k_band_assign, nblk, BAND_THREADS, 0, hd->bflag, n,
+             hd->cnt, hd->band);
   CK(cudaMemcpyAsync(hd->hint, hd->dint, 4 * sizeof(int), cudaMemcpyDeviceToHost, hd->st));
   CK(cudaStreamSynchronize(hd->st));
   const int nband = hd->hint[1];
@@ -783,13 +783,13 @@ mp_status deflation_setup(mp_poisson *hd) {
   // E_jj = -sum of the boundary faces (fixed point: |E| <= 6 beta_max nband)
   const double escale = std::ldexp(1.0, 60) / (6.0 * hd->beta_max * (double)nband + 1.0);
   CK(cudaMemsetAsync(hd->acc_a, 0, defl_acc_bytes(m), hd->st));
-  LAUNCH_PDL(hd, K_DEFL, 0, nband * 60.0, k_defl_E<double>, VEC_BLOCKS, VEC_THREADS, 0, hd->band, nband,
-         hd->comp, l0.bx, l0.by, l0.bz, l0.d, hd->acc_a, escale);
+  LAUNCH_PDL(hd, K_DEFL, 0, nband * 60.0, k_defl_E<double>, VEC_BLOCKS, VEC_THREADS, 0, hd->band,
+             nband, hd->comp, l0.bx, l0.by, l0.bz, l0.d, hd->acc_a, escale);
   LAUNCH_PDL(hd, K_DEFL, 0, m * 8.0, k_defl_einv, (m + 255) / 256, 256, 0, m, hd->acc_a, escale,
          hd->einv);
   if ((size_t)nband <= hd->row_cap)
-    LAUNCH_PDL(hd, K_DEFL, 0, nband * 72.0, k_defl_rows<double>, VEC_BLOCKS, VEC_THREADS, 0, hd->band, nband,
-           hd->comp, l0.bx, l0.by, l0.bz, l0.d, hd->row_k, hd->row_w);
+    LAUNCH_PDL(hd, K_DEFL, 0, nband * 72.0, k_defl_rows<double>, VEC_BLOCKS, VEC_THREADS, 0,
+               hd->band, nband, hd->comp, l0.bx, l0.by, l0.bz, l0.d, hd->row_k, hd->row_w);
   CKS(launch_ok());
   hd->defl_m = m;
   hd->defl_nband = nband;
@@ -810,8 +810,8 @@ mp_status defl_ztb(mp_poisson *hd) {
   CK(cudaMemsetAsync(hd->acc_a, 0, defl_acc_bytes(m), hd->st));
   CK(cudaMemsetAsync(hd->acc_b, 0, defl_acc_bytes(m), hd->st));
   CK(cudaMemsetAsync(hd->dmax, 0, sizeof(unsigned long long), hd->st));
-  LAUNCH(hd, K_DEFL_DOT, 0, hd->n * 12.0, k_defl_zt<double>, VEC_BLOCKS, VEC_THREADS, hd->comp, hd->b,
-         hd->n, hd->acc_ztb, hd->ztb_scale);
+  LAUNCH(hd, K_DEFL_DOT, 0, hd->n * 12.0, k_defl_zt<double>, VEC_BLOCKS, VEC_THREADS, hd->comp,
+         hd->b, hd->n, hd->acc_ztb, hd->ztb_scale);
   return launch_ok();
 }
 
@@ -977,9 +977,9 @@ mp_status defl_true_residual32(mp_poisson *hd, const double *p, int p_is_zero, d
            hd->ztb_scale, hd->einv, hd->coef, hd->coef32, hd->dmax);
   else
     CKS((defl_coef<double, double>(hd, p, l0.bx, l0.by, l0.bz, true)));
-  LAUNCH_PDL(hd, K_RESIDMIX, 0, n * (p_is_zero ? 12.0 : 52.0), k_residual_mixed, zgrid(l0.d), kBlock, 0,
-         p, hd->b, hd->r32, l0.bx, l0.by, l0.bz, l0.diag, l0.d, zper_of(l0.d), partials(hd),
-         p_is_zero);
+  LAUNCH_PDL(hd, K_RESIDMIX, 0, n * (p_is_zero ? 12.0 : 52.0), k_residual_mixed, zgrid(l0.d),
+             kBlock, 0, p, hd->b, hd->r32, l0.bx, l0.by, l0.bz, l0.diag, l0.d, zper_of(l0.d),
+             partials(hd), p_is_zero);
   LAUNCH_PDL(hd, K_DEFL, 0, nb * 120.0, k_defl_resid_band, VEC_BLOCKS, VEC_THREADS, 0, hd->band, nb,
          hd->comp, l0.bx, l0.by, l0.bz, l0.diag, l0.d, hd->coef,
          p_is_zero ? (const double *)nullptr : p, hd->b, hd->r32);
@@ -1029,14 +1029,15 @@ mp_status pcg_mixed(mp_poisson *hd, double *p, double rn, double tol_abs, int ma
     if (since > 0 && (rec <= std::fmax(o.inner_rtol * rn_rep, 0.5 * tol_abs) ||
                       since >= o.inner_max || it >= maxit)) {
       // reliable update: p += e32 (e32 = 0), r32 = bt - At p from FP64
-      LAUNCH(hd, K_ADDF32, 0, n * (pending ? 28.0 : 24.0), k_add_f32, VEC_BLOCKS, VEC_THREADS, p, e, n,
-             pending ? (const float *)dv : nullptr, (const double *)hd->scal);
+      LAUNCH(hd, K_ADDF32, 0, n * (pending ? 28.0 : 24.0), k_add_f32, VEC_BLOCKS, VEC_THREADS, p, e,
+             n, pending ? (const float *)dv : nullptr, (const double *)hd->scal);
       pending = false;
       if (defl) {
         CKS(project_true(rn, 0));
       } else {
-        LAUNCH_PDL(hd, K_RESIDMIX, 0, n * 52.0, k_residual_mixed, zgrid(l0.d), kBlock, 0, p, hd->b, r,
-               l0.bx, l0.by, l0.bz, l0.diag, l0.d, zper_of(l0.d), fin(hd, OP_STORE, S_RR, 0.0, true), 0);
+        LAUNCH_PDL(hd, K_RESIDMIX, 0, n * 52.0, k_residual_mixed, zgrid(l0.d), kBlock, 0, p, hd->b,
+                   r, l0.bx, l0.by, l0.bz, l0.diag, l0.d, zper_of(l0.d),
+                   fin(hd, OP_STORE, S_RR, 0.0, true), 0);
         CKS(read_scalars(hd));
         rn = std::sqrt(hd->scal_h[S_RR]);
       }
@@ -1062,11 +1063,12 @@ mp_status pcg_mixed(mp_poisson *hd, double *p, double rn, double tol_abs, int ma
       // d_new = z + beta d in the operator's loads, stored to the other buffer
       const Dims dq = chunk_dims(l0.d);
       float *dnew = dv == hd->d32 ? hd->d32b : hd->d32;
-      LAUNCH_PDL(hd, K_APPLY32, 0, (it == 0 ? 6.0 : pending ? 9.0 : 7.0) * nsz, k_apply_dot4<true>, apply_grid(dq, hd->apply_zper),
-                 kBlock, 0, (const float *)dv, q, (const float *)l0.bx32,
-                 (const float *)l0.by32, (const float *)l0.bz32, (const float *)l0.dd32, l0.d,
-                 hd->apply_zper, fin(hd, OP_ALPHA, 0, 0.0, false), (const float *)z, dnew, (const double *)hd->scal,
-                 it == 0 ? 1 : 0, pending ? e : (float *)nullptr);
+      LAUNCH_PDL(hd, K_APPLY32, 0, (it == 0 ? 6.0 : pending ? 9.0 : 7.0) * nsz, k_apply_dot4<true>,
+                 apply_grid(dq, hd->apply_zper), kBlock, 0, (const float *)dv, q,
+                 (const float *)l0.bx32, (const float *)l0.by32, (const float *)l0.bz32,
+                 (const float *)l0.dd32, l0.d, hd->apply_zper, fin(hd, OP_ALPHA, 0, 0.0, false),
+                 (const float *)z, dnew, (const double *)hd->scal, it == 0 ? 1 : 0,
+                 pending ? e : (float *)nullptr);
       dv = dnew;
     } else {
       LAUNCH(hd, K_XPBY32, 0, (it == 0 ? 2.0 : 3.0) * nsz, k_xpby<float>, VEC_BLOCKS, VEC_THREADS,
@@ -1126,7 +1128,8 @@ mp_status stationary(mp_poisson *hd, T *x, const T *bt, T *r, T *z, double tol_a
 
 // mean removal of a device FP64 vector (gauge)
 mp_status remove_mean(mp_poisson *hd, double *x) {
-  LAUNCH(hd, K_SUM, 0, hd->n * 8.0, k_sum<double>, VEC_BLOCKS, VEC_THREADS, x, hd->n, fin(hd, OP_MEAN, 0, (double)hd->n, false));
+  LAUNCH(hd, K_SUM, 0, hd->n * 8.0, k_sum<double>, VEC_BLOCKS, VEC_THREADS, x, hd->n,
+         fin(hd, OP_MEAN, 0, (double)hd->n, false));
   LAUNCH(hd, K_SUBMEAN, 0, hd->n * 16.0, k_sub_mean, VEC_BLOCKS, VEC_THREADS, x, hd->n, hd->scal,
          Fin{});
   return launch_ok();
@@ -1227,10 +1230,11 @@ mp_status solve_assembled(mp_poisson *hd, double *p, double tol, std::vector<dou
       LAUNCH(hd, K_RESIDMIX, 0, hd->n * 12.0, k_to_f32_norm, VEC_BLOCKS, VEC_THREADS, p, hd->z32,
              hd->n, partials(hd));
       const Dims dq = chunk_dims(l0.d);
-      LAUNCH(hd, K_APPLY32, 0, hd->n * 20.0, k_apply_dot4<false>, apply_grid(dq, hd->apply_zper), kBlock,
-             (const float *)hd->z32, hd->q32, l0.bx32, l0.by32, l0.bz32, (const float *)l0.dd32,
-             l0.d, hd->apply_zper, fin(hd, OP_STORE, S_TMP, 0.0, false), (const float *)nullptr, (float *)nullptr,
-             (const double *)nullptr, 0, (float *)nullptr);
+      LAUNCH(hd, K_APPLY32, 0, hd->n * 20.0, k_apply_dot4<false>, apply_grid(dq, hd->apply_zper),
+             kBlock, (const float *)hd->z32, hd->q32, l0.bx32, l0.by32, l0.bz32,
+             (const float *)l0.dd32, l0.d, hd->apply_zper, fin(hd, OP_STORE, S_TMP, 0.0, false),
+             (const float *)nullptr, (float *)nullptr, (const double *)nullptr, 0,
+             (float *)nullptr);
     } else {
       LAUNCH(hd, K_APPLY64, 0, hd->n * 48.0, k_apply_dot<double>, zgrid(l0.d), kBlock, p, hd->q,
              l0.bx, l0.by, l0.bz, l0.diag, (const double *)nullptr, l0.d, zper_of(l0.d),
@@ -1254,10 +1258,12 @@ mp_status solve_assembled(mp_poisson *hd, double *p, double tol, std::vector<dou
     } else {
       if (o.precision == 0)
         LAUNCH(hd, K_RESID64, 0, hd->n * 56.0, k_residual<double>, zgrid(l0.d), kBlock, p, hd->b,
-               hd->r, l0.bx, l0.by, l0.bz, l0.diag, l0.d, zper_of(l0.d), fin(hd, OP_STORE, S_RR, 0.0, true), 0);
+               hd->r, l0.bx, l0.by, l0.bz, l0.diag, l0.d, zper_of(l0.d),
+               fin(hd, OP_STORE, S_RR, 0.0, true), 0);
       else
         LAUNCH_PDL(hd, K_RESIDMIX, 0, hd->n * 52.0, k_residual_mixed, zgrid(l0.d), kBlock, 0, p,
-               hd->b, hd->r32, l0.bx, l0.by, l0.bz, l0.diag, l0.d, zper_of(l0.d), fin(hd, OP_STORE, S_RR, 0.0, true), 0);
+                   hd->b, hd->r32, l0.bx, l0.by, l0.bz, l0.diag, l0.d, zper_of(l0.d),
+                   fin(hd, OP_STORE, S_RR, 0.0, true), 0);
       CKS(read_scalars(hd));
       rnet = std::sqrt(hd->scal_h[S_RR]);
       if (defl_active(hd) && o.net_check == 0 && std::isfinite(rnet))
@@ -1327,8 +1333,9 @@ mp_status solve_assembled(mp_poisson *hd, double *p, double tol, std::vector<dou
       ++outer;
       LAUNCH(hd, K_ADDF32, 0, hd->n * 24.0, k_add_f32, VEC_BLOCKS, VEC_THREADS, p, hd->e32,
              hd->n, (const float *)nullptr, (const double *)nullptr);
-      LAUNCH_PDL(hd, K_RESIDMIX, 0, hd->n * 52.0, k_residual_mixed, zgrid(l0.d), kBlock, 0, p, hd->b,
-             hd->r32, l0.bx, l0.by, l0.bz, l0.diag, l0.d, zper_of(l0.d), fin(hd, OP_STORE, S_RR, 0.0, true), 0);
+      LAUNCH_PDL(hd, K_RESIDMIX, 0, hd->n * 52.0, k_residual_mixed, zgrid(l0.d), kBlock, 0, p,
+                 hd->b, hd->r32, l0.bx, l0.by, l0.bz, l0.diag, l0.d, zper_of(l0.d),
+                 fin(hd, OP_STORE, S_RR, 0.0, true), 0);
       CKS(read_scalars(hd));
       rn = std::sqrt(hd->scal_h[S_RR]);
       if (hist) hist->push_back(rn * inv_b);
@@ -1339,8 +1346,9 @@ mp_status solve_assembled(mp_poisson *hd, double *p, double tol, std::vector<dou
   if (st == MP_OK || st == MP_ERR_NOT_CONVERGED) {
     if (!hd->outflow) CKS(remove_mean(hd, p));  // gauge of the singular problem
     // final true FP64 residual of the returned p
-    LAUNCH(hd, K_RESID64, 0, hd->n * 56.0, k_residual<double>, zgrid(l0.d), kBlock, p, hd->b,
-           hd->r, l0.bx, l0.by, l0.bz, l0.diag, l0.d, zper_of(l0.d), fin(hd, OP_STORE, S_RR, 0.0, true), 0);
+    LAUNCH(hd, K_RESID64, 0, hd->n * 56.0, k_residual<double>, zgrid(l0.d), kBlock, p, hd->b, hd->r,
+           l0.bx, l0.by, l0.bz, l0.diag, l0.d, zper_of(l0.d), fin(hd, OP_STORE, S_RR, 0.0, true),
+           0);
     CKS(read_scalars(hd));
     hd->stats.relres = std::sqrt(hd->scal_h[S_RR]) * inv_b;
   }
@@ -1396,8 +1404,8 @@ mp_status geometry(mp_poisson *hd, const double *phi, double rho_l, double rho_g
   Level &l0 = hd->L[0];
   CK(cudaMemcpyAsync(hd->phi, phi, hd->n * sizeof(double), cudaMemcpyDeviceToDevice, hd->st));
   const double n0 = (double)hd->n;
-  LAUNCH_PDL(hd, K_CURV, 0, n0 * 16.0, k_curvature, cell_grid(l0.d), kBlock, 0, hd->phi, hd->kap, l0.d,
-         hd->h, hd->per);
+  LAUNCH_PDL(hd, K_CURV, 0, n0 * 16.0, k_curvature, cell_grid(l0.d), kBlock, 0, hd->phi, hd->kap,
+             l0.d, hd->h, hd->per);
   LAUNCH_PDL(hd, K_FACES, 0, n0 * 32.0, k_faces, cell_grid(l0.d), kBlock, 0, hd->phi, l0.bx, l0.by,
          l0.bz, l0.d, rho_l, rho_g, 1.0 / rho_l, 1.0 / rho_g, hd->per);
   LAUNCH_PDL(hd, K_JUMP, 0, n0 * (hd->has_mdot ? 56.0 : 48.0), k_jump, cell_grid(l0.d), kBlock, 0,
@@ -1413,8 +1421,8 @@ mp_status geometry(mp_poisson *hd, const double *phi, double rho_l, double rho_g
     Level &lv = hd->L[l];
     if (l > 0) {
       Level &lf = hd->L[l - 1];
-      LAUNCH_PDL(hd, K_COARSEN, (int)l, lv.n * 120.0, k_coarsen_faces, cell_grid(lv.d), kBlock, 0, lf.bx,
-             lf.by, lf.bz, lf.d, lv.bx, lv.by, lv.bz, lv.d);
+      LAUNCH_PDL(hd, K_COARSEN, (int)l, lv.n * 120.0, k_coarsen_faces, cell_grid(lv.d), kBlock, 0,
+                 lf.bx, lf.by, lf.bz, lf.d, lv.bx, lv.by, lv.bz, lv.d);
     }
   }
   if (hd->outflow) {  // outflow boundary faces of every level
@@ -1441,8 +1449,8 @@ mp_status geometry(mp_poisson *hd, const double *phi, double rho_l, double rho_g
   Level &lc = hd->L.back();
   const int lcl = (int)hd->L.size() - 1;
   const double nc = (double)hd->nc;
-  LAUNCH_PDL(hd, K_DENSE, lcl, nc * nc * 8.0, k_dense_build, dim3((hd->nc + 127) / 128, hd->nc), 128, 0,
-         lc.bx, lc.by, lc.bz, lc.diag, hd->Maug, lc.d, hd->outflow == 0 ? 1 : 0);
+  LAUNCH_PDL(hd, K_DENSE, lcl, nc * nc * 8.0, k_dense_build, dim3((hd->nc + 127) / 128, hd->nc),
+             128, 0, lc.bx, lc.by, lc.bz, lc.diag, hd->Maug, lc.d, hd->outflow == 0 ? 1 : 0);
   // the inverse, GJ_B columns per launch, between the two halves of Maug and
   // into Minv at the last step
   const int tile = hd->nc <= GJ_SMALL ? 16 : 32;
@@ -1804,7 +1812,6 @@ mp_status create(mp_poisson *hd, mp_grid g, double h, const mp_bc bc[3]) {
       hd->tail32_bytes = bytes;
     }
   }
-  // fused FP32 sweep: levels above the one-CTA tail with nx a multiple of 8
   CKS(visit_setup(hd));
   {
     int dev = 0, sms = 0, occ = 0;
@@ -1962,9 +1969,9 @@ mp_status mp_poisson_set_mass_flux(mp_handle hd, const double *mdot_dev) {
   hd->has_mdot = mdot_dev != nullptr;
   // the jump source of the current geometry, with or without the flux jump
   Level &l0 = hd->L[0];
-  LAUNCH_PDL(hd, K_JUMP, 0, hd->n * (hd->has_mdot ? 56.0 : 48.0), k_jump, cell_grid(l0.d), kBlock, 0,
-         hd->phi, hd->kap, l0.bx, l0.by, l0.bz, hd->Jt, l0.d, hd->sigma, mdot_of(hd), hd->rho_l,
-         hd->rho_g, hd->h);
+  LAUNCH_PDL(hd, K_JUMP, 0, hd->n * (hd->has_mdot ? 56.0 : 48.0), k_jump, cell_grid(l0.d), kBlock,
+             0, hd->phi, hd->kap, l0.bx, l0.by, l0.bz, hd->Jt, l0.d, hd->sigma, mdot_of(hd),
+             hd->rho_l, hd->rho_g, hd->h);
   CKS(launch_ok());
   CK(cudaStreamSynchronize(hd->st));
   prof_resolve(hd);

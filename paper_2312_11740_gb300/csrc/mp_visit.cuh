@@ -5,8 +5,9 @@
 // What bounds the levels between the finest and the coarse tail is latency: as
 // one launch per sweep a 64^3 level took ~8 us a sweep and a 128^3 one ~19,
 // whatever they moved.  A level whose iterate, right-hand side and face
-// coefficients fit the chip's shared memory (FP32 to about 2.1 M cells, FP64 to
-// about 0.6 M) is read once, swept in shared memory and written once.  64^3 FP32:
+// coefficients fit the chip's shared memory (FP32 to about 2.1 M cells, of which the
+// dispatch takes those up to VISIT_TOP32; FP64 to about 0.6 M, all taken) is
+// read once, swept in shared memory and written once.  64^3 FP32:
 // 1.37 us a half-sweep and ~5 us a launch; under 256^3 64 us per V-cycle for
 // the level's two visits, transfers included (167 for its sweeps alone before).
 //
