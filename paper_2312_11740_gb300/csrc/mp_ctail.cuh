@@ -19,7 +19,9 @@
 // message.  Cluster barriers separate levels.  Waits are bounded: a CTA that gives
 // up sets *err and finishes without waiting (its result is not used).  It still
 // sends and is sent to, so the last barrier follows the last exchange of the top
-// level in every CTA: none leaves while another may write to its shared memory.
+// level in every CTA: none leaves while another may write to its shared memory (about 1 us
+// a launch: a 32^3 projection step of 11 iterations takes 1629 us, 1617 with the
+// barrier arrived at before the top level's last sweeps, which did not hold this).
 //
 // Shared-memory arrays are split by colour as in mp_visit.cuh; a level's strides
 // come from its largest block, so a cell's address in its owner's shared memory
